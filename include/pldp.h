@@ -232,14 +232,11 @@ PLDP_API pldp_status pldp_extract_draft(const int32_t* ids, int64_t ids_stride,
  * bits and a tie within rounding may be broken differently).  Eq. 1-3
  * (Sec. 4.2) and Sec. 4.3.
  *
- * One launch over a flat (chunk, sequence) grid.  Each CTA streams its chunk of
- * the context, scores every occurrence of x_t it finds (cosine and attention
- * score, with all its threads) and records it with its suffix-match length in a
- * small per-sequence list held in the workspace; the CTA that finishes a
- * sequence last (an atomic ticket, no waiting) orders the list into the
- * candidate list, picks the best of each ranking and writes the draft.  More
- * than 256 occurrences in a sequence fall back to an ordered rescan of its
- * context by that CTA.
+ * One launch of a thread-block cluster per sequence.  Each CTA scans its chunk of
+ * the context once and keeps the positions with the longest suffix match it met;
+ * the cluster then knows the candidate list and deals the candidates out to its
+ * CTAs, which score them (cosine and attention score), and its first CTA picks the
+ * best of each ranking and writes the draft.
  *
  * Fields of the argument block (device pointers unless stated):
  *  ids .. match_len      as pldp_find_candidates (T_cap <= 2^27).
@@ -256,7 +253,7 @@ PLDP_API pldp_status pldp_extract_draft(const int32_t* ids, int64_t ids_stride,
  *  status                uint32 [B] or NULL.
  *  workspace             device scratch of pldp_draft_workspace_size(B) bytes,
  *                        16-byte aligned, ZEROED by the caller before its first
- *                        use; every call leaves it zeroed again.  Calls that may
+ *                        use; every call leaves it zeroed.  Calls that may
  *                        run concurrently need separate workspaces.  May be NULL
  *                        when an index is given.
  *  index, index_bytes, V optional incremental token index (NULL: scan the

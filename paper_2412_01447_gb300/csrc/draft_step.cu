@@ -10,29 +10,27 @@
 //    row keys, or on the draws of sampling) and then the indexed drafting in the
 //    same CTA.
 //
-// The scanning kernel: a flat grid of (chunk, sequence) CTAs.  Each CTA
-//  1. streams its chunk of the context with 16-byte loads and, for every
-//     occurrence j of x_t, takes the suffix-match length m and a slot in a short
-//     per-sequence list held in the workspace;
-//  2. scores each occurrence it found with all its threads -- cos(H_{j-1},
-//     H_{t-1}) and the max (or sum) of the selected attention rows at key j, both
-//     in one round trip to memory -- and stores (j, m, scores) in the slot;
-//  3. takes a ticket.  The CTA that takes a sequence's last ticket finishes it:
-//     it reads the list, takes n* = the largest m, orders the occurrences with
-//     m >= n* by position (the candidate list), picks the best of each ranking
-//     from the stored scores, writes the draft, and returns the list's header to
-//     zero for the next call.
-// No CTA waits for another.  Occurrences are scored before n* is known, so
-// those with m < n* are scored for nothing; they are few.  A list that
-// overflowed (more than kHitCap occurrences) is redone by the finishing CTA: an
-// ordered rescan of the context, then the same scorer per candidate.
+// The scanning kernel: one thread-block cluster per sequence, a chunk of the context
+// per CTA.  Each CTA
+//  1. scans its chunk once and keeps the positions with the longest suffix match it
+//     met (pldp_scan.cuh), starts their hidden rows towards L2, and tells the
+//     cluster's other CTAs its longest match and how many positions have it;
+//  2. after the cluster barrier knows n*, the candidate list and its order; the
+//     candidates are dealt out evenly to the cluster's CTAs, which read each other's
+//     lists over distributed shared memory and score them -- cos(H_{j-1}, H_{t-1})
+//     and the max (or sum) of the selected attention rows at key j, both in one round
+//     trip to memory;
+//  3. sends its best keys to CTA 0, which writes the choices and the draft.
+// Only candidates are scored, by all CTAs of the sequence, whatever the number of
+// occurrences of x_t.
 //
-// Every score comes from the same CTA-wide reduction (a fixed share per thread,
-// partial sums combined in warp order), whichever CTA computes it, so results
-// are deterministic.  Results are those of pldp_find_candidates,
-// pldp_rank_hidden, pldp_rank_attention and pldp_extract_draft called in turn
-// (fp32 score sums are split differently, so scores can differ in their last
-// bits).
+// Every score is the sum of the same partial sums in the same order (a fixed share per
+// thread of a CTA, combined in warp order), whether a CTA scores one candidate with
+// all its warps (cta_score) or each warp takes its own (warp_score), so results are
+// deterministic and do not depend on the path.  Results are those of
+// pldp_find_candidates, pldp_rank_hidden, pldp_rank_attention and pldp_extract_draft
+// called in turn (fp32 score sums are split differently, so scores can differ in
+// their last bits).
 #include <climits>
 #include <type_traits>
 
@@ -45,20 +43,23 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kScanVec = 9;                                    // int4 loads per scan thread
-constexpr int64_t kChunk = int64_t(kThreads) * kScanVec * 4;   // positions per CTA
-constexpr int kHitCap = 256;                                   // occurrences kept per sequence
-constexpr size_t kSeqWs = 16 + kHitCap * 16;                   // header + 16-byte entries
+constexpr size_t kSeqWs = 16 + 256 * 16;                       // workspace per sequence (see pldp_draft_workspace_size)
+constexpr int64_t kPositionsPerCta = 1024;                     // scanned by a CTA at least; the batch sets the rest
+constexpr int kScanLoads = 8;                                  // vectors of ids in flight per lane (scan kernel)
+constexpr int kListPerWarp = 128;                              // positions listed per warp (scan kernel)
+constexpr int kList = kListPerWarp * kWarps;                   // ... and per CTA
+constexpr int kRescanLoads = 16;                               // the same for the rescan of the indexed kernels
+constexpr int kRescanPerWarp = 128;
 constexpr int kScoreUnroll = 2;                                // 16-byte row loads in flight
-constexpr int kScoreBatch = 2;                                 // occurrences scored per pass (scan kernel)
+constexpr int kScoreBatch = 2;                                 // candidates scored by the whole CTA at once (scan kernel)
 constexpr int kMaxScoreBatch = 4;                              // ... and at most (the indexed kernel)
+constexpr int kCtaPasses = 4;                                  // passes of the whole CTA before a warp takes each candidate
+constexpr int kWarpLookahead = 2;                              // candidates per warp whose hidden rows are prefetched
 constexpr int kSpeculate = kMaxScoreBatch;                     // occurrences scored before their suffix match
 constexpr int kPrefetchOcc = 32;                                // occurrences whose rows are prefetched otherwise
 constexpr size_t kMaxQueryBytes = 196608;
 constexpr int kMaxSelRows = 8192;
 constexpr int64_t kMaxPositions = int64_t(1) << 27;            // (j << 4) | m fits 31 bits
-
-static_assert(kHitCap <= kThreads, "the finish gives each list entry its own thread");
 
 struct NoHidden {};
 
@@ -97,20 +98,6 @@ struct DraftParams {
     int32_t* draft;
     int32_t* draft_len;
     uint32_t* status;
-    unsigned char* ws;    // kSeqWs per sequence: count, ticket (u32 each), pad; entries
-};
-
-// Workspace of sequence b: header[0] = occurrences recorded, header[1] = tickets
-// taken; entry i = ((j << 4) | m, hidden score bits, attention score bits, 0).
-__device__ __forceinline__ unsigned* seq_header(unsigned char* ws, int b) {
-    return reinterpret_cast<unsigned*>(ws + static_cast<size_t>(b) * kSeqWs);
-}
-__device__ __forceinline__ uint4* seq_entries(unsigned char* ws, int b) {
-    return reinterpret_cast<uint4*>(ws + static_cast<size_t>(b) * kSeqWs + 16);
-}
-
-struct Hit {
-    int32_t j, m;
 };
 
 // Warp reduce-scatter of N values (N a power of two, <= 32): at each butterfly
@@ -151,14 +138,9 @@ __device__ __forceinline__ float (&part_buf(float (&part)[kMaxScoreBatch][kWarps
 }
 
 struct StepShared {
-    Hit hit[kHitCap];                        // occurrences this CTA found (the first kHitCap)
     alignas(16) float part[2][kMaxScoreBatch][kWarps][4];   // per-warp partials: dot, |a|^2, |q|^2, attention
-    int32_t jl[kHitCap];                     // finish: positions of the candidates (else INT_MAX)
-    unsigned long long wkey[2][kWarps];      // finish: per-warp best keys (hidden, attention)
-    int wmax[kWarps];
-    int32_t suf[PLDP_MAX_NGRAM];             // x_t, x_{t-1}, ... (n_max of them)
-    int nhit, skip, last;
-    ScanShared ss;                           // finish: the ordered rescan of an overflowed list
+    unsigned long long wkey[2][kWarps];      // per-warp best keys (hidden, attention)
+    float wnq[kWarps];                       // per-warp partials of |H_{t-1}|^2
 };
 
 // Eq. 3 and Eq. 2 for candidates j[0 .. nb) of sequence b (nb <= NB), by all
@@ -308,290 +290,369 @@ __device__ __forceinline__ void cta_score(const DraftParams& p, int b, const int
     }
 }
 
-// The finish of a sequence whose occurrences were not gathered (an overflowed
-// list, or a token the index cannot answer for): an ordered rescan of the
-// context writes the candidate list, the candidates' hidden rows start towards
-// L2, then the candidates are scored by cta_score, NB per pass.  Kept out of
-// line: its registers do not weigh on the common path.  CTA-uniform call; keys
-// are left in thread 0.
-template <typename TH, bool IVEC, int NB, typename RD = ReadOnlyIds>
-__device__ __noinline__ void finish_overflow(const DraftParams& p, int b, int64_t t, const int32_t* row,
-                                             int32_t* cand_row, float* hsc, float* asc, StepShared& sh,
-                                             unsigned long long& hk, unsigned long long& ak, int& nstar,
-                                             int& total) {
-    constexpr bool HAS_H = !std::is_same<TH, NoHidden>::value;
-    const bool has_a = p.A != nullptr;
-    const int tid = threadIdx.x;
-    int c[PLDP_MAX_NGRAM];
-#pragma unroll
-    for (int k = 0; k < PLDP_MAX_NGRAM; ++k) c[k] = 0;
-    scan_count<IVEC, GlobalIdsT<RD>, RD>(GlobalIdsT<RD>{row}, row, 0, t, t, p.ngram_max, c);
-    scan_reduce_counts(c, p.ngram_max, sh.ss);
-    __syncthreads();
-    if (tid == 0) {
-        int ns = 0, tot = 0;
-        for (int n = p.ngram_max; n >= p.ngram_min; --n)
-            if (sh.ss.cnt[n] > 0) {
-                ns = n;
-                tot = sh.ss.cnt[n];
-                break;
+// |H_{t-1}|^2 in every thread, summed as cta_score sums it.  CTA-uniform call with one
+// barrier.
+template <typename TH>
+__device__ __forceinline__ float cta_query_norm(const DraftParams& p, int b, int64_t t, float (&wnq)[kWarps]) {
+    if constexpr (std::is_same<TH, NoHidden>::value) {
+        return 0.f;
+    } else {
+        constexpr int E = 16 / sizeof(TH);
+        const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+        const TH* qrow = static_cast<const TH*>(p.H) + static_cast<int64_t>(b) * p.h_seq_stride + (t - 1) * p.d;
+        const int64_t nch = p.d / E;
+        float nq = 0.f;
+        if (t >= 2)
+            for (int64_t c = tid; c < nch; c += kThreads) {
+                const uint4 q = __ldg(reinterpret_cast<const uint4*>(qrow) + c);
+                float dead0 = 0.f, dead1 = 0.f;
+                accum16<TH>(q, q, dead0, dead1, nq);
             }
-        sh.ss.nstar = ns;
-        sh.ss.total = tot;
-        sh.ss.offset = 0;
-        sh.ss.mine = tot;
-    }
-    __syncthreads();
-    nstar = sh.ss.nstar;
-    total = sh.ss.total;
-    scan_write<IVEC, GlobalIdsT<RD>, NoHook, RD>(GlobalIdsT<RD>{row}, row, 0, t, t, p.ngram_max, sh.ss, cand_row,
-                                                 p.C_cap);
-    __syncthreads();
-    const int n = total < p.C_cap ? total : p.C_cap;
-    if (HAS_H && n > NB) {
-        const size_t h_es = p.h_bf16 ? 2 : 4;
-        for (int i = tid; i < n; i += kThreads) {
-            const int64_t j = __ldcg(cand_row + i);
-            if (j >= 1 && j < t)
-                prefetch_l2_bulk(static_cast<const char*>(p.H) + (static_cast<int64_t>(b) * p.h_seq_stride + (j - 1) * p.d) * h_es,
-                                 static_cast<uint32_t>(p.d * h_es));
-        }
-    }
-    for (int i0 = 0; i0 < n; i0 += NB) {
-        const int nb = n - i0 < NB ? n - i0 : NB;
-        int64_t j[NB];
-#pragma unroll
-        for (int h = 0; h < NB; ++h) j[h] = h < nb ? __ldcg(cand_row + i0 + h) : -1;
-        float s_h[NB], s_a[NB];
-        cta_score<TH, NB>(p, b, j, nb, t, part_buf<NB>(sh.part[(i0 / NB) & 1]), s_h, s_a);
-        if (tid == 0)
-            for (int h = 0; h < nb; ++h) {
-                const int i = i0 + h;
-                if (HAS_H) {
-                    if (hsc) hsc[i] = s_h[h];
-                    if (j[h] >= 1 && s_h[h] > p.threshold) {
-                        const unsigned long long key = pack_key(s_h[h], static_cast<uint32_t>(j[h]));
-                        hk = key > hk ? key : hk;
-                    }
-                }
-                if (has_a) {
-                    if (asc) asc[i] = s_a[h];
-                    const unsigned long long key = pack_key(s_a[h], static_cast<uint32_t>(j[h]));
-                    ak = key > ak ? key : ak;
-                }
-            }
+        nq = warp_sum(nq);
+        if (lane == 0) wnq[warp] = nq;
+        __syncthreads();
+        return ((wnq[0] + wnq[4]) + (wnq[2] + wnq[6])) + ((wnq[1] + wnq[5]) + (wnq[3] + wnq[7]));
     }
 }
 
-template <typename TH, bool IVEC>
-__global__ void __launch_bounds__(kThreads, 4) draft_step_kernel(const DraftParams p) {
+// Eq. 3 and Eq. 2 for one candidate j by one warp, the results (in every lane) those of
+// cta_score bit for bit: lane l forms the partial sums of the CTA's threads l, 32 + l,
+// ..., 224 + l in eight accumulators, each in that thread's order, and they are reduced
+// over the lanes and then over the eight in the CTA's order.  nq = |H_{t-1}|^2
+// (cta_query_norm); the query row is read through L1, which the warps share.
+template <typename TH>
+__device__ __forceinline__ void warp_score(const DraftParams& p, int b, int64_t j, int64_t t, float nq, float& s_h,
+                                           float& s_a) {
     constexpr bool HAS_H = !std::is_same<TH, NoHidden>::value;
-    __shared__ StepShared sh;
-    pdl_enter();
-    const int b = blockIdx.y;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t L = p.seq_len[b];
-    const bool valid = L >= 0 && L <= p.T_cap;
-    const int64_t t = L - 1;
-    const int32_t* row = p.ids + static_cast<int64_t>(b) * p.ids_stride;
-    unsigned* hdr = seq_header(p.ws, b);
-    const size_t h_es = p.h_bf16 ? 2 : 4;
-    // The chunk's ids do not depend on seq_len: their loads go out first, bounded
-    // by the row's capacity, and land while seq_len and the suffix arrive.
-    const int64_t c0 = static_cast<int64_t>(blockIdx.x) * kChunk;
-    const int64_t ce = c0 + kChunk < p.T_cap ? c0 + kChunk : p.T_cap;
-    constexpr int NV = IVEC ? kScanVec : kScanVec * 4;
-    using VT = typename std::conditional<IVEC, int4, int32_t>::type;
-    VT v[NV];
+    static_assert(kWarps == 8, "eight partial sums per lane");
+    const int lane = threadIdx.x & 31;
+    const bool is_max = p.agg == PLDP_AGG_MAX;
+    const bool h_ok = HAS_H && j >= 1 && j < t, a_ok = p.A != nullptr && j >= 0 && j < t;
+    s_h = -INFINITY;
+    s_a = -INFINITY;
+    // the attention values of the first 128 selected rows are requested before the
+    // hidden row is used, so both arrive in one round trip
+    const size_t a_es = p.a_bf16 ? 2 : 4;
+    const char* ab = p.A ? static_cast<const char*>(p.A) +
+                               (static_cast<int64_t>(b) * p.a_seq_stride + j * p.a_key_stride) * static_cast<int64_t>(a_es)
+                         : nullptr;
+    auto attn = [&](int k) -> float {                             // NaN: no such row
+        if (!a_ok || k >= p.n_sel) return NAN;
+        const int r = p.row_idx ? __ldg(p.row_idx + k) : k;
+        return (r >= 0 && r < p.R) ? load_attn(ab, static_cast<int64_t>(r) * p.a_row_stride, p.a_bf16) : NAN;
+    };
+    constexpr int kEarly = 4;
+    float av[kEarly];
 #pragma unroll
-    for (int u = 0; u < NV; ++u) {
-        if constexpr (IVEC) {
-            const int64_t q = (c0 >> 2) + tid + u * kThreads;
-            if (q < (ce >> 2)) v[u] = __ldg(reinterpret_cast<const int4*>(row) + q);
-        } else {
-            const int64_t j = c0 + tid + u * kThreads;
-            if (j < ce) v[u] = __ldg(row + j);
+    for (int w = 0; w < kEarly; ++w) av[w] = attn(32 * w + lane);
+    if constexpr (HAS_H) {
+        if (h_ok) {                                               // warp-uniform
+            constexpr int E = 16 / sizeof(TH);
+            const TH* hb = static_cast<const TH*>(p.H) + static_cast<int64_t>(b) * p.h_seq_stride;
+            const uint4* qrow = reinterpret_cast<const uint4*>(hb + (t - 1) * p.d);
+            const TH* arow = hb + (j - 1) * p.d;
+            const int64_t nch = p.d / E;
+            float v[16];                                          // dot of share w, then |H_{j-1}|^2 of share w
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = 0.f;
+            for (int64_t c0 = lane; c0 < nch; c0 += kThreads) {
+                uint4 a[kWarps];
+#pragma unroll
+                for (int w = 0; w < kWarps; ++w)
+                    if (c0 + 32 * w < nch) a[w] = ld_stream16(arow + (c0 + 32 * w) * E);
+#pragma unroll
+                for (int w = 0; w < kWarps; ++w) {
+                    if (c0 + 32 * w >= nch) continue;
+                    const uint4 q = __ldg(qrow + c0 + 32 * w);
+                    float dead = 0.f;
+                    accum16<TH>(a[w], q, v[w], v[8 + w], dead);
+                }
+            }
+            float r = warp_reduce_scatter<16>(v, false);          // lane l: value l / 2
+            r += __shfl_xor_sync(0xFFFFFFFFu, r, 8);
+            r += __shfl_xor_sync(0xFFFFFFFFu, r, 4);
+            r += __shfl_xor_sync(0xFFFFFFFFu, r, 2);
+            s_h = finish_cosine(__shfl_sync(0xFFFFFFFFu, r, 0), __shfl_sync(0xFFFFFFFFu, r, 16), nq);
         }
     }
-    if (tid < PLDP_MAX_NGRAM)                                     // x_t and the n_max - 1 tokens before it
-        sh.suf[tid] = (valid && tid < p.ngram_max && t - tid >= 0) ? __ldg(row + t - tid) : 0;
-    if (tid == 0) {
-        sh.nhit = 0;
-        if (HAS_H && valid && t >= 2 && blockIdx.x == 0)        // H_{t-1}: every scored candidate reads it
-            prefetch_l2_bulk(static_cast<const char*>(p.H) + (static_cast<int64_t>(b) * p.h_seq_stride + (t - 1) * p.d) * h_es,
+    if (a_ok) {                                                   // warp-uniform
+        float acc[kWarps];
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            acc[w] = is_max ? -INFINITY : 0.0f;
+            const float x = w < kEarly ? av[w] : attn(32 * w + lane);
+            if (x == x) acc[w] = is_max ? fmaxf(acc[w], x) : acc[w] + x;
+        }
+        for (int k0 = kThreads; k0 < p.n_sel; k0 += kThreads) {
+            float x[kWarps];
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) x[w] = attn(k0 + 32 * w + lane);
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w)
+                if (x[w] == x[w]) acc[w] = is_max ? fmaxf(acc[w], x[w]) : acc[w] + x[w];
+        }
+        float r = warp_reduce_scatter<8>(acc, is_max);            // lane l: value l / 4
+#pragma unroll
+        for (int o = 16; o >= 4; o >>= 1) {
+            const float x = __shfl_xor_sync(0xFFFFFFFFu, r, o);
+            r = is_max ? fmaxf(r, x) : r + x;
+        }
+        s_a = r;
+    }
+}
+
+// The best keys a thread has scored.
+struct BestKeys {
+    unsigned long long h, a;
+};
+
+// Takes in the scores of the candidate with list index i at position j.
+template <typename TH>
+__device__ __forceinline__ void take_score(const DraftParams& p, int i, int64_t j, float s_h, float s_a, float* hsc,
+                                           float* asc, BestKeys& best) {
+    if (!std::is_same<TH, NoHidden>::value) {
+        if (hsc) hsc[i] = s_h;
+        if (j >= 1 && s_h > p.threshold) {
+            const unsigned long long key = pack_key(s_h, static_cast<uint32_t>(j));
+            best.h = key > best.h ? key : best.h;
+        }
+    }
+    if (p.A != nullptr) {
+        if (asc) asc[i] = s_a;
+        const unsigned long long key = pack_key(s_a, static_cast<uint32_t>(j));
+        best.a = key > best.a ? key : best.a;
+    }
+}
+
+// This CTA's share of the candidates, a warp each: list indexes rank + S * k for
+// k < n_local, at positions near[k] (shared) for k < n_near and far[rank + S * k]
+// (global) from there.  Eight rows are on their way at once and no barrier separates
+// them; the rows of a warp's next candidates head for L2 meanwhile.  Scores go to hsc /
+// asc (if given); the best keys are returned in lane 0 of each warp.  CTA-uniform call,
+// out of line: inlined, it cost the calls with few candidates 2-5 us after an L2 flush.
+template <typename TH>
+__device__ __noinline__ BestKeys score_by_warps(const DraftParams& p, int b, int64_t t, int n_local, int rank, int S,
+                                                const int32_t* near, int n_near, const int32_t* far, float* hsc,
+                                                float* asc, float (&wnq)[kWarps]) {
+    constexpr bool HAS_H = !std::is_same<TH, NoHidden>::value;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t h_es = p.h_bf16 ? 2 : 4;
+    BestKeys best = {0, 0};
+    auto cand = [&](int k) -> int64_t { return k < n_near ? near[k] : __ldcg(far + rank + S * k); };
+    auto prefetch = [&](int k) {
+        if (!HAS_H || lane != 0 || k >= n_local) return;
+        const int64_t j = cand(k);
+        if (j >= 1 && j < t)
+            prefetch_l2_bulk(static_cast<const char*>(p.H) + (static_cast<int64_t>(b) * p.h_seq_stride + (j - 1) * p.d) * h_es,
                              static_cast<uint32_t>(p.d * h_es));
+    };
+#pragma unroll
+    for (int a = 1; a < kWarpLookahead; ++a) prefetch(warp + a * kWarps);
+    const float nq = cta_query_norm<TH>(p, b, t, wnq);
+    for (int k = warp; k < n_local; k += kWarps) {
+        prefetch(k + kWarpLookahead * kWarps);
+        const int64_t j = cand(k);
+        float s_h, s_a;
+        warp_score<TH>(p, b, j, t, nq, s_h, s_a);
+        if (lane == 0) take_score<TH>(p, rank + S * k, j, s_h, s_a, hsc, asc, best);
+    }
+    return best;
+}
+
+// The candidates of a sequence whose occurrences were not gathered (a token the index
+// cannot answer for): one CTA scans the context and writes the candidate list, its first
+// `keep` entries to `first` (shared) too.  Kept out of line: its registers do not weigh
+// on the common path.  CTA-uniform call, a barrier at the end.
+template <bool IVEC, typename RD>
+__device__ __noinline__ void rescan(const DraftParams& p, int64_t t, const int32_t* row, int32_t* cand_row,
+                                    ScanLists<kRescanPerWarp>& sl, int32_t* first, int keep, int& nstar, int& total) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid < PLDP_MAX_NGRAM) sl.suf[tid] = (tid < p.ngram_max && t - tid >= 0) ? RD::one(row + t - tid) : 0;
+    const int64_t seg = (t + kScanChunkUnit - 1) / kScanChunkUnit * kScanTile;      // positions per warp
+    const int64_t s0 = warp * seg;
+    const int nit = static_cast<int>(seg / kScanTile);
+    {
+        WarpScan<IVEC, RD, kRescanLoads> sc;
+        sc.begin(row, s0, nit, p.T_cap, lane);
+        __syncthreads();                                          // the suffix is in
+        scan_lists(sc, t, p.ngram_max, warp, sl);
     }
     __syncthreads();
-
-    // ---- 1. scan this chunk for x_t ------------------------------------------------------
-    const int64_t c1 = c0 + kChunk < t ? c0 + kChunk : t;
-    if (valid && t >= 1 && c0 < c1) {
-        const int32_t xt = sh.suf[0];
-        uint64_t mask = 0;                                        // bit i: this thread's i-th position
-#pragma unroll
-        for (int u = 0; u < NV; ++u) {
-            if constexpr (IVEC) {
-                const int64_t q = (c0 >> 2) + tid + u * kThreads;
-                const int32_t e[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (e[k] == xt && 4 * q + k < c1) mask |= 1ull << (4 * u + k);
-            } else {
-                const int64_t j = c0 + tid + u * kThreads;
-                if (j < c1 && v[u] == xt) mask |= 1ull << u;
-            }
-        }
-        while (mask) {                                            // rarely more than one
-            const int bit = __ffsll(static_cast<long long>(mask)) - 1;
-            mask &= mask - 1;
-            int64_t j;
-            if constexpr (IVEC)
-                j = 4 * ((c0 >> 2) + tid + (bit >> 2) * kThreads) + (bit & 3);
-            else
-                j = c0 + tid + static_cast<int64_t>(bit) * kThreads;
-            int m = 1;                                            // common suffix of x[..j] and x[..t]
-            while (m < p.ngram_max && j - m >= 0 && __ldg(row + j - m) == sh.suf[m]) ++m;
-            const int k = atomicAdd(&sh.nhit, 1);
-            if (k < kHitCap) {                                    // more: the list overflows anyway
-                sh.hit[k] = Hit{static_cast<int32_t>(j), m};
-                if (HAS_H && j >= 1)
-                    prefetch_l2_bulk(static_cast<const char*>(p.H) +
-                                         (static_cast<int64_t>(b) * p.h_seq_stride + (j - 1) * p.d) * h_es,
-                                     static_cast<uint32_t>(p.d * h_es));
-            }
-        }
-    }
+    const CtaMatches cm = cta_matches(sl, warp);
+    nstar = cm.m >= p.ngram_min ? cm.m : 0;
+    total = nstar > 0 ? cm.cnt : 0;
+    scan_emit<IVEC, RD>(row, s0, nit, t, p.T_cap, p.ngram_max, nstar, cm.base, p.C_cap, warp, lane, sl,
+                        [&](int64_t i, int32_t j) {
+                            cand_row[i] = j;
+                            if (i < keep) first[i] = j;
+                        });
     __syncthreads();
+}
 
-    // ---- 2. score what this CTA found ----------------------------------------------------
-    // One atomic reserves the CTA's slots in the sequence's list; its answer is
-    // needed only when the entries are written, so it runs under the scoring.
-    const int nhit = sh.nhit;
-    if (nhit > 0) {
-        unsigned base = 0;
-        if (tid == 0) base = atomicAdd(hdr, static_cast<unsigned>(nhit));
-        if (nhit > 8) {                                           // skip the scores of a list that overflowed
-            if (tid == 0) sh.skip = base + static_cast<unsigned>(nhit) > static_cast<unsigned>(kHitCap);
-            __syncthreads();
-        }
-        if (nhit <= 8 || !sh.skip)                                // (nhit > kHitCap always skips)
-            for (int k = 0; k < nhit; k += kScoreBatch) {
-                const int nb = nhit - k < kScoreBatch ? nhit - k : kScoreBatch;
-                int64_t j[kScoreBatch];
-#pragma unroll
-                for (int h = 0; h < kScoreBatch; ++h) j[h] = h < nb ? sh.hit[k + h].j : -1;
-                float s_h[kScoreBatch], s_a[kScoreBatch];
-                cta_score<TH, kScoreBatch>(p, b, j, nb, t, part_buf<kScoreBatch>(sh.part[(k / kScoreBatch) & 1]), s_h,
-                                           s_a);
-                if (tid == 0)
-                    for (int h = 0; h < nb; ++h) {
-                        const Hit e = sh.hit[k + h];
-                        const unsigned slot = base + static_cast<unsigned>(k + h);
-                        if (slot < static_cast<unsigned>(kHitCap))
-                            seq_entries(p.ws, b)[slot] = make_uint4(static_cast<unsigned>((e.j << 4) | e.m),
-                                                                    __float_as_uint(s_h[h]), __float_as_uint(s_a[h]), 0u);
-                    }
-            }
+// Per-sequence outputs of a context length outside [0, T_cap].
+template <bool HAS_H>
+__device__ __forceinline__ void no_draft(const DraftParams& p, int b) {
+    for (int i = threadIdx.x; i < p.K; i += kThreads) p.draft[static_cast<int64_t>(b) * p.K + i] = -1;
+    if (threadIdx.x != 0) return;
+    p.cand_count[b] = 0;
+    p.match_len[b] = 0;
+    if (HAS_H) {
+        p.best_h[b] = -1;
+        if (p.best_h_score) p.best_h_score[b] = -INFINITY;
     }
-
-    // ---- 3. ticket: the last CTA of the sequence finishes it -----------------------------
-    if (tid == 0) {
-        __threadfence();                                          // entries before the ticket
-        sh.last = atomicAdd(hdr + 1, 1u) == gridDim.x - 1;
-        __threadfence();
+    if (p.A != nullptr) {
+        p.best_a[b] = -1;
+        if (p.best_a_score) p.best_a_score[b] = -INFINITY;
     }
-    if (tid <= PLDP_MAX_NGRAM) sh.ss.cnt[tid] = 0;
-    __syncthreads();
-    if (!sh.last) return;
+    p.draft_len[b] = 0;
+    if (p.status) atomicOr(p.status + b, PLDP_ST_SEQ_LEN);
+}
 
+// The scanning kernel's shared memory.
+struct ScanStepShared {
+    StepShared st;
+    ScanLists<kListPerWarp> sl;
+    int32_t list[kList];                                          // this CTA's longest matches, ascending
+    int32_t mine[kList];                                          // the candidates this CTA scores
+    ScanPeer tab[kScanMaxCluster];                                // every CTA's outcome
+    unsigned long long key[kScanMaxCluster][2];                   // CTA 0: every CTA's best keys
+};
+
+template <typename TH, bool IVEC>
+__global__ void __launch_bounds__(kThreads, 3) draft_step_kernel(const DraftParams p, int CL, int64_t chunk) {
+    constexpr bool HAS_H = !std::is_same<TH, NoHidden>::value;
+    __shared__ ScanStepShared sh;
+    pdl_enter();
+    const int b = blockIdx.x / CL;
+    const int rank = blockIdx.x - b * CL;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int32_t* row = p.ids + static_cast<int64_t>(b) * p.ids_stride;
     const bool has_a = p.A != nullptr;
+    const int64_t h_es = p.h_bf16 ? 2 : 4;
+    // The chunk's first ids do not depend on seq_len: their loads go out first, bounded
+    // by the row's capacity, and land while seq_len and the suffix arrive.
+    const int64_t seg = chunk / kScanWarps;
+    const int64_t s0 = static_cast<int64_t>(rank) * chunk + warp * seg;
+    const int nit = static_cast<int>(seg / kScanTile);
+    WarpScan<IVEC, ReadOnlyIds, kScanLoads> sc;
+    sc.begin(row, s0, nit, p.T_cap, lane);
+    const int64_t L = p.seq_len[b];
+    const int64_t t = L - 1;
+    if (L < 0 || L > p.T_cap) {                                   // the same for every CTA of the cluster
+        if (rank == 0) no_draft<HAS_H>(p, b);
+        return;
+    }
+    cg::cluster_group cluster = cg::this_cluster();
+    if (CL > 1) cluster_arrive_relaxed();                         // this CTA runs: its shared memory may be written
+    if (tid < PLDP_MAX_NGRAM)                                     // x_t and the n_max - 1 tokens before it
+        sh.sl.suf[tid] = (tid < p.ngram_max && t - tid >= 0) ? __ldg(row + t - tid) : 0;
+    const char* hrows = static_cast<const char*>(p.H) + static_cast<int64_t>(b) * p.h_seq_stride * h_es;
+    if (HAS_H && tid == 32 && rank == 0 && t >= 2)                // H_{t-1}: every score reads it
+        prefetch_l2_bulk(hrows + (t - 1) * p.d * h_es, static_cast<uint32_t>(p.d * h_es));
     bool bad = false;                                             // a selected row outside [0, R)
-    if (has_a && valid && p.row_idx)
+    if (rank == 0 && has_a && p.row_idx)
         for (int k = tid; k < p.n_sel; k += kThreads) {
             const int r = __ldg(p.row_idx + k);
             bad |= r < 0 || r >= p.R;
         }
-    const unsigned nh = __ldcg(hdr);
     bad = __syncthreads_or(bad) != 0;
 
-    if (!valid) {
-        for (int i = tid; i < p.K; i += kThreads) p.draft[static_cast<int64_t>(b) * p.K + i] = -1;
-        if (tid == 0) {
-            p.cand_count[b] = 0;
-            p.match_len[b] = 0;
-            if (HAS_H) {
-                p.best_h[b] = -1;
-                if (p.best_h_score) p.best_h_score[b] = -INFINITY;
-            }
-            if (has_a) {
-                p.best_a[b] = -1;
-                if (p.best_a_score) p.best_a_score[b] = -INFINITY;
-            }
-            p.draft_len[b] = 0;
-            if (p.status) atomicOr(p.status + b, PLDP_ST_SEQ_LEN);
-            hdr[0] = 0u;
-            hdr[1] = 0u;
+    // ---- 1. this chunk's longest matches -----------------------------------------------------
+    scan_lists(sc, t, p.ngram_max, warp, sh.sl);
+    __syncthreads();
+    const CtaMatches cm = cta_matches(sh.sl, warp);
+    if (!cm.over && cm.m > 0 && sh.sl.wm[warp] == cm.m)           // their list, in order
+        for (int i = lane; i < sh.sl.wc[warp]; i += 32) {
+            const int32_t j = sh.sl.pos[warp][i];
+            sh.list[cm.base + i] = j;
+            if (HAS_H && j >= 1 && cm.m >= p.ngram_min && cm.base + i < kWarps)   // likely candidates
+                prefetch_l2_bulk(hrows + (j - 1) * p.d * h_es, static_cast<uint32_t>(p.d * h_es));
         }
-        return;
+    if (CL > 1) {
+        cluster_wait();
+        if (tid < CL) *cluster.map_shared_rank(&sh.tab[rank], tid) = ScanPeer{cm.m, cm.cnt, cm.over ? 1 : 0};
+        cluster_arrive();
+        cluster_wait();                                           // every CTA's outcome and list are in
+    } else {
+        if (tid == 0) sh.tab[0] = ScanPeer{cm.m, cm.cnt, cm.over ? 1 : 0};
+        __syncthreads();
     }
 
+    // ---- 2. the candidate list; every CTA scores its share -----------------------------------
+    const ScanTotal tt = scan_total(sh.tab, CL, rank, p.ngram_min);
+    const int n = tt.total < p.C_cap ? tt.total : p.C_cap;
+    const int n_local = n > rank ? (n - rank + CL - 1) / CL : 0;
     int32_t* cand_row = p.cand_pos + static_cast<int64_t>(b) * p.C_cap;
     float* hsc = (HAS_H && p.h_scores) ? p.h_scores + static_cast<int64_t>(b) * p.C_cap : nullptr;
     float* asc = (has_a && p.a_scores) ? p.a_scores + static_cast<int64_t>(b) * p.C_cap : nullptr;
-    unsigned long long hk = 0, ak = 0;                            // this thread's best keys
-    int nstar, total;
-    if (nh <= static_cast<unsigned>(kHitCap)) {
-        // ---- the list: one entry per thread ----
-        const bool have = tid < static_cast<int>(nh);
-        uint4 e = make_uint4(0u, 0u, 0u, 0u);
-        if (have) e = __ldcg(seq_entries(p.ws, b) + tid);
-        const int m = have ? static_cast<int>(e.x & 15u) : 0;
-        const int32_t j = static_cast<int32_t>(e.x >> 4);
-        const int wm = __reduce_max_sync(0xFFFFFFFFu, m);
-        if (lane == 0) sh.wmax[warp] = wm;
-        __syncthreads();
-        int mx = 0;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) mx = max(mx, sh.wmax[w]);
-        nstar = mx >= p.ngram_min ? mx : 0;                       // m <= ngram_max already
-        const bool cand = have && nstar > 0 && m >= nstar;
-        sh.jl[tid] = cand ? j : INT_MAX;
-        total = __syncthreads_count(cand);
-        if (cand) {
-            int r = 0;                                            // positions are distinct: so are ranks
-            for (int k = 0; k < static_cast<int>(nh); ++k) r += sh.jl[k] < j ? 1 : 0;
-            if (r < p.C_cap) {
-                cand_row[r] = j;
-                const float s_h = __uint_as_float(e.y), s_a = __uint_as_float(e.z);
-                if (HAS_H) {
-                    if (hsc) hsc[r] = s_h;
-                    if (j >= 1 && s_h > p.threshold) hk = pack_key(s_h, static_cast<uint32_t>(j));
-                }
-                if (has_a) {
-                    if (asc) asc[r] = s_a;
-                    ak = pack_key(s_a, static_cast<uint32_t>(j));
-                }
+    BestKeys best = {0, 0};
+    if (!tt.over) {
+        for (int k = tid; k < n_local; k += kThreads) {           // candidate rank + CL k: whose list, and where
+            int i = rank + CL * k, r = 0;
+            while (sh.tab[r].m != tt.nstar || i >= sh.tab[r].cnt) {
+                if (sh.tab[r].m == tt.nstar) i -= sh.tab[r].cnt;
+                ++r;
             }
+            const int32_t j = CL > 1 ? *cluster.map_shared_rank(&sh.list[i], r) : sh.list[i];
+            sh.mine[k] = j;
+            cand_row[rank + CL * k] = j;
         }
+        __syncthreads();
     } else {
-        finish_overflow<TH, IVEC, kScoreBatch>(p, b, t, row, cand_row, hsc, asc, sh, hk, ak, nstar, total);
+        // more matches in a warp's segment than its list holds: the list goes through
+        // the caller's candidate row
+        scan_emit<IVEC, ReadOnlyIds>(row, s0, nit, t, p.T_cap, p.ngram_max, tt.nstar,
+                                     static_cast<int64_t>(tt.before) + cm.base, p.C_cap, warp, lane, sh.sl,
+                                     [&](int64_t i, int32_t j) { cand_row[i] = j; });
+        if (CL > 1) {
+            cluster_arrive();
+            cluster_wait();
+        } else {
+            __syncthreads();
+        }
+    }
+    if (n_local > kCtaPasses * kScoreBatch) {
+        best = score_by_warps<TH>(p, b, t, n_local, rank, CL, sh.mine, tt.over ? 0 : n_local, cand_row, hsc, asc, sh.st.wnq);
+    } else {
+        for (int k0 = 0; k0 < n_local; k0 += kScoreBatch) {
+            int64_t j[kScoreBatch];
+#pragma unroll
+            for (int h = 0; h < kScoreBatch; ++h)
+                j[h] = k0 + h >= n_local ? -1 : tt.over ? __ldcg(cand_row + rank + CL * (k0 + h)) : sh.mine[k0 + h];
+            const int nb = n_local - k0 < kScoreBatch ? n_local - k0 : kScoreBatch;
+            float s_h[kScoreBatch], s_a[kScoreBatch];
+            cta_score<TH, kScoreBatch>(p, b, j, nb, t, part_buf<kScoreBatch>(sh.st.part[(k0 / kScoreBatch) & 1]), s_h, s_a);
+            if (tid == 0)
+#pragma unroll
+                for (int h = 0; h < kScoreBatch; ++h)
+                    if (h < nb) take_score<TH>(p, rank + CL * (k0 + h), j[h], s_h[h], s_a[h], hsc, asc, best);
+        }
     }
 
-    // ---- best of each ranking, then the draft (Sec. 4.3) ----------------------------------
-    hk = warp_max_u64(hk);
-    ak = warp_max_u64(ak);
+    // ---- 3. best of each ranking, then the draft (Sec. 4.3) ----------------------------------
+    unsigned long long hk = warp_max_u64(best.h), ak = warp_max_u64(best.a);
     if (lane == 0) {
-        sh.wkey[0][warp] = hk;
-        sh.wkey[1][warp] = ak;
+        sh.st.wkey[0][warp] = hk;
+        sh.st.wkey[1][warp] = ak;
     }
     __syncthreads();
-    if (warp != 0) return;
+    if (tid < 2) {
+        unsigned long long k = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) k = sh.st.wkey[tid][w] > k ? sh.st.wkey[tid][w] : k;
+        *(CL > 1 ? cluster.map_shared_rank(&sh.key[rank][tid], 0) : &sh.key[0][tid]) = k;
+    }
+    if (CL > 1) {
+        cluster_arrive();
+        cluster_wait();                                           // no CTA leaves while its list may be read
+    }
+    if (rank != 0 || warp != 0) return;
+    __syncwarp();
     hk = 0;
     ak = 0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-        hk = sh.wkey[0][w] > hk ? sh.wkey[0][w] : hk;
-        ak = sh.wkey[1][w] > ak ? sh.wkey[1][w] : ak;
+    for (int r = 0; r < CL; ++r) {
+        hk = sh.key[r][0] > hk ? sh.key[r][0] : hk;
+        ak = sh.key[r][1] > ak ? sh.key[r][1] : ak;
     }
     const int32_t bh = hk == 0 ? -1 : static_cast<int32_t>(key_index(hk));
     const int32_t ba = ak == 0 ? -1 : static_cast<int32_t>(key_index(ak));
@@ -601,8 +662,8 @@ __global__ void __launch_bounds__(kThreads, 4) draft_step_kernel(const DraftPara
     for (int i = lane; i < p.K; i += 32)
         p.draft[static_cast<int64_t>(b) * p.K + i] = (i < dl) ? __ldg(row + js + 1 + i) : -1;
     if (lane == 0) {
-        p.cand_count[b] = total;
-        p.match_len[b] = nstar;
+        p.cand_count[b] = tt.total;
+        p.match_len[b] = tt.nstar;
         if (HAS_H) {
             p.best_h[b] = bh;
             if (p.best_h_score) p.best_h_score[b] = bh >= 0 ? key_value(hk) : -INFINITY;
@@ -612,10 +673,8 @@ __global__ void __launch_bounds__(kThreads, 4) draft_step_kernel(const DraftPara
             if (p.best_a_score) p.best_a_score[b] = ba >= 0 ? key_value(ak) : -INFINITY;
         }
         p.draft_len[b] = static_cast<int32_t>(dl);
-        if (p.status && total > p.C_cap) atomicOr(p.status + b, PLDP_ST_CAND_OVERFLOW);
+        if (p.status && tt.total > p.C_cap) atomicOr(p.status + b, PLDP_ST_CAND_OVERFLOW);
         if (p.status && bad) atomicOr(p.status + b, PLDP_ST_ROW_INDEX);
-        hdr[0] = 0u;                                              // ready for the next call
-        hdr[1] = 0u;
     }
 }
 
@@ -630,7 +689,7 @@ __global__ void __launch_bounds__(kThreads, 4) draft_step_kernel(const DraftPara
 //    most kIndexSlots the slots are every occurrence before ilen, and the
 //    positions appended since (ilen .. t-1, read anyway) supply the rest;
 //  * otherwise (a frequent token, a stale or unusable index) falls back to the
-//    ordered rescan of the context, so results are those of the scan either way;
+//    rescan of the context, so results are those of the scan either way;
 //  * appends positions ilen .. t-1 to the index and sets ilen = t.  Each
 //    appended position takes its slot with an atomic on its token's count; the
 //    answer is used (the slot written) only at the end of the CTA, and tokens
@@ -659,12 +718,20 @@ struct IndexView {
     int V;
 };
 
+// Kept below 10 KB a CTA: the streaming pass that runs before the fused kernel leaves
+// the SMs configured for little shared memory, and CTAs that need more wait for an SM
+// to drain (16 KB measured 2.2 us more per step at the sustained-loop shape).
 struct IndexShared {
-    int32_t occ[kOccCap];              // occurrences of x_t, ascending
-    int32_t occ_m[kOccCap];            // their suffix-match lengths
+    union {
+        struct {
+            int32_t occ[kOccCap];          // occurrences of x_t, ascending
+            int32_t occ_m[kOccCap];        // their suffix-match lengths
+            int32_t occ_new[kNewCap];      // the appended occurrences, ascending
+        };
+        ScanLists<kRescanPerWarp> sl;      // the rescan, which has no occurrences at hand
+    };
     int32_t cand[kOccCap];             // the candidates (match length >= n*), ascending
     int32_t newtok[kNewCap];           // ids of positions il .. t-1
-    int32_t occ_new[kNewCap];          // the appended occurrences, ascending
     int32_t suf[PLDP_MAX_NGRAM];       // x_t, x_{t-1}, ...
     int nocc, ncand, nstar, bad_token, indexed, wmax[kWarps];
 };
@@ -714,25 +781,10 @@ __device__ __forceinline__ void index_draft(const DraftParams& p, const IndexVie
             const int r = __ldg(p.row_idx + k);
             bad |= r < 0 || r >= p.R;
         }
-    if (tid <= PLDP_MAX_NGRAM) sh.ss.cnt[tid] = 0;
     if (tid == 0) is.bad_token = 0;
     bad = __syncthreads_or(bad) != 0;
     if (!valid) {
-        for (int i = tid; i < p.K; i += kThreads) p.draft[static_cast<int64_t>(b) * p.K + i] = -1;
-        if (tid == 0) {
-            p.cand_count[b] = 0;
-            p.match_len[b] = 0;
-            if (HAS_H) {
-                p.best_h[b] = -1;
-                if (p.best_h_score) p.best_h_score[b] = -INFINITY;
-            }
-            if (has_a) {
-                p.best_a[b] = -1;
-                if (p.best_a_score) p.best_a_score[b] = -INFINITY;
-            }
-            p.draft_len[b] = 0;
-            if (p.status) atomicOr(p.status + b, PLDP_ST_SEQ_LEN);
-        }
+        no_draft<HAS_H>(p, b);
         return;
     }
     // usable: the index covers a prefix of the context; small: what was appended fits the CTA
@@ -847,12 +899,12 @@ __device__ __forceinline__ void index_draft(const DraftParams& p, const IndexVie
     // ---- the list scored: every occurrence, or the candidates --------------------------
     // spec: at most kSpeculate occurrences, all scored at once; their suffix matches
     // are read in the same round trip and n* then picks the candidates among them.
-    // Otherwise the suffix matches come first (each scored occurrence costs a
-    // d-element row and R scattered attention values) and only the candidates
-    // (the first C_cap) are scored.  Either way one loop with one call of the
-    // scorer, kSpeculate positions a pass: every case runs the same code.
+    // Otherwise the candidates (the first C_cap) are known first, from the occurrences'
+    // suffix matches or from a rescan of the context: a few go through the same code,
+    // kSpeculate a pass (one loop with one call of the scorer: a second copy, run only by
+    // the sequences with more, cost them its instruction fetch), many by a warp each.
     constexpr int NB = kSpeculate;
-    unsigned long long hk = 0, ak = 0;
+    BestKeys best = {0, 0};
     int nstar = 0, total = 0;
     const bool spec = indexed && nocc <= kSpeculate;
     if (indexed && !spec) {
@@ -901,12 +953,12 @@ __device__ __forceinline__ void index_draft(const DraftParams& p, const IndexVie
         nstar = is.nstar;
         total = is.ncand;
     } else if (!indexed) {
-        finish_overflow<TH, IVEC, kMaxScoreBatch, RD>(p, b, t, row, cand_row, hsc, asc, sh, hk, ak, nstar, total);
+        rescan<IVEC, RD>(p, t, row, cand_row, is.sl, is.cand, kOccCap, nstar, total);
     }
 
-    if (indexed) {
+    const int n = spec ? nocc : (total < p.C_cap ? total : p.C_cap);
+    if (n <= kCtaPasses * NB) {
         const int32_t* list = spec ? is.occ : is.cand;
-        const int n = spec ? nocc : (total < p.C_cap ? total : p.C_cap);
         int32_t pre[PLDP_MAX_NGRAM - 1];                          // spec, thread h < n: x_{j-1}, x_{j-2}, ...
         const int64_t jm = (spec && tid < n) ? list[tid] : -1;
 #pragma unroll
@@ -930,24 +982,12 @@ __device__ __forceinline__ void index_draft(const DraftParams& p, const IndexVie
 #pragma unroll
             for (int h = 0; h < NB; ++h) j[h] = h < nb ? list[i0 + h] : -1;
             cta_score<TH, NB>(p, b, j, nb, t, part_buf<NB>(sh.part[(i0 / NB) & 1]), s_h, s_a);
-            if (!spec && warp == 0)                               // candidates: keys now
+            if (!spec && warp == 0)                               // candidates: keys now, in every lane
 #pragma unroll
-                for (int h = 0; h < NB; ++h) {
-                    if (h >= nb) continue;
-                    const int r = i0 + h;
-                    if (HAS_H) {
-                        if (hsc && lane == 0) hsc[r] = s_h[h];
-                        if (j[h] >= 1 && s_h[h] > p.threshold) {
-                            const unsigned long long key = pack_key(s_h[h], static_cast<uint32_t>(j[h]));
-                            hk = key > hk ? key : hk;
-                        }
-                    }
-                    if (has_a) {
-                        if (asc && lane == 0) asc[r] = s_a[h];
-                        const unsigned long long key = pack_key(s_a[h], static_cast<uint32_t>(j[h]));
-                        ak = key > ak ? key : ak;
-                    }
-                }
+                for (int h = 0; h < NB; ++h)
+                    if (h < nb)
+                        take_score<TH>(p, i0 + h, j[h], s_h[h], s_a[h], lane == 0 ? hsc : nullptr,
+                                       lane == 0 ? asc : nullptr, best);
         }
         if (mine) index_put(ix, b, mytok, myslot, il + tid);      // the slot taken above
         if (warp != 0) return;
@@ -974,24 +1014,14 @@ __device__ __forceinline__ void index_draft(const DraftParams& p, const IndexVie
                     if (h >= n || mh[h] < nstar) continue;
                     if (r < p.C_cap) {
                         if (lane == 0) cand_row[r] = static_cast<int32_t>(j0[h]);
-                        if (HAS_H) {
-                            if (hsc && lane == 0) hsc[r] = s_h[h];
-                            if (j0[h] >= 1 && s_h[h] > p.threshold) {
-                                const unsigned long long key = pack_key(s_h[h], static_cast<uint32_t>(j0[h]));
-                                hk = key > hk ? key : hk;
-                            }
-                        }
-                        if (has_a) {
-                            if (asc && lane == 0) asc[r] = s_a[h];
-                            const unsigned long long key = pack_key(s_a[h], static_cast<uint32_t>(j0[h]));
-                            ak = key > ak ? key : ak;
-                        }
+                        take_score<TH>(p, r, j0[h], s_h[h], s_a[h], lane == 0 ? hsc : nullptr,
+                                       lane == 0 ? asc : nullptr, best);
                     }
                     ++r;
                 }
             total = r;
         }
-        outputs(hk, ak, nstar, total, [&](int i, int64_t js) -> int32_t {
+        outputs(best.h, best.a, nstar, total, [&](int i, int64_t js) -> int32_t {
             if (staged && i == lane) {
                 int32_t v = -1;
                 bool found = false;
@@ -1008,9 +1038,9 @@ __device__ __forceinline__ void index_draft(const DraftParams& p, const IndexVie
         return;
     }
 
-    // ---- the rescan's keys, combined over the CTA, then the outputs ---------------------
-    hk = warp_max_u64(hk);
-    ak = warp_max_u64(ak);
+    // ---- many candidates: a warp each, their keys combined over the CTA -----------------
+    best = score_by_warps<TH>(p, b, t, n, 0, 1, is.cand, kOccCap, cand_row, hsc, asc, sh.wnq);
+    unsigned long long hk = warp_max_u64(best.h), ak = warp_max_u64(best.a);
     if (lane == 0) {
         sh.wkey[0][warp] = hk;
         sh.wkey[1][warp] = ak;
@@ -1157,12 +1187,12 @@ inline IndexView index_view(void* base, int B, int V) {
 
 template <typename TH, bool IVEC>
 pldp_status launch_t(const DraftParams& p, int B, cudaStream_t s) {
-    int64_t chunks = (p.T_cap + kChunk - 1) / kChunk;
-    if (chunks < 1) chunks = 1;                                   // every sequence needs its finish
-    if (chunks > 65535) return fail(PLDP_ERR_UNSUPPORTED, "draft_step: T_cap too large for the grid");
-    cudaError_t e = launch_pdl(draft_step_kernel<TH, IVEC>,
-                               dim3(static_cast<unsigned>(chunks), static_cast<unsigned>(B)), dim3(kThreads), 0, s,
-                               0, p);
+    int CL;
+    int64_t chunk;
+    scan_shape(p.T_cap, B, resident_blocks(reinterpret_cast<const void*>(&draft_step_kernel<TH, IVEC>), kThreads, 0),
+               kPositionsPerCta, &CL, &chunk);
+    const cudaError_t e = launch_pdl(draft_step_kernel<TH, IVEC>, dim3(static_cast<unsigned>(B) * CL), dim3(kThreads), 0,
+                                     s, CL > 1 ? CL : 0, p, CL, chunk);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "draft_step: launch failed: %s", cudaGetErrorString(e));
     return PLDP_OK;
 }
@@ -1284,7 +1314,6 @@ pldp_status prepare_draft(const pldp_draft_step_args* a, const char* what, Draft
     p.draft = a->draft;
     p.draft_len = a->draft_len;
     p.status = a->status;
-    p.ws = static_cast<unsigned char*>(a->workspace);
     ivec = aligned16(a->ids) && a->ids_stride % 4 == 0 && a->T_cap % 4 == 0;
     return PLDP_OK;
 }

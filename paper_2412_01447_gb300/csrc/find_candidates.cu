@@ -1,69 +1,74 @@
 // pldp_find_candidates: the candidate search of PLD+ (Eq. 1, Sec. 4.2, with the
 // longest-suffix n-gram rule) as its own kernel -- one thread-block cluster per
-// sequence running the scan of pldp_scan.cuh.
+// sequence running the scan of pldp_scan.cuh.  Each CTA scans its chunk once, the
+// cluster's CTAs tell each other their longest match and its count over distributed
+// shared memory, and the CTAs that hold the longest write their positions.
 #include "pldp_scan.cuh"
 
 namespace pldp {
 namespace {
 
-constexpr int64_t kPositionsPerCta = 4096;
+constexpr int64_t kPositionsPerCta = 1024;   // at least; the batch sets the rest (one wave)
+constexpr int kFindList = 128;               // positions listed per warp
 
 template <bool VEC>
-__global__ void __launch_bounds__(kScanThreads)
+__global__ void __launch_bounds__(kScanThreads, 3)
 find_candidates_kernel(const int32_t* __restrict__ ids, int64_t ids_stride,
                        const int32_t* __restrict__ seq_len, int64_t T_cap, int ngram_min,
                        int ngram_max, int32_t* __restrict__ cand_pos, int C_cap,
                        int32_t* __restrict__ cand_count, int32_t* __restrict__ match_len,
-                       uint32_t* __restrict__ status, int64_t chunk) {
-    __shared__ ScanShared sh;
+                       uint32_t* __restrict__ status, int CL, int64_t chunk) {
+    __shared__ ScanLists<kFindList> sl;
+    __shared__ ScanPeer tab[kScanMaxCluster];
     pdl_enter();
-    cg::cluster_group cluster = cg::this_cluster();
-    const int CL = static_cast<int>(cluster.num_blocks());
-    const int rank = static_cast<int>(cluster.block_rank());
     const int b = blockIdx.x / CL;
-    const int tid = threadIdx.x;
+    const int rank = blockIdx.x - b * CL;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int32_t* row = ids + static_cast<int64_t>(b) * ids_stride;
+    // the chunk's first ids are requested before the context length is known
+    const int64_t seg = chunk / kScanWarps;
+    const int64_t s0 = static_cast<int64_t>(rank) * chunk + warp * seg;
+    const int nit = static_cast<int>(seg / kScanTile);
+    WarpScan<VEC, ReadOnlyIds, 8> sc;
+    sc.begin(row, s0, nit, T_cap, lane);
 
     // Every CTA of the cluster sees the same seq_len, so these exits are
     // cluster-uniform and no CTA is left waiting at a cluster barrier.
     const int64_t L = seq_len[b];
-    if (L < 0 || L > T_cap) {
-        if (rank == 0 && tid == 0) {
-            cand_count[b] = 0;
-            match_len[b] = 0;
-            if (status) status[b] |= PLDP_ST_SEQ_LEN;
-        }
-        return;
-    }
     const int64_t t = L - 1;
-    if (t < 1) {
+    if (L < 0 || L > T_cap || t < 1) {
         if (rank == 0 && tid == 0) {
             cand_count[b] = 0;
             match_len[b] = 0;
+            if ((L < 0 || L > T_cap) && status) status[b] |= PLDP_ST_SEQ_LEN;
         }
         return;
     }
-    const int32_t* row = ids + static_cast<int64_t>(b) * ids_stride;
-    if (tid <= PLDP_MAX_NGRAM) sh.cnt[tid] = 0;
-    const int64_t c0 = static_cast<int64_t>(rank) * chunk;
-    const int64_t c1 = min(c0 + chunk, t);
-    int c[PLDP_MAX_NGRAM];
-#pragma unroll
-    for (int k = 0; k < PLDP_MAX_NGRAM; ++k) c[k] = 0;
-    const GlobalIds src{row};
-    scan_count<VEC>(src, row, c0, c1, t, ngram_max, c);
-    __syncthreads();                       // sh.cnt zeroed before the adds
-    scan_reduce_counts(c, ngram_max, sh);
-
-    cluster.sync();                        // every CTA's counts are final
-    scan_decide(cluster, sh, CL, rank, ngram_min, ngram_max);
-    cluster_arrive();                      // remote reads done; waited for before exit
-    if (rank == 0 && tid == 0) {
-        cand_count[b] = sh.total;
-        match_len[b] = sh.nstar;
-        if (status && sh.total > C_cap) status[b] |= PLDP_ST_CAND_OVERFLOW;
+    if (CL > 1) cluster_arrive_relaxed();                 // this CTA runs: its shared memory may be written
+    if (tid < PLDP_MAX_NGRAM) sl.suf[tid] = (tid < ngram_max && t - tid >= 0) ? __ldg(row + t - tid) : 0;
+    __syncthreads();
+    scan_lists(sc, t, ngram_max, warp, sl);
+    __syncthreads();
+    const CtaMatches cm = cta_matches(sl, warp);
+    if (CL > 1) {
+        cluster_wait();
+        if (tid < CL)
+            *cg::this_cluster().map_shared_rank(&tab[rank], tid) = ScanPeer{cm.m, cm.cnt, cm.over ? 1 : 0};
+        cluster_arrive();
+        cluster_wait();                                   // every CTA's outcome is in
+    } else {
+        if (tid == 0) tab[0] = ScanPeer{cm.m, cm.cnt, cm.over ? 1 : 0};
+        __syncthreads();
     }
-    scan_write<VEC>(src, row, c0, c1, t, ngram_max, sh, cand_pos + static_cast<int64_t>(b) * C_cap, C_cap);
-    cluster_wait();
+    const ScanTotal st = scan_total(tab, CL, rank, ngram_min);
+    if (rank == 0 && tid == 0) {
+        cand_count[b] = st.total;
+        match_len[b] = st.nstar;
+        if (status && st.total > C_cap) status[b] |= PLDP_ST_CAND_OVERFLOW;
+    }
+    int32_t* dst = cand_pos + static_cast<int64_t>(b) * C_cap;
+    scan_emit<VEC, ReadOnlyIds>(row, s0, nit, t, T_cap, ngram_max, st.nstar, static_cast<int64_t>(st.before) + cm.base,
+                                C_cap, warp, lane, sl, [&](int64_t i, int32_t j) { dst[i] = j; });
 }
 
 }  // namespace
@@ -116,11 +121,11 @@ extern "C" PLDP_API pldp_status pldp_find_candidates(const int32_t* ids, int64_t
     if (vec)
         e = cudaLaunchKernelEx(&cfg, find_candidates_kernel<true>, ids, ids_stride, seq_len, T_cap,
                                ngram_min, ngram_max, cand_pos, C_cap, cand_count, match_len, status,
-                               chunk);
+                               CL, chunk);
     else
         e = cudaLaunchKernelEx(&cfg, find_candidates_kernel<false>, ids, ids_stride, seq_len, T_cap,
                                ngram_min, ngram_max, cand_pos, C_cap, cand_count, match_len, status,
-                               chunk);
+                               CL, chunk);
     if (e != cudaSuccess)
         return fail(PLDP_ERR_CUDA, "find_candidates: launch failed: %s", cudaGetErrorString(e));
     return PLDP_OK;
