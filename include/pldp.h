@@ -18,7 +18,7 @@
  *      model's K+1 next-token distributions (Sec. 4.4)    -> pldp_verify_greedy
  *      or by sampling at temperature T                    -> pldp_verify_sample
  *
- * Fused forms: pldp_draft_step runs 1-3 in one launch (scanning the contexts, or
+ * Fused forms: pldp_draft_step runs 1-3 in one call (scanning the contexts, or
  * with the incremental token index of pldp_index_build); pldp_verify_greedy_draft
  * and pldp_verify_sample_draft run 4 (greedy or by sampling) for the current step
  * and then 1-3 for the next step.  Offline:
@@ -232,11 +232,12 @@ PLDP_API pldp_status pldp_extract_draft(const int32_t* ids, int64_t ids_stride,
  * bits and a tie within rounding may be broken differently).  Eq. 1-3
  * (Sec. 4.2) and Sec. 4.3.
  *
- * One launch of a thread-block cluster per sequence.  Each CTA scans its chunk of
- * the context once and keeps the positions with the longest suffix match it met;
- * the cluster then knows the candidate list and deals the candidates out to its
- * CTAs, which score them (cosine and attention score), and its first CTA picks the
- * best of each ranking and writes the draft.
+ * A thread-block cluster per sequence: each CTA scans its chunk of the context once
+ * and keeps the positions with the longest suffix match it met; the cluster then
+ * knows the candidate list and deals the candidates out to its CTAs, which score
+ * them (cosine and attention score), and its first CTA picks the best of each
+ * ranking and writes the draft.  Sequences with many candidates are finished by a
+ * second launch that spreads them over the whole GPU (through the workspace).
  *
  * Fields of the argument block (device pointers unless stated):
  *  ids .. match_len      as pldp_find_candidates (T_cap <= 2^27).

@@ -14,7 +14,7 @@ PLD+ (arXiv 2412.01447), per decode step and per sequence:
   * ``pldp_extract_draft``   -- Sec. 4.3: the K tokens after the best occurrence;
   * ``pldp_verify_greedy``   -- Sec. 4.4: greedy accept against the target argmax;
   * ``pldp_verify_sample``   -- Sec. 4.4 with sampling, from caller uniforms.
-The fused calls: ``pldp_draft_step`` (the first four in one launch, optionally
+The fused calls: ``pldp_draft_step`` (the first four in one, optionally
 with the token index of ``pldp_index_build``), ``pldp_verify_greedy_draft`` and
 ``pldp_verify_sample_draft`` (verification, greedy or by sampling, then the next
 step's draft).  Also ``pldp_rank_hidden_avg``

@@ -1,6 +1,6 @@
 // pldp_draft_step: the drafting half of a PLD+ step -- candidate search (Eq. 1
 // with the longest-suffix n-gram rule), ranking by hidden states (Eq. 3) and/or
-// by attentions (Eq. 2), and draft extraction (Sec. 4.3) -- in one launch; and
+// by attentions (Eq. 2), and draft extraction (Sec. 4.3) -- in one call; and
 // pldp_verify_greedy_draft / pldp_verify_sample_draft: greedy or sampling
 // verification (Sec. 4.4) followed by the next step's drafting.  Three kernels:
 //  * draft_step_kernel scans the contexts (below);
@@ -21,8 +21,10 @@
 //     and the max (or sum) of the selected attention rows at key j, both in one round
 //     trip to memory;
 //  3. sends its best keys to CTA 0, which writes the choices and the draft.
-// Only candidates are scored, by all CTAs of the sequence, whatever the number of
-// occurrences of x_t.
+// Only candidates are scored, whatever the number of occurrences of x_t.  A sequence
+// with many of them (a frequent x_t in new text, Eq. 1's unigram match) is left to a
+// second launch behind it, score_deferred_kernel, which deals all such candidates of
+// the batch out to the whole GPU; so do the indexed kernels.
 //
 // Every score is the sum of the same partial sums in the same order (a fixed share per
 // thread of a CTA, combined in warp order), whether a CTA scores one candidate with
@@ -53,8 +55,12 @@ constexpr int kRescanPerWarp = 128;
 constexpr int kScoreUnroll = 2;                                // 16-byte row loads in flight
 constexpr int kScoreBatch = 2;                                 // candidates scored by the whole CTA at once (scan kernel)
 constexpr int kMaxScoreBatch = 4;                              // ... and at most (the indexed kernel)
-constexpr int kCtaPasses = 4;                                  // passes of the whole CTA before a warp takes each candidate
-constexpr int kWarpLookahead = 2;                              // candidates per warp whose hidden rows are prefetched
+// Scoring passes of a CTA; a sequence with more candidates is deferred.  Two passes cost
+// what the deferred launch does, which runs either way: on Zipf contexts 2 against 4
+// measured 31.2 / 32.0 us (drafting, batch 128 x 32k) and 1385 / 1400 us (index build and
+// 8 fused steps); one pass defers what uniform text often has (5-8 occurrences).
+constexpr int kCtaPasses = 2;
+constexpr int kMaxUnit = 64;                                   // candidates per unit of the deferred scoring, at most
 constexpr int kSpeculate = kMaxScoreBatch;                     // occurrences scored before their suffix match
 constexpr int kPrefetchOcc = 32;                                // occurrences whose rows are prefetched otherwise
 constexpr size_t kMaxQueryBytes = 196608;
@@ -98,7 +104,18 @@ struct DraftParams {
     int32_t* draft;
     int32_t* draft_len;
     uint32_t* status;
+    struct DeferSlot* defer;   // [B + 1], all zero between calls; null: nothing is deferred
 };
+
+// What the drafting kernels leave to score_deferred_kernel: `pending` candidates of a
+// sequence (its list is written); the best keys and the units done, while it runs.
+// Slot B counts its CTAs out.
+struct alignas(16) DeferSlot {
+    unsigned long long h, a;
+    unsigned pending, done;
+    unsigned pad[2];
+};
+static_assert(sizeof(DeferSlot) == 32 && 2 * sizeof(DeferSlot) <= kSeqWs, "B + 1 slots fit the workspace");
 
 // Warp reduce-scatter of N values (N a power of two, <= 32): at each butterfly
 // level a lane keeps half of its values and trades the other half with its
@@ -140,7 +157,6 @@ __device__ __forceinline__ float (&part_buf(float (&part)[kMaxScoreBatch][kWarps
 struct StepShared {
     alignas(16) float part[2][kMaxScoreBatch][kWarps][4];   // per-warp partials: dot, |a|^2, |q|^2, attention
     unsigned long long wkey[2][kWarps];      // per-warp best keys (hidden, attention)
-    float wnq[kWarps];                       // per-warp partials of |H_{t-1}|^2
 };
 
 // Eq. 3 and Eq. 2 for candidates j[0 .. nb) of sequence b (nb <= NB), by all
@@ -290,52 +306,51 @@ __device__ __forceinline__ void cta_score(const DraftParams& p, int b, const int
     }
 }
 
-// |H_{t-1}|^2 in every thread, summed as cta_score sums it.  CTA-uniform call with one
-// barrier.
+// This warp's share of |H_{t-1}|^2, in cta_score's order; sum_shares combines the eight.
 template <typename TH>
-__device__ __forceinline__ float cta_query_norm(const DraftParams& p, int b, int64_t t, float (&wnq)[kWarps]) {
+__device__ __forceinline__ float query_norm_share(const DraftParams& p, int b, int64_t t) {
     if constexpr (std::is_same<TH, NoHidden>::value) {
         return 0.f;
     } else {
         constexpr int E = 16 / sizeof(TH);
-        const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
         const TH* qrow = static_cast<const TH*>(p.H) + static_cast<int64_t>(b) * p.h_seq_stride + (t - 1) * p.d;
         const int64_t nch = p.d / E;
         float nq = 0.f;
         if (t >= 2)
-            for (int64_t c = tid; c < nch; c += kThreads) {
+            for (int64_t c = threadIdx.x; c < nch; c += kThreads) {
                 const uint4 q = __ldg(reinterpret_cast<const uint4*>(qrow) + c);
                 float dead0 = 0.f, dead1 = 0.f;
                 accum16<TH>(q, q, dead0, dead1, nq);
             }
-        nq = warp_sum(nq);
-        if (lane == 0) wnq[warp] = nq;
-        __syncthreads();
-        return ((wnq[0] + wnq[4]) + (wnq[2] + wnq[6])) + ((wnq[1] + wnq[5]) + (wnq[3] + wnq[7]));
+        return warp_sum(nq);
     }
 }
+__device__ __forceinline__ float sum_shares(const float (&x)[kWarps]) {
+    static_assert(kWarps == 8, "cta_score's tree over eight warps");
+    return ((x[0] + x[4]) + (x[2] + x[6])) + ((x[1] + x[5]) + (x[3] + x[7]));
+}
 
-// Eq. 3 and Eq. 2 for one candidate j by one warp, the results (in every lane) those of
-// cta_score bit for bit: lane l forms the partial sums of the CTA's threads l, 32 + l,
-// ..., 224 + l in eight accumulators, each in that thread's order, and they are reduced
-// over the lanes and then over the eight in the CTA's order.  nq = |H_{t-1}|^2
-// (cta_query_norm); the query row is read through L1, which the warps share.
+// Eq. 3 (dot product and |H_{j-1}|^2) and Eq. 2 for one candidate j by one warp, the
+// results (in every lane) those of cta_score bit for bit: lane l forms the partial sums
+// of the CTA's threads l, 32 + l, ..., 224 + l in eight accumulators, each in that
+// thread's order, and they are reduced over the lanes and then over the eight in the
+// CTA's order.  Sixteen 16-byte loads of the row are in flight per lane (8 KB a warp);
+// the query row is read through L1, which the CTA's warps share.
 template <typename TH>
-__device__ __forceinline__ void warp_score(const DraftParams& p, int b, int64_t j, int64_t t, float nq, float& s_h,
+__device__ __forceinline__ void warp_score(const DraftParams& p, int b, int64_t j, int64_t t, float& dot, float& na,
                                            float& s_a) {
     constexpr bool HAS_H = !std::is_same<TH, NoHidden>::value;
-    static_assert(kWarps == 8, "eight partial sums per lane");
     const int lane = threadIdx.x & 31;
     const bool is_max = p.agg == PLDP_AGG_MAX;
     const bool h_ok = HAS_H && j >= 1 && j < t, a_ok = p.A != nullptr && j >= 0 && j < t;
-    s_h = -INFINITY;
+    dot = 0.f;
+    na = 0.f;
     s_a = -INFINITY;
     // the attention values of the first 128 selected rows are requested before the
     // hidden row is used, so both arrive in one round trip
-    const size_t a_es = p.a_bf16 ? 2 : 4;
-    const char* ab = p.A ? static_cast<const char*>(p.A) +
-                               (static_cast<int64_t>(b) * p.a_seq_stride + j * p.a_key_stride) * static_cast<int64_t>(a_es)
-                         : nullptr;
+    const int64_t a_es = p.a_bf16 ? 2 : 4;
+    const char* ab =
+        p.A ? static_cast<const char*>(p.A) + (static_cast<int64_t>(b) * p.a_seq_stride + j * p.a_key_stride) * a_es : nullptr;
     auto attn = [&](int k) -> float {                             // NaN: no such row
         if (!a_ok || k >= p.n_sel) return NAN;
         const int r = p.row_idx ? __ldg(p.row_idx + k) : k;
@@ -347,32 +362,34 @@ __device__ __forceinline__ void warp_score(const DraftParams& p, int b, int64_t 
     for (int w = 0; w < kEarly; ++w) av[w] = attn(32 * w + lane);
     if constexpr (HAS_H) {
         if (h_ok) {                                               // warp-uniform
-            constexpr int E = 16 / sizeof(TH);
+            constexpr int E = 16 / sizeof(TH), U = 2 * kWarps;
             const TH* hb = static_cast<const TH*>(p.H) + static_cast<int64_t>(b) * p.h_seq_stride;
             const uint4* qrow = reinterpret_cast<const uint4*>(hb + (t - 1) * p.d);
             const TH* arow = hb + (j - 1) * p.d;
-            const int64_t nch = p.d / E;
-            float v[16];                                          // dot of share w, then |H_{j-1}|^2 of share w
+            const int nch = static_cast<int>(p.d / E);
+            float v[2 * kWarps];                                  // dot of share w, then |H_{j-1}|^2 of share w
 #pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = 0.f;
-            for (int64_t c0 = lane; c0 < nch; c0 += kThreads) {
-                uint4 a[kWarps];
+            for (int i = 0; i < 2 * kWarps; ++i) v[i] = 0.f;
+#pragma unroll 1
+            for (int c0 = lane; c0 < nch; c0 += 32 * U) {
+                uint4 a[U];
 #pragma unroll
-                for (int w = 0; w < kWarps; ++w)
-                    if (c0 + 32 * w < nch) a[w] = ld_stream16(arow + (c0 + 32 * w) * E);
+                for (int u = 0; u < U; ++u)
+                    if (c0 + 32 * u < nch) a[u] = ld_stream16(arow + static_cast<int64_t>(c0 + 32 * u) * E);
 #pragma unroll
-                for (int w = 0; w < kWarps; ++w) {
-                    if (c0 + 32 * w >= nch) continue;
-                    const uint4 q = __ldg(qrow + c0 + 32 * w);
+                for (int u = 0; u < U; ++u) {
+                    if (c0 + 32 * u >= nch) continue;
+                    const uint4 q = __ldg(qrow + c0 + 32 * u);
                     float dead = 0.f;
-                    accum16<TH>(a[w], q, v[w], v[8 + w], dead);
+                    accum16<TH>(a[u], q, v[u % kWarps], v[kWarps + u % kWarps], dead);
                 }
             }
-            float r = warp_reduce_scatter<16>(v, false);          // lane l: value l / 2
+            float r = warp_reduce_scatter<2 * kWarps>(v, false);  // lane l: value l / 2
             r += __shfl_xor_sync(0xFFFFFFFFu, r, 8);
             r += __shfl_xor_sync(0xFFFFFFFFu, r, 4);
             r += __shfl_xor_sync(0xFFFFFFFFu, r, 2);
-            s_h = finish_cosine(__shfl_sync(0xFFFFFFFFu, r, 0), __shfl_sync(0xFFFFFFFFu, r, 16), nq);
+            dot = __shfl_sync(0xFFFFFFFFu, r, 0);
+            na = __shfl_sync(0xFFFFFFFFu, r, 16);
         }
     }
     if (a_ok) {                                                   // warp-uniform
@@ -383,6 +400,7 @@ __device__ __forceinline__ void warp_score(const DraftParams& p, int b, int64_t 
             const float x = w < kEarly ? av[w] : attn(32 * w + lane);
             if (x == x) acc[w] = is_max ? fmaxf(acc[w], x) : acc[w] + x;
         }
+#pragma unroll 1
         for (int k0 = kThreads; k0 < p.n_sel; k0 += kThreads) {
             float x[kWarps];
 #pragma unroll
@@ -391,7 +409,7 @@ __device__ __forceinline__ void warp_score(const DraftParams& p, int b, int64_t 
             for (int w = 0; w < kWarps; ++w)
                 if (x[w] == x[w]) acc[w] = is_max ? fmaxf(acc[w], x[w]) : acc[w] + x[w];
         }
-        float r = warp_reduce_scatter<8>(acc, is_max);            // lane l: value l / 4
+        float r = warp_reduce_scatter<kWarps>(acc, is_max);       // lane l: value l / 4
 #pragma unroll
         for (int o = 16; o >= 4; o >>= 1) {
             const float x = __shfl_xor_sync(0xFFFFFFFFu, r, o);
@@ -424,39 +442,188 @@ __device__ __forceinline__ void take_score(const DraftParams& p, int i, int64_t 
     }
 }
 
-// This CTA's share of the candidates, a warp each: list indexes rank + S * k for
-// k < n_local, at positions near[k] (shared) for k < n_near and far[rank + S * k]
-// (global) from there.  Eight rows are on their way at once and no barrier separates
-// them; the rows of a warp's next candidates head for L2 meanwhile.  Scores go to hsc /
-// asc (if given); the best keys are returned in lane 0 of each warp.  CTA-uniform call,
-// out of line: inlined, it cost the calls with few candidates 2-5 us after an L2 flush.
-template <typename TH>
-__device__ __noinline__ BestKeys score_by_warps(const DraftParams& p, int b, int64_t t, int n_local, int rank, int S,
-                                                const int32_t* near, int n_near, const int32_t* far, float* hsc,
-                                                float* asc, float (&wnq)[kWarps]) {
-    constexpr bool HAS_H = !std::is_same<TH, NoHidden>::value;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t h_es = p.h_bf16 ? 2 : 4;
-    BestKeys best = {0, 0};
-    auto cand = [&](int k) -> int64_t { return k < n_near ? near[k] : __ldcg(far + rank + S * k); };
-    auto prefetch = [&](int k) {
-        if (!HAS_H || lane != 0 || k >= n_local) return;
-        const int64_t j = cand(k);
-        if (j >= 1 && j < t)
-            prefetch_l2_bulk(static_cast<const char*>(p.H) + (static_cast<int64_t>(b) * p.h_seq_stride + (j - 1) * p.d) * h_es,
-                             static_cast<uint32_t>(p.d * h_es));
-    };
-#pragma unroll
-    for (int a = 1; a < kWarpLookahead; ++a) prefetch(warp + a * kWarps);
-    const float nq = cta_query_norm<TH>(p, b, t, wnq);
-    for (int k = warp; k < n_local; k += kWarps) {
-        prefetch(k + kWarpLookahead * kWarps);
-        const int64_t j = cand(k);
-        float s_h, s_a;
-        warp_score<TH>(p, b, j, t, nq, s_h, s_a);
-        if (lane == 0) take_score<TH>(p, rank + S * k, j, s_h, s_a, hsc, asc, best);
+// One warp: the choices of both rankings (best keys hk, ak) and the draft (Sec. 4.3),
+// with draft_tok(i, j*) giving token j* + 1 + i.
+template <bool HAS_H, typename Tok>
+__device__ __forceinline__ void write_choice(const DraftParams& p, int b, int64_t t, unsigned long long hk,
+                                             unsigned long long ak, int lane, Tok draft_tok) {
+    const int32_t bh = hk == 0 ? -1 : static_cast<int32_t>(key_index(hk));
+    const int32_t ba = ak == 0 ? -1 : static_cast<int32_t>(key_index(ak));
+    const int64_t js = p.draft_from == 0 ? bh : ba;
+    int64_t dl = 0;
+    if (js >= 0 && js < t) dl = (t - js < p.K) ? (t - js) : p.K;
+    for (int i = lane; i < p.K; i += 32)
+        p.draft[static_cast<int64_t>(b) * p.K + i] = (i < dl) ? draft_tok(i, js) : -1;
+    if (lane != 0) return;
+    if (HAS_H) {
+        p.best_h[b] = bh;
+        if (p.best_h_score) p.best_h_score[b] = bh >= 0 ? key_value(hk) : -INFINITY;
     }
-    return best;
+    if (p.A != nullptr) {
+        p.best_a[b] = ba;
+        if (p.best_a_score) p.best_a_score[b] = ba >= 0 ? key_value(ak) : -INFINITY;
+    }
+    p.draft_len[b] = static_cast<int32_t>(dl);
+}
+
+// One thread: the candidate list's size and length, and the status bits of drafting.
+__device__ __forceinline__ void write_counts(const DraftParams& p, int b, int nstar, int total, bool bad_rows) {
+    p.cand_count[b] = total;
+    p.match_len[b] = nstar;
+    if (p.status && total > p.C_cap) atomicOr(p.status + b, PLDP_ST_CAND_OVERFLOW);
+    if (p.status && bad_rows) atomicOr(p.status + b, PLDP_ST_ROW_INDEX);
+}
+
+// The scores of the sequences that the drafting kernel before it left (`defer`), spread
+// over the whole GPU: the deferred candidates of the batch are cut into units of a few
+// per warp, about one unit per CTA, whatever sequences they belong to.  A unit's CTA
+// scores a candidate per warp at a time and adds its best keys to the sequence's slot;
+// the CTA that completes a sequence writes its choices and draft.  Nothing waits: the
+// last CTA out clears the slots.
+//
+// What bounds it: the candidates' hidden rows (8 KB each at d = 4096), random reads of
+// HBM.  One CTA scores about 25-40 GB/s of them, so the hundreds of candidates of a few
+// sequences took 100-400 us of a drafting launch (up to 8 CTAs a sequence, one in the
+// indexed kernels) while the other SMs were idle.  Drafting batch 128 x 32k Zipf tokens:
+// 125-190 -> 32 us; index build + 8 fused steps of it: 6083 -> 1400 us.  A batch without
+// deferred sequences pays the empty launch, about 2 us.
+template <typename TH>
+__global__ void __launch_bounds__(kThreads, 2) score_deferred_kernel(const DraftParams p, int B) {
+    constexpr bool HAS_H = !std::is_same<TH, NoHidden>::value;
+    __shared__ int n_of[kThreads];                                // deferred candidates of this tile's sequences
+    __shared__ int start[kThreads];                               // their first units, counted from the tile's
+    __shared__ int wsum[kWarps];
+    __shared__ unsigned long long wkey[2][kWarps];
+    __shared__ float wnq[kWarps];
+    __shared__ int last;
+    pdl_enter();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    DeferSlot* slots = p.defer;
+    int mine = 0;
+    for (int b = tid; b < B; b += kThreads) mine += static_cast<int>(__ldcg(&slots[b].pending));
+    const int ws = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(mine)));
+    if (lane == 0) wsum[warp] = ws;
+    __syncthreads();
+    int64_t all = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) all += wsum[w];
+    if (all == 0) return;
+    const int G = static_cast<int>(gridDim.x);
+    const int64_t per = (all + static_cast<int64_t>(G) * kWarps - 1) / (static_cast<int64_t>(G) * kWarps) * kWarps;
+    const int U = per < kMaxUnit ? static_cast<int>(per) : kMaxUnit;   // a multiple of kWarps
+    int64_t unit0 = 0;                                            // units of the tiles before
+    for (int b0 = 0; b0 < B; b0 += kThreads) {
+        // the tile's units: an exclusive scan over its sequences
+        const int n = b0 + tid < B ? static_cast<int>(__ldcg(&slots[b0 + tid].pending)) : 0;
+        const int units = (n + U - 1) / U;
+        int incl = units;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        __syncthreads();                                          // wsum, n_of and start have been read
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        int before = 0, total = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            before += w < warp ? wsum[w] : 0;
+            total += wsum[w];
+        }
+        n_of[tid] = n;
+        start[tid] = before + incl - units;
+        __syncthreads();
+        const int64_t skip = (unit0 + G - 1 - blockIdx.x) / G;    // this CTA's units below unit0
+        for (int64_t u = skip * G + blockIdx.x - unit0; u < total; u += G) {
+            int lo = 0, hi = kThreads - 1;                        // the last sequence that starts at or below u
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (start[mid] <= u) lo = mid;
+                else hi = mid - 1;
+            }
+            const int b = b0 + lo, nb = n_of[lo];
+            const int k0 = static_cast<int>(u - start[lo]) * U, k1 = k0 + U < nb ? k0 + U : nb;
+            const int64_t t = static_cast<int64_t>(p.seq_len[b]) - 1;
+            const int64_t row0 = static_cast<int64_t>(b) * p.C_cap;
+            // this warp's candidates k0 + warp, k0 + warp + kWarps, ...: lane i the i-th
+            const int kl = k0 + warp + lane * kWarps;
+            const int32_t jl = kl < k1 ? p.cand_pos[row0 + kl] : -1;
+            const int cnt = k1 > k0 + warp ? (k1 - k0 - warp + kWarps - 1) / kWarps : 0;
+            const float nqs = query_norm_share<TH>(p, b, t);
+            if (lane == 0) wnq[warp] = nqs;
+            float dl = 0.f, nl = 0.f, al = 0.f;
+            for (int i = 0; i < cnt; ++i) {
+                const int64_t j = __shfl_sync(0xFFFFFFFFu, jl, i);
+                if (HAS_H && i + 1 < cnt) {                       // the next row heads for L2
+                    const int64_t jn = __shfl_sync(0xFFFFFFFFu, jl, i + 1);
+                    const int64_t h_es = p.h_bf16 ? 2 : 4;
+                    if (lane == 0 && jn >= 1 && jn < t)
+                        prefetch_l2_bulk(static_cast<const char*>(p.H) +
+                                             (static_cast<int64_t>(b) * p.h_seq_stride + (jn - 1) * p.d) * h_es,
+                                         static_cast<uint32_t>(p.d * h_es));
+                }
+                float dot, na, s_a;
+                warp_score<TH>(p, b, j, t, dot, na, s_a);
+                if (lane == i) {
+                    dl = dot;
+                    nl = na;
+                    al = s_a;
+                }
+            }
+            __syncthreads();                                      // every share of the query norm is in
+            BestKeys best = {0, 0};
+            if (lane < cnt) {
+                const float s_h = (HAS_H && jl >= 1 && jl < t) ? finish_cosine(dl, nl, sum_shares(wnq)) : -INFINITY;
+                take_score<TH>(p, kl, jl, s_h, al, p.h_scores ? p.h_scores + row0 : nullptr,
+                               p.a_scores ? p.a_scores + row0 : nullptr, best);
+            }
+            const unsigned long long hw = warp_max_u64(best.h), aw = warp_max_u64(best.a);
+            if (lane == 0) {
+                wkey[0][warp] = hw;
+                wkey[1][warp] = aw;
+            }
+            __syncthreads();
+            if (tid == 0) {
+                unsigned long long hk = 0, ak = 0;
+#pragma unroll
+                for (int w = 0; w < kWarps; ++w) {
+                    hk = wkey[0][w] > hk ? wkey[0][w] : hk;
+                    ak = wkey[1][w] > ak ? wkey[1][w] : ak;
+                }
+                if (hk) atomicMax(&slots[b].h, hk);
+                if (ak) atomicMax(&slots[b].a, ak);
+                __threadfence();                                  // the keys before the count
+                last = atomicAdd(&slots[b].done, 1u) == static_cast<unsigned>((nb + U - 1) / U - 1);
+                __threadfence();
+            }
+            __syncthreads();
+            if (last && warp == 0) {                              // the sequence is complete
+                const unsigned long long hk = __ldcg(&slots[b].h), ak = __ldcg(&slots[b].a);
+                const int32_t* row = p.ids + static_cast<int64_t>(b) * p.ids_stride;
+                write_choice<HAS_H>(p, b, t, hk, ak, lane, [&](int i, int64_t js) -> int32_t { return row[js + 1 + i]; });
+                __syncwarp();
+                if (lane == 0) {
+                    slots[b].h = 0;
+                    slots[b].a = 0;
+                    slots[b].done = 0;
+                }
+            }
+            // (wkey and wnq are rewritten only after the next unit's first barrier or by
+            // their own warps; `last` after its second)
+        }
+        unit0 += total;
+    }
+    // the last CTA out clears `pending`, which the others read at their start
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        last = atomicAdd(&slots[B].done, 1u) == static_cast<unsigned>(G - 1);
+    }
+    __syncthreads();
+    if (!last) return;
+    for (int b = tid; b < B; b += kThreads) slots[b].pending = 0;
+    if (tid == 0) slots[B].done = 0;
 }
 
 // The candidates of a sequence whose occurrences were not gathered (a token the index
@@ -611,9 +778,8 @@ __global__ void __launch_bounds__(kThreads, 3) draft_step_kernel(const DraftPara
             __syncthreads();
         }
     }
-    if (n_local > kCtaPasses * kScoreBatch) {
-        best = score_by_warps<TH>(p, b, t, n_local, rank, CL, sh.mine, tt.over ? 0 : n_local, cand_row, hsc, asc, sh.st.wnq);
-    } else {
+    const bool deferred = p.defer != nullptr && n > kCtaPasses * kScoreBatch * CL;
+    if (!deferred) {
         for (int k0 = 0; k0 < n_local; k0 += kScoreBatch) {
             int64_t j[kScoreBatch];
 #pragma unroll
@@ -654,28 +820,12 @@ __global__ void __launch_bounds__(kThreads, 3) draft_step_kernel(const DraftPara
         hk = sh.key[r][0] > hk ? sh.key[r][0] : hk;
         ak = sh.key[r][1] > ak ? sh.key[r][1] : ak;
     }
-    const int32_t bh = hk == 0 ? -1 : static_cast<int32_t>(key_index(hk));
-    const int32_t ba = ak == 0 ? -1 : static_cast<int32_t>(key_index(ak));
-    const int64_t js = p.draft_from == 0 ? bh : ba;
-    int64_t dl = 0;
-    if (js >= 0 && js < t) dl = (t - js < p.K) ? (t - js) : p.K;
-    for (int i = lane; i < p.K; i += 32)
-        p.draft[static_cast<int64_t>(b) * p.K + i] = (i < dl) ? __ldg(row + js + 1 + i) : -1;
     if (lane == 0) {
-        p.cand_count[b] = tt.total;
-        p.match_len[b] = tt.nstar;
-        if (HAS_H) {
-            p.best_h[b] = bh;
-            if (p.best_h_score) p.best_h_score[b] = bh >= 0 ? key_value(hk) : -INFINITY;
-        }
-        if (has_a) {
-            p.best_a[b] = ba;
-            if (p.best_a_score) p.best_a_score[b] = ba >= 0 ? key_value(ak) : -INFINITY;
-        }
-        p.draft_len[b] = static_cast<int32_t>(dl);
-        if (p.status && tt.total > p.C_cap) atomicOr(p.status + b, PLDP_ST_CAND_OVERFLOW);
-        if (p.status && bad) atomicOr(p.status + b, PLDP_ST_ROW_INDEX);
+        write_counts(p, b, tt.nstar, tt.total, bad);
+        if (deferred) p.defer[b].pending = static_cast<unsigned>(n);
     }
+    if (!deferred)
+        write_choice<HAS_H>(p, b, t, hk, ak, lane, [&](int i, int64_t js) -> int32_t { return __ldg(row + js + 1 + i); });
 }
 
 // ---------------------------------------------------------------------------
@@ -712,6 +862,7 @@ constexpr int kDraftWin = 32;                      // draft tokens staged per oc
 static_assert(kEntryWords * 4 == 64 && kEntryWords <= 32, "an entry is 64 bytes, a word per lane");
 
 struct IndexView {
+    DeferSlot* defer;   // [B + 1], after the entries
     int32_t* ilen;      // [B]
     int32_t* flags;     // [B], build scratch
     int32_t* entries;   // [B][V][kEntryWords]
@@ -866,34 +1017,12 @@ __device__ __forceinline__ void index_draft(const DraftParams& p, const IndexVie
         }
     }
 
-    // Warp 0: the choices of both rankings (best keys hk, ak), the draft (Sec. 4.3)
-    // with draft_tok(i, j*) giving token j* + 1 + i, and the per-sequence outputs.
-    auto outputs = [&](unsigned long long hk, unsigned long long ak, int nstar, int total, auto draft_tok) {
-        const int32_t bh = hk == 0 ? -1 : static_cast<int32_t>(key_index(hk));
-        const int32_t ba = ak == 0 ? -1 : static_cast<int32_t>(key_index(ak));
-        const int64_t js = p.draft_from == 0 ? bh : ba;
-        int64_t dl = 0;
-        if (js >= 0 && js < t) dl = (t - js < p.K) ? (t - js) : p.K;
-        for (int i = lane; i < p.K; i += 32)
-            p.draft[static_cast<int64_t>(b) * p.K + i] = (i < dl) ? draft_tok(i, js) : -1;
-        if (lane == 0) {
-            p.cand_count[b] = total;
-            p.match_len[b] = nstar;
-            if (HAS_H) {
-                p.best_h[b] = bh;
-                if (p.best_h_score) p.best_h_score[b] = bh >= 0 ? key_value(hk) : -INFINITY;
-            }
-            if (has_a) {
-                p.best_a[b] = ba;
-                if (p.best_a_score) p.best_a_score[b] = ba >= 0 ? key_value(ak) : -INFINITY;
-            }
-            p.draft_len[b] = static_cast<int32_t>(dl);
-            if (p.status && total > p.C_cap) atomicOr(p.status + b, PLDP_ST_CAND_OVERFLOW);
-            if (p.status && bad) atomicOr(p.status + b, PLDP_ST_ROW_INDEX);
-            // the index now covers 0 .. t-1 (or is unusable: a token it cannot hold, or stale)
-            if (usable) ix.ilen[b] = is.bad_token ? -1 : static_cast<int32_t>(t);
-            else if (il > t && il > 0) ix.ilen[b] = -1;         // shrunk (an empty context keeps il = 0)
-        }
+    // One thread: the counts, and the index's new state.
+    auto counts = [&](int nstar, int total) {
+        write_counts(p, b, nstar, total, bad);
+        // the index now covers 0 .. t-1 (or is unusable: a token it cannot hold, or stale)
+        if (usable) ix.ilen[b] = is.bad_token ? -1 : static_cast<int32_t>(t);
+        else if (il > t && il > 0) ix.ilen[b] = -1;             // shrunk (an empty context keeps il = 0)
     };
 
     // ---- the list scored: every occurrence, or the candidates --------------------------
@@ -902,7 +1031,8 @@ __device__ __forceinline__ void index_draft(const DraftParams& p, const IndexVie
     // Otherwise the candidates (the first C_cap) are known first, from the occurrences'
     // suffix matches or from a rescan of the context: a few go through the same code,
     // kSpeculate a pass (one loop with one call of the scorer: a second copy, run only by
-    // the sequences with more, cost them its instruction fetch), many by a warp each.
+    // the sequences with more, cost them its instruction fetch); many are left to
+    // score_deferred_kernel.
     constexpr int NB = kSpeculate;
     BestKeys best = {0, 0};
     int nstar = 0, total = 0;
@@ -957,7 +1087,15 @@ __device__ __forceinline__ void index_draft(const DraftParams& p, const IndexVie
     }
 
     const int n = spec ? nocc : (total < p.C_cap ? total : p.C_cap);
-    if (n <= kCtaPasses * NB) {
+    if (p.defer != nullptr && n > kCtaPasses * NB) {
+        if (mine) index_put(ix, b, mytok, myslot, il + tid);      // the slot taken above
+        if (tid == 0) {
+            counts(nstar, total);
+            p.defer[b].pending = static_cast<unsigned>(n);
+        }
+        return;
+    }
+    {
         const int32_t* list = spec ? is.occ : is.cand;
         int32_t pre[PLDP_MAX_NGRAM - 1];                          // spec, thread h < n: x_{j-1}, x_{j-2}, ...
         const int64_t jm = (spec && tid < n) ? list[tid] : -1;
@@ -1021,7 +1159,8 @@ __device__ __forceinline__ void index_draft(const DraftParams& p, const IndexVie
                 }
             total = r;
         }
-        outputs(best.h, best.a, nstar, total, [&](int i, int64_t js) -> int32_t {
+        if (lane == 0) counts(nstar, total);
+        write_choice<HAS_H>(p, b, t, best.h, best.a, lane, [&](int i, int64_t js) -> int32_t {
             if (staged && i == lane) {
                 int32_t v = -1;
                 bool found = false;
@@ -1035,27 +1174,7 @@ __device__ __forceinline__ void index_draft(const DraftParams& p, const IndexVie
             }
             return RD::one(row + js + 1 + i);
         });
-        return;
     }
-
-    // ---- many candidates: a warp each, their keys combined over the CTA -----------------
-    best = score_by_warps<TH>(p, b, t, n, 0, 1, is.cand, kOccCap, cand_row, hsc, asc, sh.wnq);
-    unsigned long long hk = warp_max_u64(best.h), ak = warp_max_u64(best.a);
-    if (lane == 0) {
-        sh.wkey[0][warp] = hk;
-        sh.wkey[1][warp] = ak;
-    }
-    if (mine) index_put(ix, b, mytok, myslot, il + tid);          // the slot taken above
-    __syncthreads();
-    if (warp != 0) return;
-    hk = 0;
-    ak = 0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-        hk = sh.wkey[0][w] > hk ? sh.wkey[0][w] : hk;
-        ak = sh.wkey[1][w] > ak ? sh.wkey[1][w] : ak;
-    }
-    outputs(hk, ak, nstar, total, [&](int i, int64_t js) -> int32_t { return RD::one(row + js + 1 + i); });
 }
 
 template <typename TH, bool IVEC>
@@ -1165,9 +1284,10 @@ __global__ void index_finish_kernel(const int32_t* __restrict__ seq_len, int B, 
     if (bad_token && status) atomicOr(status + b, PLDP_ST_TOKEN_RANGE);
 }
 
-// Byte offsets of the index parts (ilen, flags, entries), 256-byte aligned.
+// Byte offsets of the index parts (ilen, flags, entries, the drafting calls' scratch),
+// 256-byte aligned.
 struct IndexLayout {
-    size_t ilen, flags, entries, total;
+    size_t ilen, flags, entries, defer, total;
 };
 inline IndexLayout index_layout(int B, int V) {
     auto up = [](size_t x) { return (x + 255) / 256 * 256; };
@@ -1175,34 +1295,55 @@ inline IndexLayout index_layout(int B, int V) {
     l.ilen = 0;
     l.flags = up(static_cast<size_t>(B) * 4);
     l.entries = l.flags + up(static_cast<size_t>(B) * 4);
-    l.total = l.entries + up(static_cast<size_t>(B) * V * kEntryWords * 4);
+    l.defer = l.entries + up(static_cast<size_t>(B) * V * kEntryWords * 4);
+    l.total = l.defer + up((static_cast<size_t>(B) + 1) * sizeof(DeferSlot));
     return l;
 }
 inline IndexView index_view(void* base, int B, int V) {
     const IndexLayout l = index_layout(B, V);
     char* c = static_cast<char*>(base);
-    return IndexView{reinterpret_cast<int32_t*>(c + l.ilen), reinterpret_cast<int32_t*>(c + l.flags),
-                     reinterpret_cast<int32_t*>(c + l.entries), V};
+    return IndexView{reinterpret_cast<DeferSlot*>(c + l.defer), reinterpret_cast<int32_t*>(c + l.ilen),
+                     reinterpret_cast<int32_t*>(c + l.flags), reinterpret_cast<int32_t*>(c + l.entries), V};
+}
+
+// Whether a drafting kernel that scores up to `here` candidates of a sequence by itself
+// may have to leave some: then its launch is followed by score_deferred_kernel's.
+inline bool may_defer(const DraftParams& p, int64_t here) { return p.C_cap > here && p.T_cap > here; }
+
+template <typename TH>
+pldp_status launch_deferred(const DraftParams& p, int B, cudaStream_t s, const char* what) {
+    int64_t blocks = resident_blocks(reinterpret_cast<const void*>(&score_deferred_kernel<TH>), kThreads, 0);
+    const int64_t most = p.C_cap < p.T_cap ? p.C_cap : p.T_cap;               // candidates of a sequence
+    const int64_t need = (most + kWarps - 1) / kWarps * B;                    // units of one per warp
+    if (blocks > need) blocks = need;
+    const cudaError_t e = launch_pdl(score_deferred_kernel<TH>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, s,
+                                     0, p, B);
+    if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "%s: launch failed: %s", what, cudaGetErrorString(e));
+    return PLDP_OK;
 }
 
 template <typename TH, bool IVEC>
-pldp_status launch_t(const DraftParams& p, int B, cudaStream_t s) {
+pldp_status launch_t(const DraftParams& p0, int B, cudaStream_t s) {
     int CL;
     int64_t chunk;
-    scan_shape(p.T_cap, B, resident_blocks(reinterpret_cast<const void*>(&draft_step_kernel<TH, IVEC>), kThreads, 0),
+    scan_shape(p0.T_cap, B, resident_blocks(reinterpret_cast<const void*>(&draft_step_kernel<TH, IVEC>), kThreads, 0),
                kPositionsPerCta, &CL, &chunk);
+    DraftParams p = p0;
+    if (!may_defer(p, static_cast<int64_t>(kCtaPasses) * kScoreBatch * CL)) p.defer = nullptr;
     const cudaError_t e = launch_pdl(draft_step_kernel<TH, IVEC>, dim3(static_cast<unsigned>(B) * CL), dim3(kThreads), 0,
                                      s, CL > 1 ? CL : 0, p, CL, chunk);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "draft_step: launch failed: %s", cudaGetErrorString(e));
-    return PLDP_OK;
+    return p.defer ? launch_deferred<TH>(p, B, s, "draft_step") : PLDP_OK;
 }
 
 template <typename TH, bool IVEC>
-pldp_status launch_index_t(const DraftParams& p, const IndexView& ix, int B, cudaStream_t s) {
+pldp_status launch_index_t(const DraftParams& p0, const IndexView& ix, int B, cudaStream_t s) {
+    DraftParams p = p0;
+    p.defer = may_defer(p, kCtaPasses * kMaxScoreBatch) ? ix.defer : nullptr;
     cudaError_t e = launch_pdl(draft_index_kernel<TH, IVEC>, dim3(static_cast<unsigned>(B)), dim3(kThreads), 0, s, 0,
                                p, ix);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "draft_step (indexed): launch failed: %s", cudaGetErrorString(e));
-    return PLDP_OK;
+    return p.defer ? launch_deferred<TH>(p, B, s, "draft_step (indexed)") : PLDP_OK;
 }
 
 template <typename TH>
@@ -1314,17 +1455,20 @@ pldp_status prepare_draft(const pldp_draft_step_args* a, const char* what, Draft
     p.draft = a->draft;
     p.draft_len = a->draft_len;
     p.status = a->status;
+    p.defer = has_ix ? nullptr : reinterpret_cast<DeferSlot*>(a->workspace);
     ivec = aligned16(a->ids) && a->ids_stride % 4 == 0 && a->T_cap % 4 == 0;
     return PLDP_OK;
 }
 
 template <typename TH, bool IVEC>
-pldp_status launch_verify_draft_t(const VerifyArgs& va, const DraftParams& p, const IndexView& ix, int B,
+pldp_status launch_verify_draft_t(const VerifyArgs& va, const DraftParams& p0, const IndexView& ix, int B,
                                   cudaStream_t s) {
+    DraftParams p = p0;
+    p.defer = may_defer(p, kCtaPasses * kMaxScoreBatch) ? ix.defer : nullptr;
     const cudaError_t e = launch_pdl(verify_draft_kernel<TH, IVEC>, dim3(static_cast<unsigned>(B)), dim3(kThreads), 0,
                                      s, 0, va, p, ix);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "verify_draft: launch failed: %s", cudaGetErrorString(e));
-    return PLDP_OK;
+    return p.defer ? launch_deferred<TH>(p, B, s, "verify_draft") : PLDP_OK;
 }
 
 template <typename TH>

@@ -56,7 +56,9 @@ def test_find_candidates_edges(lib, T, V, B):
 @pytest.mark.parametrize("T,V,B,d,R,agg,dtype", [
     (9000, 1, 3, 64, 20, 0, torch.bfloat16), (9000, 2, 150, 64, 8, 1, torch.bfloat16),
     (6000, 12, 4, 4096, 300, 1, torch.float32), (6001, 12, 4, 4104, 300, 1, torch.bfloat16),
-    (700, 6, 5, 1000, 600, 0, torch.float32)])
+    (700, 6, 5, 1000, 600, 0, torch.float32),
+    # around what a CTA scores by itself (8 or 4 a CTA), and more sequences than a tile of the deferred launch
+    (90, 10, 40, 64, 8, 0, torch.bfloat16), (200, 7, 700, 64, 8, 1, torch.bfloat16)])
 @pytest.mark.parametrize("ngram", [(1, 1), (1, 3)])
 def test_many_candidates(lib, T, V, B, d, R, agg, dtype, ngram):
     K, C = 6, 1100
@@ -75,6 +77,7 @@ def test_many_candidates(lib, T, V, B, d, R, agg, dtype, ngram):
                            best_h_score=buf.bscore_h, A=A, best_a=buf.best_a, agg=agg, a_scores=buf.scores_a,
                            best_a_score=buf.bscore_a, status=buf.status, index=ix, V=V)
         out.append(snapshot(buf))
+        assert not buf.dws.any()                       # the scratch is left zeroed
         _compare(out[-1], ids, lens, H, A, None, agg, ngram, C, K, "hidden")
     for k in ("cand", "scores_h", "scores_a", "best_h", "best_a", "draft"):
         assert np.array_equal(out[0][k], out[1][k], equal_nan=True), k
