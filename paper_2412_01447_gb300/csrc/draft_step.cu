@@ -50,8 +50,7 @@ constexpr int64_t kPositionsPerCta = 1024;                     // scanned by a C
 constexpr int kScanLoads = 8;                                  // vectors of ids in flight per lane (scan kernel)
 constexpr int kListPerWarp = 128;                              // positions listed per warp (scan kernel)
 constexpr int kList = kListPerWarp * kWarps;                   // ... and per CTA
-constexpr int kRescanLoads = 16;                               // the same for the rescan of the indexed kernels
-constexpr int kRescanPerWarp = 128;
+constexpr int kRescanPerWarp = 128;                            // the same for the rescan of the indexed kernels
 constexpr int kScoreUnroll = 2;                                // 16-byte row loads in flight
 constexpr int kScoreBatch = 2;                                 // candidates scored by the whole CTA at once (scan kernel)
 constexpr int kMaxScoreBatch = 4;                              // ... and at most (the indexed kernel)
@@ -639,7 +638,7 @@ __device__ __noinline__ void rescan(const DraftParams& p, int64_t t, const int32
     const int64_t s0 = warp * seg;
     const int nit = static_cast<int>(seg / kScanTile);
     {
-        WarpScan<IVEC, RD, kRescanLoads> sc;
+        WarpScan<IVEC, RD, kScanLoads, true> sc;
         sc.begin(row, s0, nit, p.T_cap, lane);
         __syncthreads();                                          // the suffix is in
         scan_lists(sc, t, p.ngram_max, warp, sl);

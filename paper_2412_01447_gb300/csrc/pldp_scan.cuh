@@ -2,22 +2,24 @@
 // as device building blocks shared by pldp_find_candidates and the drafting calls.
 //
 // A CTA owns a contiguous chunk of one context and each of its warps a contiguous
-// segment of the chunk, 128 positions an iteration (a 16-byte vector per lane).  The
-// tokens before a vector's are in the lanes below it, so the suffix-match lengths of
-// all 128 positions come from shuffles and compares, without another load and
-// without a loop over the matches.  A warp keeps only the positions with the longest
-// match it has met so far, in ascending order, in a short list in shared memory: a
-// shorter match can no longer be a candidate.  One pass over the ids is thus enough,
-// however often x_t occurs (text repeats its frequent tokens thousands of times in a
-// long context); a list that overflows is written by a second pass over its segment.
+// segment of the chunk, 1024 positions a round: eight 16-byte vectors per lane, a bit
+// per position in a lane's mask.  The positions equal to x_{t-k} are a mask of 32
+// compares; moved up by k positions (shifts inside a lane, one or two shuffles for what
+// crosses lanes) it says where the k-th token of the suffix matches, so the longest
+// match of the round is a chain of ANDs, whatever the number of matches.  A warp keeps
+// only the positions with the longest match it has met so far, in ascending order, in a
+// short list in shared memory: a shorter match can no longer be a candidate.  One pass
+// over the ids is thus enough, however often x_t occurs (text repeats its frequent
+// tokens thousands of times in a long context); a list that overflows is written by a
+// second pass over its segment.
 //
-// What bounds it: the ids' DRAM round trips (8 vectors in flight per lane) and, for a
-// frequent x_t, about 60 instructions per iteration that meets one.  Before, every
-// occurrence walked its suffix with one dependent load per token and the positions
-// were written by a second pass with two CTA barriers per 1024 positions: on 32k-token
-// Zipf contexts (batch 128) the drafting launch took 1240-1490 us and now 125-190 us,
-// what is left being the scores of its hundreds of candidates; pldp_find_candidates on
-// 16k-token contexts (batch 64, L2 flushed) went from 12.2 to 8.2 us.
+// What bounds it: the ids' DRAM round trips (8 vectors in flight per lane).  Match
+// lengths worked out per position cost 150 instructions per 128 positions wherever x_t
+// is frequent (drafting batch 128 x 32k Zipf tokens through the index: 34 us, 21 us with
+// masks; its scanning kernel 22 -> 17 us); before that, every occurrence walked its suffix with one dependent load
+// per token and the positions were written by a second pass with two CTA barriers per
+// 1024 positions, which took most of 1240-1490 us of a drafting launch over 32k-token
+// Zipf contexts (batch 128).  pldp_find_candidates, batch 64 x 16k, L2 flushed: 12.2 -> 8-9.6 us.
 #pragma once
 
 #include "pldp_internal.cuh"
@@ -59,83 +61,51 @@ __device__ __forceinline__ int4 scan_load(const int32_t* __restrict__ row, int64
     return v;
 }
 
-// The vector `back` (1 or 2) places before each lane's: from the lanes below, and for
-// the first lanes from the last lanes of the warp's previous vectors (vp).
-__device__ __forceinline__ int4 scan_before(const int4& v, const int4& vp, int back, int lane) {
-    const bool hi = lane >= 32 - back;
-    const int src = (lane + 32 - back) & 31;
-    int4 r;
-    r.x = __shfl_sync(0xFFFFFFFFu, hi ? vp.x : v.x, src);
-    r.y = __shfl_sync(0xFFFFFFFFu, hi ? vp.y : v.y, src);
-    r.z = __shfl_sync(0xFFFFFFFFu, hi ? vp.z : v.z, src);
-    r.w = __shfl_sync(0xFFFFFFFFu, hi ? vp.w : v.w, src);
-    return r;
-}
-
-// Suffix-match lengths of the lane's four positions p .. p + 3 (those below `lim`;
-// 0 where the token is not x_t), capped at n_max and at the tokens there are.
-// suf = x_t, x_{t-1}, ...
-__device__ __forceinline__ void scan_match(const int4& v, const int4& vp, int64_t p, int64_t lim,
-                                           const int32_t* suf, int n_max, int lane, int (&m)[4]) {
-    const int32_t xt = suf[0];
-    bool ok[4] = {v.x == xt && p < lim, v.y == xt && p + 1 < lim, v.z == xt && p + 2 < lim, v.w == xt && p + 3 < lim};
+// Where a lane's vectors hold token s: bit 4 u + c for component c of vector u.
+template <int U>
+__device__ __forceinline__ uint32_t scan_equal(const int4 (&v)[U], int32_t s) {
+    static_assert(U <= 8, "a bit per position");
+    uint32_t m = 0;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) m[c] = ok[c] ? 1 : 0;
-    if (n_max > 1) {                                          // the tokens at p - 8 .. p + 3
-        const int4 b1 = scan_before(v, vp, 1, lane);
-        int32_t w[12] = {0, 0, 0, 0, b1.x, b1.y, b1.z, b1.w, v.x, v.y, v.z, v.w};
-        if (n_max > 5) {
-            const int4 b2 = scan_before(v, vp, 2, lane);
-            w[0] = b2.x;
-            w[1] = b2.y;
-            w[2] = b2.z;
-            w[3] = b2.w;
-        }
-#pragma unroll
-        for (int k = 1; k < PLDP_MAX_NGRAM; ++k) {
-            if (k >= n_max) break;
-            const int32_t s = suf[k];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                ok[c] = ok[c] && p + c >= k && w[8 + c - k] == s;
-                m[c] += ok[c] ? 1 : 0;
-            }
-        }
+    for (int u = 0; u < U; ++u) {
+        m |= v[u].x == s ? 1u << (4 * u) : 0u;
+        m |= v[u].y == s ? 2u << (4 * u) : 0u;
+        m |= v[u].z == s ? 4u << (4 * u) : 0u;
+        m |= v[u].w == s ? 8u << (4 * u) : 0u;
     }
+    return m;
 }
 
-// Calls put(index, position) for the lane's positions with m == level, index counting
-// the warp's from `base` in ascending position order; returns how many the warp has.
-template <typename Put>
-__device__ __forceinline__ int scan_put(const int (&m)[4], int level, int64_t p, int base, int lane, Put put) {
-    const unsigned lt = (1u << lane) - 1u;
-    int off = base, n = 0;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const unsigned bal = __ballot_sync(0xFFFFFFFFu, m[c] == level);
-        off += __popc(bal & lt);
-        n += __popc(bal);
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-        if (m[c] == level) put(off++, p + c);
-    return n;
+// The mask f moved up by k positions (1 <= k < 8): a bit stays in its lane or comes from
+// one of the two lanes below; the first lanes take theirs from the vector before, in the
+// last lanes (before a round's first vectors: fp, the mask of lanes 30 and 31 there).
+__device__ __forceinline__ uint32_t scan_move(uint32_t f, uint32_t fp, int k, int lane) {
+    const int a = k >> 2, r = k & 3;
+    auto below = [&](int d) -> uint32_t {
+        return __shfl_sync(0xFFFFFFFFu, lane >= 32 - d ? (f << 4) | fp : f, (lane + 32 - d) & 31);
+    };
+    const uint32_t near = a ? below(1) : f;
+    if (r == 0) return near;
+    const uint32_t far = below(a + 1);
+    const uint32_t keep = 0x11111111u * ((0xFu << r) & 0xFu);    // components that stay in their lane
+    return ((near << r) & keep) | ((far >> (4 - r)) & ~keep);
 }
 
-// One warp's scan of positions [s0, s0 + nit * kScanTile), those below `lim`, U vectors
-// in flight per lane.  begin() issues the first loads (ids up to `cap` may be read), so
-// that they can be under way before the suffix and the context length are known.
-template <bool VEC, typename RD, int U>
+// One warp's scan of positions [s0, s0 + nit * kScanTile), those below a limit, U
+// vectors in flight per lane (AHEAD: the next U too, while these are worked on).
+// begin() issues the first loads (ids up to `cap` may be read), so that they can be
+// under way before the suffix and the context length are known.
+template <bool VEC, typename RD, int U, bool AHEAD = false>
 struct WarpScan {
     const int32_t* row;
     int64_t q0, cap;                     // the lane's first vector; readable positions
     int nit, lane;
     int4 v[U], vp;
 
-    __device__ __forceinline__ void load(int it0) {
+    __device__ __forceinline__ void load(int4 (&x)[U], int it0) const {
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (it0 + u < nit) v[u] = scan_load<VEC, RD>(row, q0 + static_cast<int64_t>(it0 + u) * 32, cap);
+            if (it0 + u < nit) x[u] = scan_load<VEC, RD>(row, q0 + static_cast<int64_t>(it0 + u) * 32, cap);
     }
     __device__ __forceinline__ void begin(const int32_t* r, int64_t s0, int iters, int64_t cap_, int lane_) {
         row = r;
@@ -145,40 +115,85 @@ struct WarpScan {
         q0 = (s0 >> 2) + lane;
         vp = make_int4(0, 0, 0, 0);      // lanes 30, 31: the vectors before the segment
         if (lane >= 30 && nit > 0) vp = scan_load<VEC, RD>(row, q0 - 32, cap);
-        load(0);
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = make_int4(0, 0, 0, 0);
+        load(v, 0);
     }
-    // each(m, p): the match lengths of a tile with at least one occurrence of x_t.  One
-    // copy of the tile's code walks the vectors by shifting them down (after an L2 flush
-    // the kernel's code comes from DRAM: unrolled over the vectors, it cost a
-    // drafting call 2-6 us of instruction fetch); tiles without x_t skip it.
+    // each(m, mask, p) for every round with an occurrence of x_t = suf[0]: its longest
+    // suffix match m (at most n_max) and the positions that have it, bit 4 u + c of a
+    // lane's mask standing for p + u * kScanTile + c.
     template <typename Each>
     __device__ __forceinline__ void run(int64_t lim, const int32_t* suf, int n_max, Each each) {
         const int32_t xt = suf[0];
 #pragma unroll 1
-        for (int it0 = 0; it0 < nit && 4 * (q0 - lane) + static_cast<int64_t>(it0) * kScanTile < lim; it0 += U) {
-            if (it0 > 0) load(it0);
-            unsigned tiles = 0;                               // bit u: this lane has x_t in vector u
+        for (int it0 = 0; it0 < nit; it0 += U) {
+            const int64_t p = 4 * (q0 + static_cast<int64_t>(it0) * 32);      // the lane's first position
+            if (p - 4 * lane >= lim) break;                                   // warp-uniform
+            int4 nx[AHEAD ? U : 1];
+            if constexpr (AHEAD) {
 #pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (it0 + u < nit && (v[u].x == xt || v[u].y == xt || v[u].z == xt || v[u].w == xt)) tiles |= 1u << u;
-            tiles = __reduce_or_sync(0xFFFFFFFFu, tiles);     // bit u: the warp has
-            const int4 last = v[U - 1];
-            int64_t p = 4 * (q0 + static_cast<int64_t>(it0) * 32);
-#pragma unroll 1
-            for (; tiles != 0; tiles >>= 1, p += kScanTile) {
-                if (tiles & 1u) {
-                    int m[4];
-                    scan_match(v[0], vp, p, lim, suf, n_max, lane, m);
-                    each(m, p);
-                }
-                vp = v[0];
-#pragma unroll
-                for (int k = 0; k + 1 < U; ++k) v[k] = v[k + 1];
+                for (int u = 0; u < U; ++u) nx[u] = make_int4(0, 0, 0, 0);
+                load(nx, it0 + U);
+            } else if (it0 > 0) {
+                load(v, it0);
             }
-            vp = last;
+            uint32_t mask = scan_equal<U>(v, xt);
+            if (it0 + U > nit) mask &= (1u << (4 * (nit - it0))) - 1u;
+            if (p - 4 * lane + static_cast<int64_t>(U) * kScanTile > lim) {   // the context ends in this round
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int64_t left = lim - (p + u * kScanTile);
+                    if (left < 4) mask &= ~((0xFu << (left > 0 ? static_cast<int>(left) : 0) & 0xFu) << (4 * u));
+                }
+            }
+            if (__any_sync(0xFFFFFFFFu, mask != 0)) {
+                int m = 1;
+#pragma unroll 1
+                for (; m < n_max; ++m) {                                      // mask: matches of m tokens
+                    const int32_t sk = suf[m];
+                    const int4 before[1] = {vp};
+                    uint32_t f = scan_move(scan_equal<U>(v, sk), scan_equal<1>(before, sk), m, lane);
+                    if (p < m) f &= ~0u << (m - p < 4 ? static_cast<int>(m - p) : 4);   // no token there
+                    f &= mask;
+                    if (!__any_sync(0xFFFFFFFFu, f != 0)) break;
+                    mask = f;
+                }
+                each(m, mask, p);
+            }
+            vp = v[U - 1];
+            if constexpr (AHEAD) {
+#pragma unroll
+                for (int u = 0; u < U; ++u) v[u] = nx[u];
+            }
         }
     }
 };
+
+// put(i, j) for the i-th of the warp's positions in a round's mask (see WarpScan::run),
+// counting from `base` in ascending order; returns how many there are.
+template <typename Put>
+__device__ __forceinline__ int scan_put(uint32_t mask, int64_t p, int base, int lane, Put put) {
+    const unsigned lt = (1u << lane) - 1u;
+    uint32_t tiles = (mask | mask >> 1 | mask >> 2 | mask >> 3) & 0x11111111u;
+    tiles = __reduce_or_sync(0xFFFFFFFFu, tiles);
+    int n = 0;
+#pragma unroll 1
+    for (; tiles != 0; tiles &= tiles - 1u) {
+        const int at = __ffs(tiles) - 1;                          // 4 u
+        const uint32_t nib = mask >> at;
+        int off = base + n;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const unsigned bal = __ballot_sync(0xFFFFFFFFu, (nib >> c) & 1u);
+            off += __popc(bal & lt);
+            n += __popc(bal);
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if ((nib >> c) & 1u) put(off++, p + (at >> 2) * kScanTile + c);
+    }
+    return n;
+}
 
 // What a CTA found: per warp the longest match length and how many positions have it,
 // the first LW of them listed in ascending order.
@@ -193,14 +208,13 @@ struct ScanLists {
 template <typename Scan, int LW>
 __device__ __forceinline__ void scan_lists(Scan& sc, int64_t lim, int n_max, int warp, ScanLists<LW>& sl) {
     int wm = 0, wc = 0;
-    sc.run(lim, sl.suf, n_max, [&](const int (&m)[4], int64_t p) {
-        const int mx = __reduce_max_sync(0xFFFFFFFFu, max(max(m[0], m[1]), max(m[2], m[3])));
-        if (mx < wm) return;                                  // warp-uniform
-        if (mx > wm) {
-            wm = mx;
+    sc.run(lim, sl.suf, n_max, [&](int m, uint32_t mask, int64_t p) {
+        if (m < wm) return;                                       // warp-uniform
+        if (m > wm) {
+            wm = m;
             wc = 0;
         }
-        wc += scan_put(m, wm, p, wc, sc.lane, [&](int i, int64_t j) {
+        wc += scan_put(mask, p, wc, sc.lane, [&](int i, int64_t j) {
             if (i < LW) sl.pos[warp][i] = static_cast<int32_t>(j);
         });
     });
@@ -241,9 +255,10 @@ __device__ __noinline__ void scan_again(const int32_t* __restrict__ row, int64_t
                                         Put put) {
     WarpScan<VEC, RD, 8> sc;
     sc.begin(row, s0, nit, cap, lane);
-    sc.run(lim, suf, n_max, [&](const int (&m)[4], int64_t p) {
+    sc.run(lim, suf, n_max, [&](int m, uint32_t mask, int64_t p) {
+        if (m != level) return;
         const int64_t base = at;
-        at += scan_put(m, level, p, 0, lane, [&](int i, int64_t j) {
+        at += scan_put(mask, p, 0, lane, [&](int i, int64_t j) {
             if (base + i < C_cap) put(base + i, static_cast<int32_t>(j));
         });
     });
