@@ -51,6 +51,7 @@ constexpr int kScanLoads = 8;                                  // vectors of ids
 constexpr int kListPerWarp = 128;                              // positions listed per warp (scan kernel)
 constexpr int kList = kListPerWarp * kWarps;                   // ... and per CTA
 constexpr int kRescanPerWarp = 128;                            // the same for the rescan of the indexed kernels
+constexpr int kRescanRounds = 5;                               // rounds of 1024 positions a warp keeps masks of there
 constexpr int kScoreUnroll = 2;                                // 16-byte row loads in flight
 constexpr int kScoreBatch = 2;                                 // candidates scored by the whole CTA at once (scan kernel)
 constexpr int kMaxScoreBatch = 4;                              // ... and at most (the indexed kernel)
@@ -625,33 +626,92 @@ __global__ void __launch_bounds__(kThreads, 2) score_deferred_kernel(const Draft
     if (tid == 0) slots[B].done = 0;
 }
 
+// What the rescan keeps per warp: every round's longest match and its mask (see
+// WarpScan::run) for the first kRescanRounds rounds of 1024 positions, i.e. contexts of
+// up to 40k tokens; of a longer context a list of positions.
+union RescanShared {
+    struct {
+        uint32_t mask[kScanWarps][kRescanRounds][32];
+        int32_t suf[PLDP_MAX_NGRAM];
+        int wm[kScanWarps], wc[kScanWarps];
+        uint8_t level[kScanWarps][kRescanRounds];
+    };
+    ScanLists<kRescanPerWarp> sl;
+};
+
 // The candidates of a sequence whose occurrences were not gathered (a token the index
 // cannot answer for): one CTA scans the context and writes the candidate list, its first
-// `keep` entries to `first` (shared) too.  Kept out of line: its registers do not weigh
-// on the common path.  CTA-uniform call, a barrier at the end.
+// `keep` entries to `first` (shared) too.  With the rounds' masks kept, the list is
+// written without reading the ids again, however long it is (a token that makes up 8 % of
+// 32k tokens overflowed a warp's list of 128, and its second pass took 18 us: index build
+// and 8 fused steps of batch 128 x 32k 1252 -> 1142 us).  Kept out of line: its registers
+// do not weigh on the common path.  CTA-uniform call, a barrier at the end.
 template <bool IVEC, typename RD>
 __device__ __noinline__ void rescan(const DraftParams& p, int64_t t, const int32_t* row, int32_t* cand_row,
-                                    ScanLists<kRescanPerWarp>& sl, int32_t* first, int keep, int& nstar, int& total) {
+                                    RescanShared& rs, int32_t* first, int keep, int& nstar, int& total) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid < PLDP_MAX_NGRAM) sl.suf[tid] = (tid < p.ngram_max && t - tid >= 0) ? RD::one(row + t - tid) : 0;
     const int64_t seg = (t + kScanChunkUnit - 1) / kScanChunkUnit * kScanTile;      // positions per warp
     const int64_t s0 = warp * seg;
     const int nit = static_cast<int>(seg / kScanTile);
-    {
-        WarpScan<IVEC, RD, kScanLoads, true> sc;
-        sc.begin(row, s0, nit, p.T_cap, lane);
+    if (IVEC && lane == 0 && s0 < t)                              // the warp's ids head for L2 all at once
+        prefetch_l2_bulk(row + s0, static_cast<uint32_t>((s0 + seg < t ? seg : (t - s0 + 3) & ~int64_t(3)) * 4));
+    WarpScan<IVEC, RD, kScanLoads, true> sc;
+    sc.begin(row, s0, nit, p.T_cap, lane);
+    auto put = [&](int64_t i, int32_t j) {
+        cand_row[i] = j;
+        if (i < keep) first[i] = j;
+    };
+    if (nit <= kRescanRounds * kScanLoads) {
+        if (tid < PLDP_MAX_NGRAM) rs.suf[tid] = (tid < p.ngram_max && t - tid >= 0) ? RD::one(row + t - tid) : 0;
+        if (lane < kRescanRounds) rs.level[warp][lane] = 0;
+        __syncthreads();                                          // the suffix is in
+        int wm = 0, wc = 0;                                       // wc: this lane's
+        sc.run(t, rs.suf, p.ngram_max, [&](int m, uint32_t mask, int64_t q) {
+            if (m < wm) return;                                   // warp-uniform
+            if (m > wm) wc = 0;
+            wm = m;
+            wc += __popc(mask);
+            const int r = static_cast<int>((q - 4 * lane - s0) / (kScanTile * kScanLoads));
+            rs.mask[warp][r][lane] = mask;
+            if (lane == 0) rs.level[warp][r] = static_cast<uint8_t>(m);
+        });
+        wc = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(wc)));
+        if (lane == 0) {
+            rs.wm[warp] = wm;
+            rs.wc[warp] = wc;
+        }
+        __syncthreads();
+        int best = 0, cnt = 0, at = 0;
+#pragma unroll
+        for (int w = 0; w < kScanWarps; ++w) best = max(best, rs.wm[w]);
+#pragma unroll
+        for (int w = 0; w < kScanWarps; ++w) {
+            const int c = rs.wm[w] == best ? rs.wc[w] : 0;
+            at += w < warp ? c : 0;
+            cnt += c;
+        }
+        nstar = best >= p.ngram_min ? best : 0;
+        total = nstar > 0 ? cnt : 0;
+        if (nstar > 0 && wm == nstar)
+            for (int r = 0; r * kScanLoads < nit && at < p.C_cap; ++r) {
+                if (rs.level[warp][r] != nstar) continue;
+                const int base = at;
+                at += scan_put(rs.mask[warp][r][lane], s0 + r * (kScanTile * kScanLoads) + 4 * lane, 0, lane,
+                               [&](int i, int64_t j) {
+                                   if (base + i < p.C_cap) put(base + i, static_cast<int32_t>(j));
+                               });
+            }
+    } else {
+        ScanLists<kRescanPerWarp>& sl = rs.sl;
+        if (tid < PLDP_MAX_NGRAM) sl.suf[tid] = (tid < p.ngram_max && t - tid >= 0) ? RD::one(row + t - tid) : 0;
         __syncthreads();                                          // the suffix is in
         scan_lists(sc, t, p.ngram_max, warp, sl);
+        __syncthreads();
+        const CtaMatches cm = cta_matches(sl, warp);
+        nstar = cm.m >= p.ngram_min ? cm.m : 0;
+        total = nstar > 0 ? cm.cnt : 0;
+        scan_emit<IVEC, RD>(row, s0, nit, t, p.T_cap, p.ngram_max, nstar, cm.base, p.C_cap, warp, lane, sl, put);
     }
-    __syncthreads();
-    const CtaMatches cm = cta_matches(sl, warp);
-    nstar = cm.m >= p.ngram_min ? cm.m : 0;
-    total = nstar > 0 ? cm.cnt : 0;
-    scan_emit<IVEC, RD>(row, s0, nit, t, p.T_cap, p.ngram_max, nstar, cm.base, p.C_cap, warp, lane, sl,
-                        [&](int64_t i, int32_t j) {
-                            cand_row[i] = j;
-                            if (i < keep) first[i] = j;
-                        });
     __syncthreads();
 }
 
@@ -878,7 +938,7 @@ struct IndexShared {
             int32_t occ_m[kOccCap];        // their suffix-match lengths
             int32_t occ_new[kNewCap];      // the appended occurrences, ascending
         };
-        ScanLists<kRescanPerWarp> sl;      // the rescan, which has no occurrences at hand
+        RescanShared rs;                   // the rescan, which has no occurrences at hand
     };
     int32_t cand[kOccCap];             // the candidates (match length >= n*), ascending
     int32_t newtok[kNewCap];           // ids of positions il .. t-1
@@ -1082,7 +1142,7 @@ __device__ __forceinline__ void index_draft(const DraftParams& p, const IndexVie
         nstar = is.nstar;
         total = is.ncand;
     } else if (!indexed) {
-        rescan<IVEC, RD>(p, t, row, cand_row, is.sl, is.cand, kOccCap, nstar, total);
+        rescan<IVEC, RD>(p, t, row, cand_row, is.rs, is.cand, kOccCap, nstar, total);
     }
 
     const int n = spec ? nocc : (total < p.C_cap ? total : p.C_cap);

@@ -57,6 +57,9 @@ def test_find_candidates_edges(lib, T, V, B):
     (9000, 1, 3, 64, 20, 0, torch.bfloat16), (9000, 2, 150, 64, 8, 1, torch.bfloat16),
     (6000, 12, 4, 4096, 300, 1, torch.float32), (6001, 12, 4, 4104, 300, 1, torch.bfloat16),
     (700, 6, 5, 1000, 600, 0, torch.float32),
+    # the rescan's masks at their last context length, and the lists beyond it
+    (40960, 3, 3, 64, 8, 0, torch.bfloat16), (42001, 3, 3, 64, 8, 0, torch.bfloat16),
+    (50000, 400, 3, 64, 8, 1, torch.bfloat16),
     # around what a CTA scores by itself (8 or 4 a CTA), and more sequences than a tile of the deferred launch
     (90, 10, 40, 64, 8, 0, torch.bfloat16), (200, 7, 700, 64, 8, 1, torch.bfloat16)])
 @pytest.mark.parametrize("ngram", [(1, 1), (1, 3)])
