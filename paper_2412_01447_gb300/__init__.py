@@ -20,6 +20,9 @@ with the token index of ``pldp_index_build``), ``pldp_verify_greedy_draft`` and
 step's draft).  Also ``pldp_rank_hidden_avg``
 (App. B.2) and ``pldp_identify_heads`` / ``pldp_top_heads`` (Sec. 4.2.1).
 
+The marshalling of the calls a decode step makes is native as well
+(``csrc/host_calls.cpp``), with the Python below as its wording of errors.
+
 Device buffers are passed as raw pointers, so the binding checks what the C
 side cannot: every tensor is a CUDA tensor of the stated dtype, dense where
 the call wants it, and holds at least the elements the call will touch.
@@ -27,6 +30,7 @@ the call wants it, and holds at least the elements the call will touch.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 import threading
 
@@ -79,6 +83,7 @@ class PldpError(RuntimeError):
 
 _lock = threading.Lock()
 _lib = None
+_calls = None            # the native checks and marshalling (csrc/host_calls.cpp), once loaded
 
 
 class pldp_draft_step_args(ctypes.Structure):
@@ -133,8 +138,28 @@ def build(force: bool = False) -> str:
     return _build.build(force=force)
 
 
+# The entry points _calls makes, in the order of its `Library`.
+_CALLS = ("pldp_find_candidates", "pldp_rank_hidden", "pldp_rank_attention", "pldp_extract_draft", "pldp_draft_step",
+          "pldp_index_build", "pldp_verify_greedy", "pldp_verify_greedy_draft", "pldp_verify_sample",
+          "pldp_verify_sample_draft", "pldp_identify_heads", "pldp_top_heads")
+
+
+def _load_calls(lib):
+    """The native form of the calls below, bound to the loaded library.  Each takes a
+    call's arguments, makes its checks and returns the library's status, or None when a
+    check does not pass or an argument is of a kind it does not handle; the Python that
+    follows then does the same and words the error."""
+    if not os.path.exists(_build.CALLS):
+        return None
+    spec = importlib.util.spec_from_file_location("_pldp_calls", _build.CALLS)
+    m = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(m)
+    m.bind(tuple(ctypes.cast(getattr(lib, f), ctypes.c_void_p).value for f in _CALLS))
+    return m
+
+
 def _load():
-    global _lib
+    global _lib, _calls
     if _lib is not None:
         return _lib
     with _lock:
@@ -191,6 +216,7 @@ def _load():
             lib.pldp_last_error.restype = ctypes.c_char_p
             lib.pldp_version.argtypes = []
             lib.pldp_version.restype = ctypes.c_int
+            _calls = _load_calls(lib)
             _lib = lib
     return _lib
 
@@ -268,6 +294,13 @@ def _code(x):
     raise ValueError(f"unsupported dtype {x}")
 
 
+def _done(fn, rc):
+    """Whether a native call was made (rc is not None); raises when it failed."""
+    if rc:
+        _check(fn, rc)
+    return rc is not None
+
+
 def _check(fn, rc):
     if rc != 0:
         raise PldpError(fn, rc, _load().pldp_last_error().decode())
@@ -281,6 +314,9 @@ def pldp_find_candidates(ids, seq_len, ngram_min, ngram_max, cand_pos, cand_coun
     """Eq. 1 with the longest-suffix n-gram rule.  ids: int32 [B, T] (rows may be
     strided), seq_len int32 [B]; outputs cand_pos int32 [B, C_cap], cand_count and
     match_len int32 [B], status uint32-as-int32 [B] (optional)."""
+    if _calls is not None and _done("pldp_find_candidates", _calls.find_candidates(
+            ids, seq_len, ngram_min, ngram_max, cand_pos, cand_count, match_len, status, T_cap, stream)):
+        return
     p_ids, stride, T = _rows(ids, "ids", T_cap=T_cap)
     B = ids.shape[0]
     C_cap = cand_pos.shape[1] if cand_pos is not None and cand_pos.dim() == 2 else 0
@@ -296,6 +332,9 @@ def pldp_rank_hidden(H, seq_len, cand_pos, cand_count, best_pos, scores=None, be
     """Eq. 3.  H: [B, T_cap, d] float32/bfloat16 (the chosen layer), contiguous rows;
     cand_pos int32 [B, C_cap]; outputs best_pos int32 [B], scores float32 [B, C_cap]
     and best_score float32 [B] (optional)."""
+    if _calls is not None and _done("pldp_rank_hidden", _calls.rank_hidden(
+            H, seq_len, cand_pos, cand_count, best_pos, scores, best_score, threshold, status, stream)):
+        return
     if H.dim() != 3 or H.stride(2) != 1 or H.stride(1) != H.shape[2]:
         raise ValueError("H must be [B, T_cap, d] with contiguous rows")
     B, T_cap, d = H.shape
@@ -331,6 +370,9 @@ def pldp_identify_heads(ids, pos, A, counts, max_suffix=64, r_star=None, status=
     generated token's position p); A [B, R, T_cap] float32/bfloat16, the attention
     rows of query p-1 (unit inner stride); counts int32/uint32 [R] CUDA tensor,
     added to.  r_star int32 [B] out (optional)."""
+    if _calls is not None and _done("pldp_identify_heads", _calls.identify_heads(
+            ids, pos, A, counts, max_suffix, r_star, status, stream)):
+        return
     if A.dim() != 3 or A.stride(2) != 1:
         raise ValueError("A must be [B, R, T_cap] with unit inner stride")
     B, R = A.shape[0], A.shape[1]
@@ -346,6 +388,8 @@ def pldp_identify_heads(ids, pos, A, counts, max_suffix=64, r_star=None, status=
 
 def pldp_top_heads(counts, k, row_idx, stream=None):
     """The k rows with the most counts (ties to the smaller index) into row_idx int32 [k]."""
+    if _calls is not None and _done("pldp_top_heads", _calls.top_heads(counts, k, row_idx, stream)):
+        return
     _check("pldp_top_heads", _load().pldp_top_heads(_dense(counts, "counts", _WORD), counts.numel(), int(k),
                                                     _dense(row_idx, "row_idx", torch.int32, n=int(k)),
                                                     _stream(stream)))
@@ -358,6 +402,9 @@ def pldp_rank_attention(A, seq_len, cand_pos, cand_count, best_pos, row_idx=None
     of a key dense: e.g. a [B, T_cap, R] tensor transposed to [B, R, T_cap]), on the
     device or in pinned host memory (read in place: only the selected rows' values at the
     candidate keys cross the link); row_idx int32 [n_sel] device or None (all)."""
+    if _calls is not None and _done("pldp_rank_attention", _calls.rank_attention(
+            A, seq_len, cand_pos, cand_count, best_pos, row_idx, agg, scores, best_score, status, stream)):
+        return
     if A.dim() != 3:
         raise ValueError("A must be [B, R, T_cap]")
     B, R, T_cap = A.shape
@@ -376,6 +423,8 @@ def pldp_rank_attention(A, seq_len, cand_pos, cand_count, best_pos, row_idx=None
 
 def pldp_extract_draft(ids, seq_len, best_pos, draft, draft_len, T_cap=None, stream=None):
     """Sec. 4.3.  draft int32 [B, K] and draft_len int32 [B] are written."""
+    if _calls is not None and _done("pldp_extract_draft", _calls.extract_draft(ids, seq_len, best_pos, draft, draft_len, T_cap, stream)):
+        return
     B, K = draft.shape
     p_ids, stride, T = _rows(ids, "ids", B, T_cap)
     _check("pldp_extract_draft", _load().pldp_extract_draft(
@@ -454,6 +503,9 @@ def pldp_draft_step(ids, seq_len, ngram_min, ngram_max, cand_pos, cand_count, ma
     up instead of scanning, with the same results.  Keyword arguments: H, best_h,
     h_scores, best_h_score, threshold, A, best_a, row_idx, agg, a_scores,
     best_a_score, draft_from, status, T_cap, index, V."""
+    if _calls is not None and _done("pldp_draft_step", _calls.draft_step(
+            ids, seq_len, ngram_min, ngram_max, cand_pos, cand_count, match_len, K, draft, draft_len, workspace, stream, kw)):
+        return
     a = _draft_args(ids, seq_len, ngram_min, ngram_max, cand_pos, cand_count, match_len, K, draft,
                     draft_len, workspace, **kw)
     _check("pldp_draft_step", _load().pldp_draft_step(ctypes.byref(a), _stream(stream)))
@@ -467,6 +519,10 @@ def pldp_verify_greedy_draft(logits, draft, draft_len, accept_len, next_token, w
     pldp_draft_step on the extended context), in one call.  next_draft /
     next_draft_len receive the next draft (they may be draft / draft_len).  Keyword
     arguments are pldp_draft_step's (H, best_h, A, best_a, status, ...)."""
+    if _calls is not None and _done("pldp_verify_greedy_draft", _calls.verify_greedy_draft(
+            logits, draft, draft_len, accept_len, next_token, workspace, ids, seq_len, ngram_min, ngram_max, cand_pos,
+            cand_count, match_len, next_draft, next_draft_len, index, argmax, kv_keep_len, stream, kw)):
+        return
     B, K1, V = logits.shape
     K = K1 - 1
     if draft.shape != (B, K) or next_draft.shape != (B, K):
@@ -501,6 +557,11 @@ def pldp_verify_sample_draft(logits, uniforms, draft, draft_len, accept_len, nex
     context), in one call.  workspace: uint8 CUDA tensor of
     pldp_verify_sample_draft_workspace_size(B, K, V, dtype) bytes.  Other arguments
     as pldp_verify_greedy_draft."""
+    if _calls is not None and _done("pldp_verify_sample_draft", _calls.verify_sample_draft(
+            logits, uniforms, draft, draft_len, accept_len, next_token, workspace, ids, seq_len, ngram_min, ngram_max,
+            cand_pos, cand_count, match_len, next_draft, next_draft_len, index, temperature, sampled, kv_keep_len, stream,
+            kw)):
+        return
     B, K1, V = logits.shape
     K = K1 - 1
     if draft.shape != (B, K) or next_draft.shape != (B, K):
@@ -534,6 +595,8 @@ def pldp_index_build(ids, seq_len, V, index, status=None, T_cap=None, stream=Non
     """Builds the incremental token index of pldp_draft_step over positions
     0 .. seq_len[b]-2 of every sequence.  index: uint8 CUDA tensor of
     pldp_index_size(B, V) bytes (cleared by the call)."""
+    if _calls is not None and _done("pldp_index_build", _calls.index_build(ids, seq_len, V, index, status, T_cap, stream)):
+        return
     p_ids, stride, T = _rows(ids, "ids", T_cap=T_cap)
     B = ids.shape[0]
     _check("pldp_index_build", _load().pldp_index_build(
@@ -553,6 +616,10 @@ def pldp_verify_greedy(logits, draft, draft_len, accept_len, next_token, workspa
     uint8 CUDA tensor of pldp_verify_workspace_size(B, K, V) bytes, zeroed once before
     first use (every call leaves it zeroed).  ids/seq_len (optional, modified in place)
     get the accepted tokens and the bonus token appended."""
+    if _calls is not None and _done("pldp_verify_greedy", _calls.verify_greedy(
+            logits, draft, draft_len, accept_len, next_token, workspace, argmax, ids, seq_len, kv_keep_len, status, T_cap,
+            stream)):
+        return
     B, K1, V = logits.shape
     K = K1 - 1
     if draft.shape != (B, K):
@@ -582,6 +649,10 @@ def pldp_verify_sample(logits, uniforms, draft, draft_len, accept_len, next_toke
     smallest v whose cumulative softmax(logits / T) probability exceeds uniforms[b, i]
     (float32 [B, K+1] CUDA tensor); acceptance and bookkeeping as pldp_verify_greedy.
     workspace: uint8 CUDA tensor of pldp_verify_sample_workspace_size(B, K, V, dtype) bytes."""
+    if _calls is not None and _done("pldp_verify_sample", _calls.verify_sample(
+            logits, uniforms, draft, draft_len, accept_len, next_token, workspace, temperature, sampled, ids, seq_len,
+            kv_keep_len, status, T_cap, stream)):
+        return
     B, K1, V = logits.shape
     K = K1 - 1
     if draft.shape != (B, K):

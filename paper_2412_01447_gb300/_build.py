@@ -11,12 +11,15 @@ import glob
 import os
 import shutil
 import subprocess
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(PKG, "libpldp.so")
+CALLS = os.path.join(PKG, "_pldp_calls.so")
+CALLS_SRC = os.path.join(CSRC, "host_calls.cpp")
 BUILD_DIR = os.path.join(PKG, "_build")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
@@ -47,8 +50,32 @@ def up_to_date() -> bool:
     return all(os.path.getmtime(p) <= t for p in _deps())
 
 
+def build_calls(force: bool = False) -> str:
+    """The binding's native checks and marshalling: a Python extension against the
+    installed torch's headers and libraries (host code only)."""
+    deps = [CALLS_SRC, os.path.join(INCLUDE, "pldp.h"), os.path.abspath(__file__)]
+    if not force and os.path.exists(CALLS) and all(os.path.getmtime(p) <= os.path.getmtime(CALLS) for p in deps):
+        return CALLS
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(nvcc())))
+    tmp = CALLS + f".tmp{os.getpid()}"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", INCLUDE, "-I", os.path.join(root, "include"),
+           "-I", os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include"), CALLS_SRC, "-o", tmp,
+           "-L", os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"building the binding's native calls failed:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, CALLS)
+    return CALLS
+
+
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     if not force and up_to_date():
+        build_calls()
         return LIB
     os.makedirs(BUILD_DIR, exist_ok=True)
     cc = nvcc()
@@ -65,7 +92,9 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
         return obj
 
     with cf.ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 1)) as ex:
+        calls = ex.submit(build_calls, force)
         objs = list(ex.map(compile_one, sources()))
+        calls.result()
     tmp = LIB + f".tmp{os.getpid()}"
     cmd = [cc, *ARCH, "-shared", "-Xcompiler", "-fPIC", "-o", tmp, *objs]
     r = subprocess.run(cmd, capture_output=True, text=True)

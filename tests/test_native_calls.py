@@ -1,0 +1,97 @@
+"""The binding's native checks (csrc/host_calls.cpp) against the Python ones: the same
+calls are made, with the same results, and what a check refuses is refused the same way."""
+import pytest
+import torch
+
+import paper_2412_01447_gb300 as pk
+import workloads as wl
+from tests._parity import Buffers, snapshot
+
+DEV = "cuda"
+
+
+def test_nothing_is_taken_off_the_device():
+    """Host tensors, wrong counts of arguments and other kinds are left to Python."""
+    pk.build()
+    pk._load()
+    c = pk._calls
+    x, y = torch.zeros((2, 8), dtype=torch.int32), torch.zeros(2, dtype=torch.int32)
+    assert c.find_candidates(x, y, 1, 3, x, y, y, None, None, None) is None
+    assert c.find_candidates(x) is None and c.top_heads(None, 1, y, None) is None
+    assert c.draft_step(x, y, 1, 3, x, y, y, 4, x, y, None, None, {"H": None}) is None
+    assert c.verify_greedy(None, x, y, y, y, y, None, None, None, None, None, None, None) is None
+    with pytest.raises(ValueError):
+        c.bind((1, 2))
+
+
+def _steps(buf, inp, w, index, calls):
+    """Every call of a decode step once, through the native checks or without them."""
+    B, K, V = w.B, w.K, w.V
+    ids, L, H, A = inp["ids"].clone(), inp["seq_len"].clone(), inp["H"], inp["A"]
+    rows = torch.arange(0, w.R, 2, dtype=torch.int32, device=DEV)
+    u = torch.linspace(0.05, 0.95, B * (K + 1), device=DEV).reshape(B, K + 1)
+    ws = torch.zeros(pk.pldp_verify_sample_draft_workspace_size(B, K, V), dtype=torch.uint8, device=DEV)
+    counts = torch.zeros(w.R, dtype=torch.int32, device=DEV)
+    top = torch.zeros(3, dtype=torch.int32, device=DEV)
+    kw = dict(H=H, best_h=buf.best_h, h_scores=buf.scores_h, A=A, best_a=buf.best_a, row_idx=rows, agg=1,
+              a_scores=buf.scores_a, draft_from="attention", status=buf.status, threshold=-0.5)
+    out = []
+    pk.pldp_find_candidates(ids, L, 1, 3, buf.cand, buf.cnt, buf.ml, buf.status, T_cap=w.T)
+    pk.pldp_rank_hidden(H, L, buf.cand, buf.cnt, buf.best_h, scores=buf.scores_h, best_score=buf.bscore_h)
+    pk.pldp_rank_attention(A, L, buf.cand, buf.cnt, buf.best_a, row_idx=rows, agg=1, scores=buf.scores_a)
+    pk.pldp_extract_draft(ids, L, buf.best_h, buf.draft, buf.dlen)
+    pk.pldp_verify_greedy(inp["logits"], buf.draft, buf.dlen, buf.acc, buf.nxt, buf.ws, argmax=buf.argmax)
+    pk.pldp_verify_sample(inp["logits"], u, buf.draft, buf.dlen, buf.acc, buf.nxt, ws, temperature=0.7)
+    out.append(snapshot(buf))
+    pk.pldp_index_build(ids, L, V, index, status=buf.status)
+    pk.pldp_draft_step(ids, L, 1, 3, buf.cand, buf.cnt, buf.ml, K, buf.draft, buf.dlen, buf.dws, **kw)
+    pk.pldp_verify_greedy_draft(inp["logits"], buf.draft, buf.dlen, buf.acc, buf.nxt, buf.ws, ids, L, 1, 3, buf.cand,
+                                buf.cnt, buf.ml, buf.draft, buf.dlen, index, argmax=buf.argmax, **kw)
+    pk.pldp_verify_sample_draft(inp["logits"], u, buf.draft, buf.dlen, buf.acc, buf.nxt, ws, ids, L, 1, 3, buf.cand,
+                                buf.cnt, buf.ml, buf.draft, buf.dlen, index, kv_keep_len=buf.kv, **kw)
+    pk.pldp_identify_heads(inp["ids"], inp["seq_len"] - 1, A.contiguous(), counts, max_suffix=16)
+    pk.pldp_top_heads(counts, 3, top)
+    out.append(snapshot(buf))
+    return out + [dict(ids=ids.cpu().numpy(), L=L.cpu().numpy(), counts=counts.cpu().numpy(), top=top.cpu().numpy())]
+
+
+@pytest.mark.gpu
+def test_native_and_python_calls_agree(lib, monkeypatch):
+    w = wl.CONFIGS["attention_b32_ctx8k"].replace(B=3, prompt_len=600, out_len=200, V=4000, d=256, h_dtype="bf16",
+                                                  layers=2, heads=4, planted_heads=2, C_cap=64)
+    inp = wl.single_step(w, device=DEV)
+    index = torch.empty(pk.pldp_index_size(w.B, w.V), dtype=torch.uint8, device=DEV)
+    taken = []
+
+    class Counted:
+        def __getattr__(self, name):
+            def call(*args):
+                rc = getattr(native, name)(*args)
+                taken.append((name, rc))
+                return rc
+            return call
+
+    native = pk._calls
+    assert native is not None
+    got = []
+    for calls in (Counted(), None):
+        monkeypatch.setattr(pk, "_calls", calls)
+        got.append(_steps(Buffers(w.B, w.K, w.V, w.C_cap, DEV), inp, w, index, calls))
+    assert len(taken) == 12 and all(rc == 0 for _, rc in taken), taken
+    for a, b in zip(*got):
+        for k in a:
+            assert (a[k] == b[k]).all() or ((a[k] != a[k]) == (b[k] != b[k])).all(), k
+
+
+@pytest.mark.gpu
+def test_errors_of_the_library_are_raised(lib):
+    """A call whose buffers pass and that the library refuses raises its message."""
+    ids = torch.zeros((2, 64), dtype=torch.int32, device=DEV)
+    L = torch.full((2,), 10, dtype=torch.int32, device=DEV)
+    buf = Buffers(2, 4, 8, 8, DEV)
+    with pytest.raises(pk.PldpError, match="ngram"):
+        pk.pldp_find_candidates(ids, L, 3, 1, buf.cand, buf.cnt, buf.ml)
+    with pytest.raises(TypeError):
+        pk.pldp_draft_step(ids, L, 1, 3, buf.cand, buf.cnt, buf.ml, 4, buf.draft, buf.dlen, buf.dws, no_such=1)
+    with pytest.raises(ValueError):
+        pk.pldp_extract_draft(ids, L, buf.best_h, buf.draft.t(), buf.dlen)
