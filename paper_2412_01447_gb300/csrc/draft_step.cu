@@ -117,38 +117,6 @@ struct alignas(16) DeferSlot {
 };
 static_assert(sizeof(DeferSlot) == 32 && 2 * sizeof(DeferSlot) <= kSeqWs, "B + 1 slots fit the workspace");
 
-// Warp reduce-scatter of N values (N a power of two, <= 32): at each butterfly
-// level a lane keeps half of its values and trades the other half with its
-// partner, so the N totals take N - 1 + 5 - log2(N) shuffles instead of 5 N.
-// Returns the total (sum, or max when use_max) of value lane >> (5 - log2 N).
-// Every total is formed in one fixed order, the same in every lane holding it.
-template <int N>
-__device__ __forceinline__ float warp_reduce_scatter(float (&v)[N], bool use_max) {
-    static_assert(N >= 1 && N <= 32 && (N & (N - 1)) == 0, "N: a power of two up to 32");
-    constexpr int LOG2N = N >= 32 ? 5 : N >= 16 ? 4 : N >= 8 ? 3 : N >= 4 ? 2 : N >= 2 ? 1 : 0;
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int s = 0; s < LOG2N; ++s) {
-        const int n = N >> s, o = 16 >> s;
-        const bool upper = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < N / 2; ++i) {
-            if (i >= n / 2) continue;
-            const float keep = upper ? v[i + n / 2] : v[i];
-            const float send = upper ? v[i] : v[i + n / 2];
-            const float got = __shfl_xor_sync(0xFFFFFFFFu, send, o);
-            v[i] = use_max ? fmaxf(keep, got) : keep + got;
-        }
-    }
-    float r = v[0];
-#pragma unroll
-    for (int o = 16 >> LOG2N; o > 0; o >>= 1) {
-        const float got = __shfl_xor_sync(0xFFFFFFFFu, r, o);
-        r = use_max ? fmaxf(r, got) : r + got;
-    }
-    return r;
-}
-
 template <int NB>
 __device__ __forceinline__ float (&part_buf(float (&part)[kMaxScoreBatch][kWarps][4]))[NB][kWarps][4] {
     return *reinterpret_cast<float(*)[NB][kWarps][4]>(&part[0]);

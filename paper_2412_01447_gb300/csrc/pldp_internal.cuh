@@ -20,6 +20,8 @@ pldp_status check_launch(const char* what);
 int sm_count();  // SMs of the current device
 // CTAs of `kernel` that fit on the whole current device at once (cached).
 int resident_blocks(const void* kernel, int threads, size_t smem);
+// Clusters of `size` CTAs of `kernel` that fit at once; 0 when it takes none (cached).
+int resident_clusters(const void* kernel, int threads, size_t smem, int size);
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -93,6 +95,34 @@ __device__ __forceinline__ int vfirst(const uint4& x, float m, float) {
     if (__uint_as_float(x.y) == m) return 1;
     if (__uint_as_float(x.z) == m) return 2;
     return 3;
+}
+
+// Two floats in one 64-bit register pair, and the packed fp32 operations on them (one
+// instruction for two lanes of fp32 FMA or add).
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float lo_f32(uint64_t x) {
+    [[maybe_unused]] float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x));
+    return lo;
+}
+__device__ __forceinline__ float hi_f32(uint64_t x) {
+    [[maybe_unused]] float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x));
+    return hi;
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
 }
 
 // Streaming 16-byte global load (read-once data: no L1 allocation).

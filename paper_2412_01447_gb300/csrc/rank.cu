@@ -15,7 +15,8 @@ namespace pldp {
 namespace {
 
 constexpr int kThreads = kRankThreads;
-constexpr int kMaxCluster = 8;
+constexpr int kMaxCluster = 8;                // portable
+constexpr int kWideCluster = 16;
 constexpr size_t kMaxQueryBytes = 196608;     // d * sizeof(dtype) limit
 constexpr int kMaxSelRows = 8192;             // row_idx entries staged in shared memory
 
@@ -85,12 +86,8 @@ __device__ __forceinline__ void prefetch_first(RankShared& sh, const int32_t* ca
     }
 }
 
-// 72 registers: the compiler's own choice for 256 threads was 64 with spills of the
-// per-warp candidate stream (8 loads in flight per lane); without them, at 3 CTAs per
-// SM, Eq. 3 on 510 candidates per sequence measured 116.6 -> 109.5 us (128 candidates:
-// 42.8 -> 43.3 us), alternated on one box.
 template <typename T, bool VEC, bool CLUSTER>
-__global__ void __maxnreg__(72)
+__global__ void __launch_bounds__(kThreads, 2)
 rank_hidden_kernel(const T* __restrict__ H, int64_t d, int64_t seq_stride,
                    const int32_t* __restrict__ seq_len, int64_t T_cap,
                    const int32_t* __restrict__ cand_pos, const int32_t* __restrict__ cand_count,
@@ -354,10 +351,20 @@ rank_attention_kernel(const void* __restrict__ A, bool a_bf16, int R, int64_t ro
 // CTAs per sequence: as many as the kernel's resident CTA slots allow for the
 // batch (all of its CTAs in one wave), up to a cluster of 8, never more than the
 // candidate capacity.  `kernel` is the variant launched when S > 1.
-int pick_split(int B, int C_cap, const void* kernel, size_t smem) {
+//
+// wide: up to a cluster of 16, where the slots allow it and most of the batch's clusters
+// are resident at once.  The sequence with the most candidates sets the time of Eq. 3's
+// call: 1024 of them (batch 16 x 32k Zipf tokens, unigram match) took 43.4 us with 8 CTAs
+// and one candidate per warp, 30.1 us with two per warp, 18.0 us with 16 CTAs.  Eq. 2
+// stays at 8: 16 gave it 8.8 -> 7.2 us there, but 9.3 -> 10.2 us with one candidate a
+// sequence after an L2 flush.
+int pick_split(int B, int C_cap, const void* kernel, size_t smem, bool wide = false) {
     int s = resident_blocks(kernel, kThreads, smem) / (B > 0 ? B : 1);
     if (s > C_cap) s = C_cap;
-    return s < 1 ? 1 : (s > kMaxCluster ? kMaxCluster : s);
+    if (s > kMaxCluster)
+        s = wide && s >= kWideCluster && 4 * resident_clusters(kernel, kThreads, smem, kWideCluster) >= 3 * B ? kWideCluster
+                                                                                                             : kMaxCluster;
+    return s < 1 ? 1 : s;
 }
 
 template <typename K, typename... Args>
@@ -379,6 +386,10 @@ cudaError_t launch_rank(K kernel, int B, int S, size_t smem, void* stream, Args.
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(smem));
+        if (e != cudaSuccess) return e;
+    }
+    if (S > kMaxCluster) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
     }
     return cudaLaunchKernelEx(&cfg, kernel, args..., S);
@@ -514,8 +525,9 @@ extern "C" PLDP_API pldp_status pldp_rank_hidden(const void* H, pldp_dtype dtype
 
     const bool vec = aligned16(H) && (d * es) % 16 == 0 && (seq_stride * es) % 16 == 0;
     const size_t smem = (static_cast<size_t>(d) * es + 127) / 128 * 128;
+    // (every variant fits as many CTAs an SM as this one)
     const int S = pick_split(B, C_cap, reinterpret_cast<const void*>(&rank_hidden_kernel<__nv_bfloat16, true, true>),
-                             smem);
+                             smem, true);
     cudaError_t e;
     if (dtype == PLDP_BF16) {
         const __nv_bfloat16* h = static_cast<const __nv_bfloat16*>(H);

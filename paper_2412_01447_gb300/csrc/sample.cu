@@ -62,35 +62,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
-// Two floats in one 64-bit register pair, and the packed fp32 operations on them
-// (one instruction for two lanes of fp32 FMA or add): the stats pass weighs its
-// elements two at a time.
-__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float lo_f32(uint64_t x) {
-    float lo, hi;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x));
-    return lo;
-}
-__device__ __forceinline__ float hi_f32(uint64_t x) {
-    float lo, hi;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x));
-    return hi;
-}
-__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
 // The elements of one 16-byte vector as floats.
 __device__ __forceinline__ void unpack(const uint4& x, float (&e)[8], __nv_bfloat16) {
     const uint32_t w[4] = {x.x, x.y, x.z, x.w};

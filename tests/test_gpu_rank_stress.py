@@ -68,3 +68,29 @@ def test_candidate_heavy_rankings(lib, B, T, V, d, R, dtype, C_cap, thr, agg, ke
     else:
         check_choice(g["best_a"], o_ba, o_sa, o_cand, o_cnt, C_cap)
     assert np.array_equal(g["status"].view(np.uint32), st)
+
+
+# Eq. 3 with a warp's candidates two at a time: counts around one and two per warp of a
+# CTA and of a cluster of 16, more than 32 per warp, rows of less than a load per lane and
+# of several passes, j = 0 and invalid entries among them
+@pytest.mark.parametrize("B,n,d,dtype", [(1, 8, 8, torch.bfloat16), (1, 127, 64, torch.float32), (2, 129, 4104, torch.bfloat16),
+                                         (3, 257, 1000, torch.float32), (16, 1024, 256, torch.bfloat16),
+                                         (130, 300, 64, torch.bfloat16), (150, 17, 520, torch.bfloat16)])
+def test_paired_candidates(lib, B, n, d, dtype):
+    T = 1400
+    gen = torch.Generator(device=DEV).manual_seed(n + d)
+    H = torch.randn((B, T, d), generator=gen, device=DEV).to(dtype)
+    cand = torch.stack([torch.randperm(T - 2, generator=gen, device=DEV)[:n].sort().values for _ in range(B)]).to(torch.int32)
+    cand[:, 0] = 0                                       # no H_{-1}
+    cand[:, n // 2] = T + 5                              # outside the context
+    cnt = torch.full((B,), n, dtype=torch.int32, device=DEV)
+    cnt[B // 2] = max(1, n - 5)
+    L = torch.full((B,), T, dtype=torch.int32, device=DEV)
+    sc = torch.zeros((B, n), dtype=torch.float32, device=DEV)
+    best = torch.zeros(B, dtype=torch.int32, device=DEV)
+    st = torch.zeros(B, dtype=torch.int32, device=DEV)
+    lib.pldp_rank_hidden(H, L, cand, cnt, best, scores=sc, status=st)
+    o_s, o_b, _ = oracle.rank_hidden(host(H), host(L), host(cand), host(cnt))
+    check_scores(host(sc), o_s, host(cnt), n)
+    check_choice(host(best), o_b, o_s, host(cand), host(cnt), n)
+    assert not st.any()
