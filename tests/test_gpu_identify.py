@@ -88,3 +88,28 @@ def test_top_heads_matches_stable_sort(lib, R, k):
     lib.pldp_top_heads(i32(c), k, out)
     want = np.argsort(-c.astype(np.int64), kind="stable")[:k]
     assert np.array_equal(host(out), want)
+
+
+# batches whose rows come two and four to a warp (16 and 32 a CTA), with a last CTA that
+# is not full and a last warp without rows; overlaps around what a lane compares by itself
+@pytest.mark.parametrize("B,R,T,dtype", [(40, 500, 64, torch.bfloat16), (40, 1000, 72, torch.bfloat16),
+                                         (60, 330, 60, torch.float32), (50, 801, 61, torch.bfloat16)])
+@pytest.mark.parametrize("V,max_suffix", [(2, 64), (3, 4), (3, 5), (9, 6)])
+def test_several_rows_per_warp(lib, B, R, T, dtype, V, max_suffix):
+    rng = np.random.default_rng(B + R + T + V)
+    ids = rng.integers(0, V, size=(B, T)).astype(np.int32)
+    pos = rng.integers(1, T, size=B).astype(np.int32)
+    A = torch.from_numpy(rng.integers(0, 4, size=(B, R, T)).astype(np.float32)).to(dtype)   # ties
+    for b in range(0, B, 2):                                        # rows that peak at an earlier copy
+        occ = np.nonzero(ids[b, :pos[b]] == ids[b, pos[b]])[0]
+        if occ.size:
+            A[b, rng.integers(0, R, size=R // 4), occ[-1]] = 9.0
+    counts = torch.zeros(R, dtype=torch.int32, device=DEV)
+    rs = torch.full((B,), -7, dtype=torch.int32, device=DEV)
+    lib.pldp_identify_heads(i32(ids), i32(pos), A.to(DEV), counts, max_suffix=max_suffix, r_star=rs)
+    oc, ors, _ = oracle.identify_heads(ids, pos, host(A), max_suffix, counts=np.zeros(R, np.uint32))
+    assert np.array_equal(host(rs), ors)
+    assert np.array_equal(host(counts).view(np.uint32), oc)
+    top = torch.full((R,), -1, dtype=torch.int32, device=DEV)
+    lib.pldp_top_heads(counts, R, top)
+    assert np.array_equal(host(top), np.argsort(-oc.astype(np.int64), kind="stable"))
