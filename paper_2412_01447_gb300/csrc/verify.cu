@@ -169,6 +169,73 @@ __device__ __forceinline__ SegKeys segment_argmax(const uint4* __restrict__ p, u
     return SegKeys{k0, k1};
 }
 
+// The same where rows are not a whole number of vectors: `rem` and V count elements, and
+// nvec whole vectors hold all but the last N - nvec * VW elements.  A row then starts
+// inside a vector: in the vector it starts in, and at the ragged end, the elements are
+// taken one by one.  Most segments lie inside a row and take the path above.
+template <typename T>
+__device__ __forceinline__ SegKeys ragged_argmax(const T* __restrict__ logits, uint32_t s0, uint32_t nvec, uint32_t N,
+                                                 uint32_t rem, uint32_t V, int lane) {
+    constexpr uint32_t VW = 16 / sizeof(T);
+    constexpr uint32_t seg = 32 * kSegLoads;
+    const uint4* p = reinterpret_cast<const uint4*>(logits);
+    if (rem + seg * VW <= V && s0 + seg <= nvec) {             // warp-uniform
+        uint4 x[kSegLoads];
+#pragma unroll
+        for (int u = 0; u < kSegLoads; ++u) x[u] = ld_stream16(p + s0 + lane + 32 * u);
+        float m = vmax(x[0], T());
+#pragma unroll
+        for (int u = 1; u < kSegLoads; ++u) m = fmaxf(m, vmax(x[u], T()));
+        const uint32_t ok = ordered_key(m);
+        const uint32_t wk = __reduce_max_sync(0xFFFFFFFFu, ok);
+        uint32_t idx = 0xFFFFFFFFu;
+        if (ok == wk) {
+#pragma unroll
+            for (int u = 0; u < kSegLoads; ++u)
+                if (idx == 0xFFFFFFFFu && vmax(x[u], T()) == m) idx = rem + (lane + 32 * u) * VW + vfirst(x[u], m, T());
+        }
+        idx = __reduce_min_sync(0xFFFFFFFFu, idx);
+        return SegKeys{pack_ordered(wk, idx), 0ull};
+    }
+    const uint32_t bnd = V - rem;                              // first element of the next row, from the segment's start
+    float b0 = -INFINITY, b1 = -INFINITY;
+    uint32_t i0 = rem, i1 = 0;
+#pragma unroll 1
+    for (int u = 0; u < kSegLoads; ++u) {
+        const uint32_t v = s0 + lane + 32 * u, e = (lane + 32 * u) * VW;      // e: from the segment's start
+        if (v < nvec && (e + VW <= bnd || e >= bnd)) {
+            const uint4 x = ld_stream16(p + v);
+            const float m = vmax(x, T());
+            if (e < bnd) {
+                if (m > b0) {
+                    b0 = m;
+                    i0 = rem + e + vfirst(x, m, T());
+                }
+            } else if (m > b1) {
+                b1 = m;
+                i1 = e - bnd + vfirst(x, m, T());
+            }
+        } else if (v <= nvec) {
+            for (uint32_t j = 0; j < VW && v * VW + j < N; ++j) {
+                const float x = to_f32(logits[static_cast<size_t>(v) * VW + j]);
+                if (e + j < bnd) {
+                    if (x > b0) {
+                        b0 = x;
+                        i0 = rem + e + j;
+                    }
+                } else if (x > b1) {
+                    b1 = x;
+                    i1 = e + j - bnd;
+                }
+            }
+        }
+    }
+    const unsigned long long k0 = warp_max_u64(pack_key(b0, i0));
+    unsigned long long k1 = 0ull;
+    if (seg * VW > bnd && s0 * VW + bnd < N) k1 = warp_max_u64(pack_key(b1, i1));
+    return SegKeys{k0, k1};
+}
+
 // Any segment: row by row, each row piece with the lane loop above.
 template <typename T, bool VEC>
 __device__ __forceinline__ void segment_rows(const T* __restrict__ logits, int64_t e0, int64_t e1, int64_t V,
@@ -187,16 +254,17 @@ __device__ __forceinline__ void segment_rows(const T* __restrict__ logits, int64
 }
 
 // 1. the row argmax pass.  W = warps in the grid.  PATH 0: 16-byte loads, rows of
-// at least a segment (the streaming path); 1: 16-byte loads, short rows; 2: element
-// loads (unaligned logits or rows that are not a whole number of 16 bytes).
+// at least a segment (the streaming path); 3: the same for rows that are not a whole number of 16
+// bytes (a vocabulary with an added token); 1: 16-byte loads, short rows; 2: element loads
+// (unaligned logits, and short rows that are not a whole number of 16 bytes).
 template <typename T, int PATH>
-__global__ void __launch_bounds__(kThreads, PATH == 0 ? kPassBlocksPerSm : 4)
+__global__ void __launch_bounds__(kThreads, PATH == 0 || PATH == 3 ? kPassBlocksPerSm : 4)
 verify_argmax_kernel(const T* __restrict__ logits, int64_t N, int64_t V, int64_t W,
                      unsigned long long* __restrict__ keys) {
     pdl_enter();
     const int lane = threadIdx.x & 31;
     const int64_t w = static_cast<int64_t>(blockIdx.x) * kWarps + (threadIdx.x >> 5);
-    if constexpr (PATH == 0) {
+    if constexpr (PATH == 0 || PATH == 3) {
         // Per round the CTA's warps hold 8 consecutive segments (16 KB, rarely more
         // than one row): their keys meet in shared memory and thread 0 issues one
         // atomicMax per row touched.  Rounds are counted from the CTA's first warp,
@@ -206,17 +274,24 @@ verify_argmax_kernel(const T* __restrict__ logits, int64_t N, int64_t V, int64_t
         const int warp = threadIdx.x >> 5;
         constexpr uint32_t VW = 16 / sizeof(T);
         constexpr uint32_t seg = 32 * kSegLoads;
-        const uint32_t nvec = static_cast<uint32_t>(N / VW), vrow = static_cast<uint32_t>(V / VW);
+        // rows and the offset in one are counted in vectors, or (ragged rows) in elements
+        constexpr uint32_t unit = PATH == 0 ? 1 : VW;
+        const uint32_t nvec = static_cast<uint32_t>(N / VW);
+        const uint32_t vrow = static_cast<uint32_t>(PATH == 0 ? V / VW : V);
+        const uint32_t end = PATH == 0 ? nvec : static_cast<uint32_t>((N + VW - 1) / VW);   // vectors, the last one ragged
         const uint32_t stride = static_cast<uint32_t>(W) * seg;
         const uint4* p = reinterpret_cast<const uint4*>(logits);
-        const uint32_t dq = stride / vrow, dr = stride - dq * vrow;      // rows and vectors per stride
+        const uint32_t dq = stride * unit / vrow, dr = stride * unit - dq * vrow;   // rows and units per stride
         uint32_t s0 = static_cast<uint32_t>(w) * seg;
-        uint32_t r0 = s0 / vrow, rem = s0 - r0 * vrow;
+        uint32_t r0 = s0 * unit / vrow, rem = s0 * unit - r0 * vrow;
         uint32_t first = blockIdx.x * kWarps * seg;                       // the CTA's first segment
-        for (int buf = 0; first < nvec; first += stride, buf ^= 1) {
-            const bool mine = s0 < nvec;
+        for (int buf = 0; first < end; first += stride, buf ^= 1) {
+            const bool mine = s0 < end;
             SegKeys k = {0ull, 0ull};
-            if (mine) k = segment_argmax<T>(p, s0, nvec, r0, rem, vrow, lane);
+            if (mine) {
+                if constexpr (PATH == 0) k = segment_argmax<T>(p, s0, nvec, r0, rem, vrow, lane);
+                else k = ragged_argmax<T>(logits, s0, nvec, static_cast<uint32_t>(N), rem, vrow, lane);
+            }
             if (lane == 0) {
                 srow[buf][warp] = mine ? r0 : 0xFFFFFFFFu;
                 sk[buf][warp][0] = k.k0;
@@ -304,14 +379,21 @@ pldp_status launch_verify_pass(const void* logits, pldp_dtype dtype, VerifyArgs&
     const int64_t bytes = static_cast<int64_t>(a.B) * (a.K + 1) * a.V * static_cast<int64_t>(es);
     const bool long_rows = static_cast<int64_t>(a.V) * static_cast<int64_t>(es) >= kSegBytes;
     const bool small = bytes / 16 < (int64_t(1) << 31);     // 32-bit vector indices
-    const int path = vec ? (long_rows && small ? 0 : 1) : 2;
+    // Ragged rows of at least a segment stream like the others where their element indices
+    // fit 32 bits (one stride past the end among them).  By element loads, 2 bytes a lane,
+    // batch 128 x 13 rows of 128255 bf16 took 150 us, and 64 x 11 rows of 32001 27.5 us; so
+    // they take 68 and 18.4 us (rows of 128256 and 32000: 66 and 16.3), L2 flushed.
+    const bool ragged = !vec && aligned16(logits) && long_rows && bytes / static_cast<int64_t>(es) < (int64_t(1) << 31);
+    const int path = vec ? (long_rows && small ? 0 : 1) : ragged ? 3 : 2;
     if (dtype == PLDP_BF16) {
         if (path == 0) return launch_pass_t<__nv_bfloat16, 0>(logits, a, scratch, s, what);
         if (path == 1) return launch_pass_t<__nv_bfloat16, 1>(logits, a, scratch, s, what);
+        if (path == 3) return launch_pass_t<__nv_bfloat16, 3>(logits, a, scratch, s, what);
         return launch_pass_t<__nv_bfloat16, 2>(logits, a, scratch, s, what);
     }
     if (path == 0) return launch_pass_t<float, 0>(logits, a, scratch, s, what);
     if (path == 1) return launch_pass_t<float, 1>(logits, a, scratch, s, what);
+    if (path == 3) return launch_pass_t<float, 3>(logits, a, scratch, s, what);
     return launch_pass_t<float, 2>(logits, a, scratch, s, what);
 }
 
