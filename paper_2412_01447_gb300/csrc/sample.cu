@@ -47,6 +47,32 @@ namespace {
 
 constexpr int64_t kPieceBytes = 2048;
 
+// How the logits are read: element by element, in 16-byte vectors, or in vectors where
+// rows are not a whole number of them (pieces cut as the stats kernel's RAGGED form says).
+enum class Rows { kElements, kVectors, kRagged };
+
+// Elements of a row's first vector that belong to the row before.
+template <typename T>
+__device__ __forceinline__ uint32_t row_head(uint64_t r, uint32_t V) {
+    constexpr uint32_t VW = 16 / sizeof(T);
+    return (static_cast<uint32_t>(r) % VW) * (V % VW) % VW;
+}
+
+// Ragged pieces stay as many as whole rows' would be when a row's last piece has room for
+// the elements that the cut at its start moves there.
+template <typename T>
+bool ragged_pieces(int V) {
+    constexpr int P = static_cast<int>(kPieceBytes / sizeof(T)), VW = 16 / static_cast<int>(sizeof(T));
+    return (V - 1) % P + 1 + (VW - 1) <= P;
+}
+// `units`: pieces in all (the ragged form has 32-bit unit arithmetic only).
+template <typename T>
+Rows rows_of(const void* logits, int V, int64_t units) {
+    if (!aligned16(logits)) return Rows::kElements;
+    if ((static_cast<size_t>(V) * sizeof(T)) % 16 == 0) return Rows::kVectors;
+    return ragged_pieces<T>(V) && units < (int64_t(1) << 31) ? Rows::kRagged : Rows::kElements;
+}
+
 struct SampleArgs {
     VerifyArgs v;                   // draft, bookkeeping; v.argmax receives the draws
     const float* uniforms;          // [B*(K+1)]
@@ -101,10 +127,35 @@ __device__ __forceinline__ float ordered_value(uint32_t o) {
 // the 32 registers of 8 CTAs per SM without spilling: 72.2 -> 69.5 us per call at
 // the sustained-loop shape against the earlier 64-bit form, which spilled.  Each
 // lane's weights are summed in even/odd pairs with packed fp32 FMA and add.
+//
+// RAGGED: rows that are not a whole number of vectors (a vocabulary with an added token).
+// A row then starts `head` elements into a vector, and its pieces are cut at whole vectors
+// all the same: piece k covers the row's elements [k P - head, (k+1) P - head) (those there
+// are), so only a row's first and last vector are cut.  These are read element by element,
+// with -inf, which weighs nothing, in the place of the neighbouring rows' elements.
+// Batch 128 x 13 rows of 128255 bf16, L2 flushed: 155 us a call by element loads, 80 us so
+// (rows of 128256: 68 us); cutting every row's pieces at its own start, two cut vectors a
+// piece, took 118 us.
 template <typename T>
+__device__ __noinline__ uint4 edge_vector(const T* base, uint64_t first, uint64_t total, int lo, int hi) {
+    // the vector that starts at element `first`, its elements outside [lo, hi) -inf
+    constexpr int VW = 16 / static_cast<int>(sizeof(T));
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int j = 0; j < VW; ++j) {
+        const bool in = j >= lo && j < hi && first + j < total;
+        if constexpr (sizeof(T) == 2)
+            w[j / 2] |= (in ? static_cast<uint32_t>(__bfloat16_as_ushort(base[first + j])) : 0xFF80u) << (16 * (j % 2));
+        else
+            w[j] = in ? __float_as_uint(base[first + j]) : 0xFF800000u;
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+template <typename T, bool RAGGED>
 __global__ void __launch_bounds__(kThreads, kPassBlocksPerSm)
 sample_stats_vec_kernel(const T* __restrict__ logits, uint32_t V, uint32_t units, uint32_t npieces, uint32_t P,
-                        float c, uint32_t W, uint32_t dr, uint32_t dk, float2* __restrict__ stats) {
+                        float c, uint32_t W, uint32_t dr, uint32_t dk, float2* __restrict__ stats, uint64_t total) {
     // W = warps in the grid = dr rows and dk pieces
     pdl_wait_only();                        // the finish (a full SM per CTA) starts as this grid ends
     constexpr uint32_t VW = 16 / sizeof(T);
@@ -113,12 +164,28 @@ sample_stats_vec_kernel(const T* __restrict__ logits, uint32_t V, uint32_t units
     uint32_t r = w / npieces, k = w - r * npieces;
     for (uint32_t u = w; u < units; u += W) {
         const uint32_t e0 = k * P;
-        const uint32_t nv = (V - e0 < P ? V - e0 : P) / VW;            // vectors in this piece
-        const uint4* pv = reinterpret_cast<const uint4*>(logits + (static_cast<uint64_t>(r) * V + e0));
+        const uint32_t head = RAGGED ? row_head<T>(r, V) : 0u;
+        const uint32_t end = V + head;                                 // of the row, from its first vector's start
+        const uint32_t nv = ((end - e0 < P ? end - e0 : P) + VW - 1) / VW;   // vectors in this piece
+        const uint64_t f0 = static_cast<uint64_t>(r) * V - head + e0;  // the element its first vector starts with
+        const uint4* pv = reinterpret_cast<const uint4*>(logits + f0);
         uint4 raw[kSegLoads];
 #pragma unroll
-        for (int q = 0; q < kSegLoads; ++q)
-            if (lane + 32u * q < nv) raw[q] = ld_stream16(pv + lane + 32 * q);
+        for (int q = 0; q < kSegLoads; ++q) {
+            const uint32_t i = lane + 32u * q;
+            if (i < nv && (!RAGGED || e0 + (i + 1) * VW <= end)) raw[q] = ld_stream16(pv + i);
+        }
+        if constexpr (RAGGED) {
+            if (e0 == 0 || e0 + P >= end)                              // a cut vector in this piece (warp-uniform)
+#pragma unroll
+                for (int q = 0; q < kSegLoads; ++q) {
+                    const uint32_t i = lane + 32u * q, at = e0 + i * VW;
+                    if (i < nv && (at < head || at + VW > end))
+                        raw[q] = edge_vector<T>(logits, f0 + static_cast<uint64_t>(i) * VW, total,
+                                                at < head ? static_cast<int>(head - at) : 0,
+                                                at + VW > end ? static_cast<int>(end - at) : static_cast<int>(VW));
+                }
+        }
         float m = -INFINITY, sum = 0.f;
 #pragma unroll
         for (int q = 0; q < kSegLoads; ++q)
@@ -153,8 +220,7 @@ sample_stats_vec_kernel(const T* __restrict__ logits, uint32_t V, uint32_t units
     }
 }
 
-// The element-load form, for unaligned logits or rows that are not a whole number
-// of 16-byte vectors.
+// The element-load form, for unaligned logits.
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 4)
 sample_stats_kernel(const T* __restrict__ logits, int64_t V, int64_t rows, int npieces, int P, float c,
@@ -289,7 +355,7 @@ __device__ __forceinline__ PiecePick pick_piece(const float2* __restrict__ st, i
 }
 
 // The draw of row r (one warp).
-template <typename T, bool VEC>
+template <typename T, Rows RD>
 __device__ int sample_row(const T* __restrict__ logits, const SampleArgs& a, int64_t r, int lane) {
     const int64_t V = a.v.V;
     const int np = a.npieces;
@@ -314,23 +380,27 @@ __device__ int sample_row(const T* __restrict__ logits, const SampleArgs& a, int
     const int ks = pk.k;
     // the piece, lane L holding its elements [L E, (L+1) E) in index order
     constexpr int E = static_cast<int>(kPieceBytes / sizeof(T)) / 32;
-    const int64_t e0 = static_cast<int64_t>(ks) * a.P;
+    const int64_t e0 = static_cast<int64_t>(ks) * a.P - (RD == Rows::kRagged ? row_head<T>(r, V) : 0);   // may be negative
     const int64_t n = (V - e0 < a.P) ? V - e0 : a.P;
     const T* piece = logits + r * V + e0;
     const float Mkc = pk.Mk * a.c;
     float x[E];
-    if constexpr (VEC) {
+    if constexpr (RD != Rows::kElements) {
         constexpr int VW = 16 / static_cast<int>(sizeof(T));
         const uint4* pv = reinterpret_cast<const uint4*>(piece) + lane * (E / VW);
+        const int64_t left = RD == Rows::kRagged ? static_cast<int64_t>(a.v.B) * (a.v.K + 1) * V - (r * V + e0) : n;
 #pragma unroll
         for (int q = 0; q < E / VW; ++q) {
             const int64_t ei = static_cast<int64_t>(lane) * E + q * VW;
             uint4 raw = make_uint4(0u, 0u, 0u, 0u);
-            if (ei < n) raw = __ldcg(pv + q);
+            if (ei < n && ei + VW <= left) raw = __ldcg(pv + q);
             float e[8];
             unpack(raw, e, T());
+            if (RD == Rows::kRagged && ei < n && ei + VW > left)       // the last vector of the logits, not whole
 #pragma unroll
-            for (int j = 0; j < VW; ++j) x[q * VW + j] = ei + j < n ? e[j] : -INFINITY;
+                for (int j = 0; j < VW; ++j) e[j] = ei + j < n ? to_f32(piece[ei + j]) : 0.f;
+#pragma unroll
+            for (int j = 0; j < VW; ++j) x[q * VW + j] = ei + j < n && e0 + ei + j >= 0 ? e[j] : -INFINITY;
         }
     } else {
 #pragma unroll
@@ -363,7 +433,8 @@ __device__ int sample_row(const T* __restrict__ logits, const SampleArgs& a, int
         }
         if (y < 0) y = last;                                      // rounding inside the lane
         if (y < 0) y = 0;
-        y = static_cast<int>(static_cast<int64_t>(L0) * E + y + e0);
+        const int64_t at = static_cast<int64_t>(L0) * E + y + e0;
+        y = at > 0 ? static_cast<int>(at) : 0;
     }
     return __shfl_sync(0xFFFFFFFFu, y, L0);
 }
@@ -371,7 +442,7 @@ __device__ int sample_row(const T* __restrict__ logits, const SampleArgs& a, int
 // 2. draws and acceptance: one CTA per sequence, warp w draws rows w, w + 16, ...
 constexpr int kFinishWarps = 16;
 
-template <typename T, bool VEC>
+template <typename T, Rows RD>
 __global__ void __launch_bounds__(32 * kFinishWarps, 1) sample_finish_kernel(const T* __restrict__ logits,
                                                                             SampleArgs a) {
     extern __shared__ int32_t draws[];                           // [K+1]
@@ -386,7 +457,7 @@ __global__ void __launch_bounds__(32 * kFinishWarps, 1) sample_finish_kernel(con
         if (lane == 1 && a.v.seq_len) asm volatile("prefetch.global.L1 [%0];" ::"l"(a.v.seq_len + b));
     }
     for (int i = warp; i < K1; i += kFinishWarps) {
-        const int y = sample_row<T, VEC>(logits, a, b * K1 + i, lane);
+        const int y = sample_row<T, RD>(logits, a, b * K1 + i, lane);
         if (lane == 0) draws[i] = y;
     }
     __syncthreads();
@@ -396,14 +467,14 @@ __global__ void __launch_bounds__(32 * kFinishWarps, 1) sample_finish_kernel(con
 // Draws only, for the fused sampling + next draft call: one warp per row, each
 // draw to draws[row]; the accept/bonus/append and the drafting follow in the
 // next kernel.
-template <typename T, bool VEC>
+template <typename T, Rows RD>
 __global__ void __launch_bounds__(kThreads) sample_draw_kernel(const T* __restrict__ logits, SampleArgs a,
                                                                 int32_t* __restrict__ draws) {
     pdl_enter();
     const int64_t r = static_cast<int64_t>(blockIdx.x) * kWarps + (threadIdx.x >> 5);   // warp-uniform
     const int64_t rows = static_cast<int64_t>(a.v.B) * (a.v.K + 1);
     if (r >= rows) return;
-    const int y = sample_row<T, VEC>(logits, a, r, threadIdx.x & 31);
+    const int y = sample_row<T, RD>(logits, a, r, threadIdx.x & 31);
     if ((threadIdx.x & 31) == 0) draws[r] = y;
 }
 
@@ -412,13 +483,14 @@ int sample_pieces(int V, size_t es) {
     return static_cast<int>((V + P - 1) / P);
 }
 
-template <typename T, bool VEC>
+template <typename T, Rows RD>
 pldp_status launch_stats_t(const void* logits, const SampleArgs& a, cudaStream_t s, const char* what) {
     const int64_t rows = static_cast<int64_t>(a.v.B) * (a.v.K + 1);
     const int64_t units = rows * a.npieces;
-    const bool vec = VEC && units < (int64_t(1) << 31);               // 32-bit unit arithmetic
-    const void* fn = vec ? reinterpret_cast<const void*>(&sample_stats_vec_kernel<T>)
-                         : reinterpret_cast<const void*>(&sample_stats_kernel<T>);
+    const bool stream = RD != Rows::kElements && units < (int64_t(1) << 31);   // 32-bit unit arithmetic
+    void (*const vec)(const T*, uint32_t, uint32_t, uint32_t, uint32_t, float, uint32_t, uint32_t, uint32_t, float2*,
+                      uint64_t) = sample_stats_vec_kernel<T, RD == Rows::kRagged>;
+    const void* fn = stream ? reinterpret_cast<const void*>(vec) : reinterpret_cast<const void*>(&sample_stats_kernel<T>);
     int64_t blocks = static_cast<int64_t>(resident_blocks(fn, kThreads, 0)) * kPassWaves;
     const int64_t need = (units + kWarps - 1) / kWarps;
     if (blocks > need) blocks = need;
@@ -426,42 +498,42 @@ pldp_status launch_stats_t(const void* logits, const SampleArgs& a, cudaStream_t
     const T* lp = static_cast<const T*>(logits);
     float2* st = const_cast<float2*>(a.stats);
     const cudaError_t e =
-        vec ? launch_pdl(sample_stats_vec_kernel<T>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, s, 0, lp,
-                         static_cast<uint32_t>(a.v.V), static_cast<uint32_t>(units), static_cast<uint32_t>(a.npieces),
-                         static_cast<uint32_t>(a.P), a.c, static_cast<uint32_t>(blocks * kWarps),
-                         static_cast<uint32_t>(blocks * kWarps / a.npieces),
-                         static_cast<uint32_t>(blocks * kWarps % a.npieces), st)
-            : launch_pdl(sample_stats_kernel<T>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, s, 0, lp,
-                         static_cast<int64_t>(a.v.V), rows, a.npieces, a.P, a.c, blocks * kWarps, st);
+        stream ? launch_pdl(vec, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, s, 0, lp,
+                            static_cast<uint32_t>(a.v.V), static_cast<uint32_t>(units), static_cast<uint32_t>(a.npieces),
+                            static_cast<uint32_t>(a.P), a.c, static_cast<uint32_t>(blocks * kWarps),
+                            static_cast<uint32_t>(blocks * kWarps / a.npieces),
+                            static_cast<uint32_t>(blocks * kWarps % a.npieces), st, static_cast<uint64_t>(rows) * a.v.V)
+               : launch_pdl(sample_stats_kernel<T>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, s, 0, lp,
+                            static_cast<int64_t>(a.v.V), rows, a.npieces, a.P, a.c, blocks * kWarps, st);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "%s: launch failed: %s", what, cudaGetErrorString(e));
     return PLDP_OK;
 }
 
-template <typename T, bool VEC>
+template <typename T, Rows RD>
 pldp_status launch_draws_t(const void* logits, const SampleArgs& a, int32_t* draws, cudaStream_t s,
                            const char* what) {
-    const pldp_status st = launch_stats_t<T, VEC>(logits, a, s, what);
+    const pldp_status st = launch_stats_t<T, RD>(logits, a, s, what);
     if (st != PLDP_OK) return st;
     const int64_t rows = static_cast<int64_t>(a.v.B) * (a.v.K + 1);
-    const cudaError_t e = launch_pdl(sample_draw_kernel<T, VEC>, dim3(static_cast<unsigned>((rows + kWarps - 1) / kWarps)),
+    const cudaError_t e = launch_pdl(sample_draw_kernel<T, RD>, dim3(static_cast<unsigned>((rows + kWarps - 1) / kWarps)),
                                      dim3(kThreads), 0, s, 0, static_cast<const T*>(logits), a, draws);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "%s: launch failed: %s", what, cudaGetErrorString(e));
     return PLDP_OK;
 }
 
-template <typename T, bool VEC>
+template <typename T, Rows RD>
 pldp_status launch_sample_t(const void* logits, SampleArgs a, cudaStream_t s) {
-    const pldp_status st = launch_stats_t<T, VEC>(logits, a, s, "verify_sample");
+    const pldp_status st = launch_stats_t<T, RD>(logits, a, s, "verify_sample");
     if (st != PLDP_OK) return st;
     cudaError_t e;
     const size_t smem = static_cast<size_t>(a.v.K + 1) * sizeof(int32_t);
     if (smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(sample_finish_kernel<T, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(sample_finish_kernel<T, RD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  static_cast<int>(smem));
         if (e != cudaSuccess)
             return fail(PLDP_ERR_CUDA, "verify_sample: shared memory attribute: %s", cudaGetErrorString(e));
     }
-    e = launch_pdl(sample_finish_kernel<T, VEC>, dim3(static_cast<unsigned>(a.v.B)), dim3(32 * kFinishWarps), smem, s, 0,
+    e = launch_pdl(sample_finish_kernel<T, RD>, dim3(static_cast<unsigned>(a.v.B)), dim3(32 * kFinishWarps), smem, s, 0,
                    static_cast<const T*>(logits), a);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "verify_sample: launch failed: %s", cudaGetErrorString(e));
     return PLDP_OK;
@@ -494,12 +566,19 @@ pldp_status launch_sample_draws(const void* logits, pldp_dtype dtype, VerifyArgs
     int32_t* draws = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) +
                                                 (rows * a.npieces * sizeof(float2) + 255) / 256 * 256);
     v.row_draws = draws;
-    const bool vec = aligned16(logits) && (static_cast<size_t>(v.V) * es) % 16 == 0;
-    if (dtype == PLDP_BF16)
-        return vec ? launch_draws_t<__nv_bfloat16, true>(logits, a, draws, s, what)
-                   : launch_draws_t<__nv_bfloat16, false>(logits, a, draws, s, what);
-    return vec ? launch_draws_t<float, true>(logits, a, draws, s, what)
-               : launch_draws_t<float, false>(logits, a, draws, s, what);
+    const int64_t units = static_cast<int64_t>(rows) * a.npieces;
+    if (dtype == PLDP_BF16) {
+        switch (rows_of<__nv_bfloat16>(logits, v.V, units)) {
+            case Rows::kVectors: return launch_draws_t<__nv_bfloat16, Rows::kVectors>(logits, a, draws, s, what);
+            case Rows::kRagged: return launch_draws_t<__nv_bfloat16, Rows::kRagged>(logits, a, draws, s, what);
+            default: return launch_draws_t<__nv_bfloat16, Rows::kElements>(logits, a, draws, s, what);
+        }
+    }
+    switch (rows_of<float>(logits, v.V, units)) {
+        case Rows::kVectors: return launch_draws_t<float, Rows::kVectors>(logits, a, draws, s, what);
+        case Rows::kRagged: return launch_draws_t<float, Rows::kRagged>(logits, a, draws, s, what);
+        default: return launch_draws_t<float, Rows::kElements>(logits, a, draws, s, what);
+    }
 }
 
 }  // namespace pldp
@@ -548,9 +627,17 @@ extern "C" PLDP_API pldp_status pldp_verify_sample(
     a.npieces = sample_pieces(V, es);
     a.P = static_cast<int>(kPieceBytes / static_cast<int64_t>(es));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const bool vec = aligned16(logits) && (static_cast<size_t>(V) * es) % 16 == 0;
-    if (dtype == PLDP_BF16)
-        return vec ? launch_sample_t<__nv_bfloat16, true>(logits, a, s) : launch_sample_t<__nv_bfloat16, false>(logits, a, s);
-    return vec ? launch_sample_t<float, true>(logits, a, s) : launch_sample_t<float, false>(logits, a, s);
+    const int64_t units = static_cast<int64_t>(B) * (K + 1) * a.npieces;
+    if (dtype == PLDP_BF16) {
+        switch (rows_of<__nv_bfloat16>(logits, V, units)) {
+            case Rows::kVectors: return launch_sample_t<__nv_bfloat16, Rows::kVectors>(logits, a, s);
+            case Rows::kRagged: return launch_sample_t<__nv_bfloat16, Rows::kRagged>(logits, a, s);
+            default: return launch_sample_t<__nv_bfloat16, Rows::kElements>(logits, a, s);
+        }
+    }
+    switch (rows_of<float>(logits, V, units)) {
+        case Rows::kVectors: return launch_sample_t<float, Rows::kVectors>(logits, a, s);
+        case Rows::kRagged: return launch_sample_t<float, Rows::kRagged>(logits, a, s);
+        default: return launch_sample_t<float, Rows::kElements>(logits, a, s);
+    }
 }
-

@@ -1,7 +1,7 @@
 """Verification where rows of logits are not a whole number of 16 bytes (a vocabulary with
-an added token): the streaming pass cuts rows inside vectors.  Argmaxes against the oracle
-bit for bit, at row lengths around the limits of the paths, with maxima and ties at the
-rows' ends."""
+an added token): the streaming passes cut rows inside vectors.  Greedy argmaxes against the
+oracle bit for bit, sampling draws as in test_gpu_sample.py, at row lengths around the
+limits of the paths, with maxima and ties at the rows' ends."""
 import numpy as np
 import pytest
 import torch
@@ -9,6 +9,7 @@ import torch
 import oracle
 import paper_2412_01447_gb300 as pk
 from tests._parity import host
+from tests.test_gpu_sample import _f64, _run, _valid_draw
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -43,3 +44,27 @@ def test_greedy(lib, V, dtype, B, K):
         assert np.array_equal(host(am), o["argmax"])
         assert np.array_equal(host(acc), o["accept_len"]) and np.array_equal(host(nxt), o["next_token"])
         assert not ws.any()
+
+
+# a last piece with and without room for the elements that a cut row start moves there
+# (1017 and 1021 of 1024, 509 and 510 of 512), rows shorter than a vector, several pieces
+@pytest.mark.parametrize("V,dtype", [(3, torch.bfloat16), (1017, torch.bfloat16), (1021, torch.bfloat16),
+                                     (2041, torch.bfloat16), (32001, torch.bfloat16), (509, torch.float32),
+                                     (510, torch.float32), (32003, torch.float32)])
+@pytest.mark.parametrize("T", [0.6, 1.0])
+def test_sampling(lib, V, dtype, T):
+    B, K = 5, 12
+    gen = torch.Generator(device=DEV).manual_seed(V)
+    logits = (torch.randn((B, K + 1, V), generator=gen, device=DEV) * 2).to(dtype)
+    logits[:, ::3, 0] += 9.0                             # weight at the rows' ends
+    logits[:, 1::3, V - 1] += 9.0
+    u = torch.rand((B, K + 1), generator=gen, device=DEV)
+    u[0, :3] = torch.tensor([0.0, 1.0, 0.999999], device=DEV)
+    draft, dlen = torch.zeros((B, K), dtype=torch.int32, device=DEV), torch.zeros(B, dtype=torch.int32, device=DEV)
+    _, ys, _ = _run(logits, u, draft, dlen, T)
+    o = oracle.verify_sample(host(logits), host(u), host(draft), host(dlen), T)["sampled"]
+    l64 = _f64(logits)
+    diff = np.argwhere(ys != o)
+    assert len(diff) <= 2, diff
+    for b, i in diff:
+        assert _valid_draw(l64[b, i], T, float(u[b, i]), int(ys[b, i])), (b, i, ys[b, i], o[b, i])
