@@ -328,7 +328,7 @@ PLDP_API size_t pldp_draft_workspace_size(int B);
  * Per sequence and token it holds the number of occurrences among the indexed
  * positions and up to 15 of them (one 64-byte entry); per sequence the number of
  * positions indexed.
- * pldp_index_build clears `index` and indexes positions 0 .. seq_len[b]-2 of
+ * pldp_index_build overwrites `index` and indexes positions 0 .. seq_len[b]-2 of
  * every sequence (all but the last token, which the next draft step looks up).
  * Token ids outside [0, V) mark that sequence's index unusable (TOKEN_RANGE);
  * seq_len outside [0, T_cap] too (SEQ_LEN).  Memory: about B * V * 64 bytes.

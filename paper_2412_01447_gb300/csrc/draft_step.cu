@@ -1280,35 +1280,84 @@ __global__ void __launch_bounds__(kThreads, 1) verify_draft_kernel(const VerifyA
     index_draft<TH, IVEC, CoherentIds, true>(p, ix, b, L, sh, is, il);
 }
 
-// Index build: positions 0 .. seq_len-2 of every sequence.
-__global__ void __launch_bounds__(kThreads) index_build_kernel(const int32_t* __restrict__ ids, int64_t ids_stride,
-                                                               const int32_t* __restrict__ seq_len, int64_t T_cap,
-                                                               IndexView ix) {
-    pdl_enter();
-    const int b = blockIdx.y;
-    const int64_t L = seq_len[b];
-    if (L < 0 || L > T_cap) return;
-    const int64_t t = L - 1;
-    const int32_t* row = ids + static_cast<int64_t>(b) * ids_stride;
-    for (int64_t q = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; q < t;
-         q += static_cast<int64_t>(gridDim.x) * kThreads)
-        if (!index_insert(ix, b, q, __ldg(row + q))) atomicOr(ix.flags + b, 1);
-}
+// Index build: positions 0 .. seq_len-2 of every sequence, by a cluster per sequence that
+// clears the sequence's entries and then inserts its positions.  Only the first half of
+// an entry is cleared (a 32-byte sector: the count and seven slots; a slot is read only
+// below the count), which is all that most entries of a vocabulary ever see.
+//
+// What bounds it: the clearing, V * 32 bytes a sequence (525 MB at batch 128, V = 128256:
+// 85 us alone), and the atomics, whose entries leave L2 again when many sequences are
+// under way.  A memset of everything (1.05 GB, 155 us), a kernel that inserted (83 us) and
+// one that wrote the lengths took 230-240 us there, 207 us now; batch 16 x 8k, V = 128256:
+// 64 -> 28 us; batch 64 x 16k, V = 32000: 69 -> 38 us; batch 1 x 4k: 19.5 -> 13 us.
+constexpr int kBuildThreads = 1024;
+constexpr int kBuildLoads = 4;                     // positions in flight per thread
+// Tokens cleared and counted at a time, when there are more sequences than clusters at
+// once: entries then wait less long for their positions (228 -> 207 us at the first size
+// above; 16384 gave 197, and 45 for 28 us at the second, where one pass is best).
+constexpr int64_t kBuildTokens = 32768;
 
-__global__ void index_finish_kernel(const int32_t* __restrict__ seq_len, int B, int64_t T_cap, IndexView ix,
-                                    uint32_t* __restrict__ status) {
+__global__ void __launch_bounds__(kBuildThreads, 2)
+index_build_kernel(const int32_t* __restrict__ ids, int64_t ids_stride, const int32_t* __restrict__ seq_len, int B,
+                   int64_t T_cap, IndexView ix, uint32_t* __restrict__ status, int S,
+                   int64_t tokens) {
     pdl_enter();
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
+    const int b = blockIdx.x / S;
+    const int rank = blockIdx.x - b * S;
+    const int tid = threadIdx.x;
     const int64_t L = seq_len[b];
-    if (L < 0 || L > T_cap) {
-        ix.ilen[b] = -1;
-        if (status) atomicOr(status + b, PLDP_ST_SEQ_LEN);
-        return;
+    const bool valid = L >= 0 && L <= T_cap;
+    const int64_t t = valid ? L - 1 : 0;
+    if (rank == 0 && tid == 0) {
+        ix.flags[b] = 0;
+        ix.defer[b] = DeferSlot{};
+        if (b == 0) ix.defer[B] = DeferSlot{};
     }
-    const bool bad_token = ix.flags[b] != 0;
-    ix.ilen[b] = bad_token ? -1 : static_cast<int32_t>(L >= 1 ? L - 1 : 0);
-    if (bad_token && status) atomicOr(status + b, PLDP_ST_TOKEN_RANGE);
+    const int step = S * kBuildThreads, first = rank * kBuildThreads + tid;
+    uint4* entries = reinterpret_cast<uint4*>(index_entry(ix, b, 0));   // four vectors each
+    const int32_t* row = ids + static_cast<int64_t>(b) * ids_stride;
+    bool bad = false;                              // a token the index cannot hold
+    for (int64_t v0 = 0; v0 < ix.V; v0 += tokens) {                    // cluster-uniform
+        const int64_t v1 = v0 + tokens < ix.V ? v0 + tokens : ix.V;
+#pragma unroll 4
+        for (int64_t u = 2 * v0 + first; u < 2 * v1; u += step)
+            entries[(u >> 1) * (kEntryWords / 4) + (u & 1)] = make_uint4(0u, 0u, 0u, 0u);   // a sector per two lanes
+        if (S > 1) {
+            cluster_arrive();
+            cluster_wait();
+        } else {
+            __syncthreads();
+        }
+        for (int64_t q0 = first; q0 < t; q0 += static_cast<int64_t>(step) * kBuildLoads) {
+            int32_t tok[kBuildLoads];
+            int slot[kBuildLoads];
+#pragma unroll
+            for (int u = 0; u < kBuildLoads; ++u) {
+                const int64_t q = q0 + static_cast<int64_t>(u) * step;
+                tok[u] = q < t ? __ldg(row + q) : static_cast<int32_t>(v0);
+                bad |= tok[u] < 0 || tok[u] >= ix.V;
+            }
+#pragma unroll
+            for (int u = 0; u < kBuildLoads; ++u) {
+                const bool in = q0 + static_cast<int64_t>(u) * step < t && tok[u] >= v0 && tok[u] < v1;
+                slot[u] = in ? index_take(ix, b, tok[u]) : kIndexSlots;
+            }
+#pragma unroll
+            for (int u = 0; u < kBuildLoads; ++u) index_put(ix, b, tok[u], slot[u], q0 + static_cast<int64_t>(u) * step);
+        }
+    }
+    if (bad) atomicOr(ix.flags + b, 1);
+    if (S > 1) {
+        cluster_arrive();
+        cluster_wait();
+    } else {
+        __syncthreads();
+    }
+    if (rank != 0 || tid != 0) return;
+    const bool bad_token = __ldcg(ix.flags + b) != 0;
+    ix.ilen[b] = (!valid || bad_token) ? -1 : static_cast<int32_t>(L >= 1 ? L - 1 : 0);
+    if (status && !valid) atomicOr(status + b, PLDP_ST_SEQ_LEN);
+    if (status && bad_token) atomicOr(status + b, PLDP_ST_TOKEN_RANGE);
 }
 
 // Byte offsets of the index parts (ilen, flags, entries, the drafting calls' scratch),
@@ -1620,17 +1669,16 @@ extern "C" PLDP_API pldp_status pldp_index_build(const int32_t* ids, int64_t ids
     if (index_bytes < need || !aligned16(index))
         return fail(PLDP_ERR_INVALID_ARG, "index_build: index needs %zu bytes, 16-byte aligned", need);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t e = cudaMemsetAsync(index, 0, need, s);
-    if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "index_build: clearing the index: %s", cudaGetErrorString(e));
     const IndexView ix = index_view(index, B, V);
-    int64_t chunks = (T_cap + 8191) / 8192;
-    if (chunks < 1) chunks = 1;
-    if (chunks > 65535) chunks = 65535;
-    e = launch_pdl(index_build_kernel, dim3(static_cast<unsigned>(chunks), static_cast<unsigned>(B)), dim3(kThreads), 0,
-                   s, 0, ids, ids_stride, seq_len, T_cap, ix);
-    if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "index_build: launch failed: %s", cudaGetErrorString(e));
-    e = launch_pdl(index_finish_kernel, dim3(static_cast<unsigned>((B + 255) / 256)), dim3(256), 0, s, 0, seq_len, B,
-                   T_cap, ix, status);
+    // a cluster of 8 where its CTAs have a few entries or positions a thread
+    const int64_t work = T_cap > V ? T_cap : V;
+    int64_t S = work / (4 * kBuildThreads);
+    S = S < 1 ? 1 : (S > kScanMaxCluster ? kScanMaxCluster : S);
+    const int64_t at_once = resident_blocks(reinterpret_cast<const void*>(&index_build_kernel), kBuildThreads, 0) / S;
+    const int64_t tokens = B > at_once ? kBuildTokens : V;
+    const cudaError_t e = launch_pdl(index_build_kernel, dim3(static_cast<unsigned>(B * S)), dim3(kBuildThreads), 0, s,
+                                     S > 1 ? static_cast<int>(S) : 0, ids, ids_stride, seq_len, B, T_cap, ix, status,
+                                     static_cast<int>(S), tokens);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "index_build: launch failed: %s", cudaGetErrorString(e));
     return PLDP_OK;
 }

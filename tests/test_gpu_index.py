@@ -150,3 +150,38 @@ def test_indexed_decode_loop(lib):
     ids, gt = host(loop.ids), loop.gt_host
     for b in range(B):
         assert np.array_equal(ids[b, :L[b]], gt[b, :L[b]]), b
+
+
+# the index built over memory that holds anything: one CTA a sequence and a cluster, one
+# pass over the vocabulary and several (more sequences than clusters at once), entries that
+# fill and overflow, invalid lengths and tokens out of range
+@pytest.mark.parametrize("B,T,V", [(3, 700, 40), (2, 5000, 9000), (60, 9000, 70001), (45, 300, 40000)])
+def test_build_over_garbage(lib, B, T, V):
+    rng = np.random.default_rng(B + V)
+    ids = (rng.zipf(1.3, size=(B, T)) % V).astype(np.int32)
+    lens = rng.integers(0, T + 1, size=B).astype(np.int32)
+    lens[0], lens[1] = T, T + 1                                      # the second invalid
+    if B > 2:
+        ids[2, 5], lens[2] = V, 50                                   # a token it cannot hold
+    size = pk.pldp_index_size(B, V)
+    index = torch.randint(0, 256, (size,), dtype=torch.uint8, device=DEV)
+    st = torch.zeros(B, dtype=torch.int32, device=DEV)
+    pk.pldp_index_build(i32(ids), i32(lens), V, index, status=st)
+    want = np.maximum(lens - 1, 0)
+    want[1] = -1
+    if B > 2:
+        want[2] = -1
+    assert np.array_equal(_ilen(index, B), want)
+    assert host(st)[1] == pk.PLDP_ST_SEQ_LEN and (B < 3 or host(st)[2] == pk.PLDP_ST_TOKEN_RANGE)
+    off = 2 * ((4 * B + 255) // 256 * 256)
+    e = host(index[off:off + B * V * 64].view(torch.int32)).reshape(B, V, 16)
+    for b in range(B):
+        x = ids[b, :max(int(lens[b]) - 1, 0)] if lens[b] <= T else ids[b, :0]
+        x = np.where((x >= 0) & (x < V), x, -1)
+        assert np.array_equal(e[b, :, 0], np.bincount(x[x >= 0], minlength=V)), b
+        for v in np.unique(x[x >= 0]):
+            at = np.nonzero(x == v)[0]
+            if at.size <= 15:
+                assert np.array_equal(np.sort(e[b, v, 1:1 + at.size]), at), (b, v)
+            else:
+                assert np.isin(e[b, v, 1:], at).all(), (b, v)
