@@ -302,8 +302,9 @@ __device__ __forceinline__ float sum_shares(const float (&x)[kWarps]) {
 // results (in every lane) those of cta_score bit for bit: lane l forms the partial sums
 // of the CTA's threads l, 32 + l, ..., 224 + l in eight accumulators, each in that
 // thread's order, and they are reduced over the lanes and then over the eight in the
-// CTA's order.  Sixteen 16-byte loads of the row are in flight per lane (8 KB a warp);
-// the query row is read through L1, which the CTA's warps share.
+// CTA's order.  Eight 16-byte loads of the row are in flight per lane (sixteen measured
+// 0.5-1.5 us more per launch); the query row is read through L1, which the CTA's warps
+// share.
 template <typename TH>
 __device__ __forceinline__ void warp_score(const DraftParams& p, int b, int64_t j, int64_t t, float& dot, float& na,
                                            float& s_a) {
@@ -330,7 +331,7 @@ __device__ __forceinline__ void warp_score(const DraftParams& p, int b, int64_t 
     for (int w = 0; w < kEarly; ++w) av[w] = attn(32 * w + lane);
     if constexpr (HAS_H) {
         if (h_ok) {                                               // warp-uniform
-            constexpr int E = 16 / sizeof(TH), U = 2 * kWarps;
+            constexpr int E = 16 / sizeof(TH), U = kWarps;
             const TH* hb = static_cast<const TH*>(p.H) + static_cast<int64_t>(b) * p.h_seq_stride;
             const uint4* qrow = reinterpret_cast<const uint4*>(hb + (t - 1) * p.d);
             const TH* arow = hb + (j - 1) * p.d;
@@ -446,15 +447,20 @@ __device__ __forceinline__ void write_counts(const DraftParams& p, int b, int ns
 // over the whole GPU: the deferred candidates of the batch are cut into units of a few
 // per warp, about one unit per CTA, whatever sequences they belong to.  A unit's CTA
 // scores a candidate per warp at a time and adds its best keys to the sequence's slot;
-// the CTA that completes a sequence writes its choices and draft.  Nothing waits: the
-// last CTA out clears the slots.
+// the CTA that completes a sequence writes its choices and draft.  Nothing waits.
 //
-// What bounds it: the candidates' hidden rows (8 KB each at d = 4096), random reads of
-// HBM.  One CTA scores about 25-40 GB/s of them, so the hundreds of candidates of a few
-// sequences took 100-400 us of a drafting launch (up to 8 CTAs a sequence, one in the
-// indexed kernels) while the other SMs were idle.  Drafting batch 128 x 32k Zipf tokens:
-// 125-190 -> 32 us; index build + 8 fused steps of it: 6083 -> 1400 us.  A batch without
-// deferred sequences pays the empty launch, about 2 us.
+// What bounds it: latency, about 9 us from the drafting kernel's end to its own with one
+// candidate per warp (the slots, the candidates, their rows, the keys and the count, the
+// draft: a round trip to memory each), then the translation of the rows' addresses: they
+// are random 8 KB rows of a tensor of tens of GB, and the first half of one arrives 4-8 us
+// after its load, about 500 rows/us in all (23 us for the 7154 candidates of a fused step
+// of batch 128 x 32k).  Sending the rows to L2 while the drafting kernel ends, loading the
+// next candidate's row while one is summed, and scoring with whole CTAs gave nothing.
+//
+// The same work by the sequences' own CTAs (up to 8, one in the indexed kernels) took
+// 100-400 us of a drafting launch on Zipf contexts while the other SMs were idle: drafting
+// batch 128 x 32k 125-190 -> 30 us; index build + 8 fused steps of it 6083 -> 1400 us.  A
+// batch without deferred sequences pays the empty launch, 1-2 us.
 template <typename TH>
 __global__ void __launch_bounds__(kThreads, 2) score_deferred_kernel(const DraftParams p, int B) {
     constexpr bool HAS_H = !std::is_same<TH, NoHidden>::value;
@@ -467,22 +473,42 @@ __global__ void __launch_bounds__(kThreads, 2) score_deferred_kernel(const Draft
     pdl_enter();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     DeferSlot* slots = p.defer;
-    int mine = 0;
-    for (int b = tid; b < B; b += kThreads) mine += static_cast<int>(__ldcg(&slots[b].pending));
-    const int ws = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(mine)));
-    if (lane == 0) wsum[warp] = ws;
-    __syncthreads();
-    int64_t all = 0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) all += wsum[w];
-    if (all == 0) return;
     const int G = static_cast<int>(gridDim.x);
-    const int64_t per = (all + static_cast<int64_t>(G) * kWarps - 1) / (static_cast<int64_t>(G) * kWarps) * kWarps;
-    const int U = per < kMaxUnit ? static_cast<int>(per) : kMaxUnit;   // a multiple of kWarps
+    const int n0 = tid < B ? static_cast<int>(__ldcg(&slots[tid].pending)) : 0;   // the first tile's
+    unsigned sum = n0, seqs = n0 > 0;
+    for (int b = tid + kThreads; b < B; b += kThreads) {
+        const unsigned n = __ldcg(&slots[b].pending);
+        sum += n;
+        seqs += n > 0;
+    }
+    sum = __reduce_add_sync(0xFFFFFFFFu, sum);
+    seqs = __reduce_add_sync(0xFFFFFFFFu, seqs);
+    if (lane == 0) {
+        wsum[warp] = static_cast<int>(sum);
+        n_of[warp] = static_cast<int>(seqs);
+    }
+    __syncthreads();
+    int64_t all = 0, heavy = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+        all += wsum[w];
+        heavy += n_of[w];
+    }
+    if (all == 0) return;
+    // The last CTA to have read every `pending` clears them on its way out: known at once
+    // when they are one tile, else after the last tile.
+    bool clears = false;
+    auto count_in = [&]() { clears = tid == 0 && atomicAdd(&slots[B].done, 1u) == static_cast<unsigned>(G - 1); };
+    if (B <= kThreads) count_in();
+    // units of U candidates, a multiple of one per warp, at most one unit per CTA where
+    // that fits (the last unit of every sequence may be short)
+    const int64_t ctas = (2 * heavy < G ? G - heavy : (G + 1) / 2) * kWarps;
+    const int64_t per = (all + ctas - 1) / ctas * kWarps;
+    const int U = per < kMaxUnit ? static_cast<int>(per) : kMaxUnit;
     int64_t unit0 = 0;                                            // units of the tiles before
     for (int b0 = 0; b0 < B; b0 += kThreads) {
         // the tile's units: an exclusive scan over its sequences
-        const int n = b0 + tid < B ? static_cast<int>(__ldcg(&slots[b0 + tid].pending)) : 0;
+        const int n = b0 == 0 ? n0 : b0 + tid < B ? static_cast<int>(__ldcg(&slots[b0 + tid].pending)) : 0;
         const int units = (n + U - 1) / U;
         int incl = units;
 #pragma unroll
@@ -582,14 +608,11 @@ __global__ void __launch_bounds__(kThreads, 2) score_deferred_kernel(const Draft
         }
         unit0 += total;
     }
-    // the last CTA out clears `pending`, which the others read at their start
-    __syncthreads();
-    if (tid == 0) {
-        __threadfence();
-        last = atomicAdd(&slots[B].done, 1u) == static_cast<unsigned>(G - 1);
+    if (B > kThreads) {
+        __syncthreads();                                          // this CTA's reads are done
+        count_in();
     }
-    __syncthreads();
-    if (!last) return;
+    if (!__syncthreads_or(clears)) return;
     for (int b = tid; b < B; b += kThreads) slots[b].pending = 0;
     if (tid == 0) slots[B].done = 0;
 }
