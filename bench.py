@@ -253,10 +253,10 @@ class Path:
                       if (index or self.vd) and fused else None)
         self.fused = fused
         if self.vd:
-            self.launches_per_step = 2                  # the argmax pass, then verification + next draft
+            self.launches_per_step = 3                  # the argmax pass, verification + next draft, deferred scoring
             self.kernels = ["verify_greedy_draft"]
         else:
-            self.launches_per_step = 3 if fused else 6  # pldp_verify_greedy launches two kernels
+            self.launches_per_step = 4 if fused else 6  # pldp_draft_step and pldp_verify_greedy launch two each
             self.kernels = (["draft_step"] if fused else
                             ["find_candidates", "rank_hidden", "rank_attention", "extract_draft"]) + ["verify_greedy"]
 
@@ -662,7 +662,7 @@ def time_sample_draft_loop(pk, loop, path, w, flush_l2, peak, steps=64, warm=3, 
     return {"temperature": temperature, "steps": steps, "us_per_step": round(float(us.mean()), 2),
             "us_p50_p90": [round(float(np.percentile(us, 50)), 2), round(float(np.percentile(us, 90)), 2)],
             "logits_bytes": by, "logits_gbs": round(by / (us.mean() * 1e-6) / 1e9, 1),
-            "mean_accept": round(float(acc) / (steps * B), 3), "launches_per_step": 3,
+            "mean_accept": round(float(acc) / (steps * B), 3), "launches_per_step": 4,
             "timing": "CUDA events around each pldp_verify_sample_draft call, L2 flushed before each step"}
 
 

@@ -459,8 +459,8 @@ __device__ __forceinline__ void write_counts(const DraftParams& p, int b, int ns
 //
 // The same work by the sequences' own CTAs (up to 8, one in the indexed kernels) took
 // 100-400 us of a drafting launch on Zipf contexts while the other SMs were idle: drafting
-// batch 128 x 32k 125-190 -> 30 us; index build + 8 fused steps of it 6083 -> 1400 us.  A
-// batch without deferred sequences pays the empty launch, 1-2 us.
+// batch 128 x 32k 125-190 -> 30 us (28 now); index build + 8 fused steps of it 6083 -> 1400
+// us (1100 now).  A batch without deferred sequences pays the empty launch, 1-2 us.
 template <typename TH>
 __global__ void __launch_bounds__(kThreads, 2) score_deferred_kernel(const DraftParams p, int B) {
     constexpr bool HAS_H = !std::is_same<TH, NoHidden>::value;

@@ -16,10 +16,11 @@
 // What bounds it: the ids' DRAM round trips (8 vectors in flight per lane).  Match
 // lengths worked out per position cost 150 instructions per 128 positions wherever x_t
 // is frequent (drafting batch 128 x 32k Zipf tokens through the index: 34 us, 21 us with
-// masks; its scanning kernel 22 -> 17 us); before that, every occurrence walked its suffix with one dependent load
-// per token and the positions were written by a second pass with two CTA barriers per
-// 1024 positions, which took most of 1240-1490 us of a drafting launch over 32k-token
-// Zipf contexts (batch 128).  pldp_find_candidates, batch 64 x 16k, L2 flushed: 12.2 -> 8-9.6 us.
+// masks; its scanning kernel 22 -> 17 us).  Before that, every occurrence walked its
+// suffix with one dependent load per token and the positions were written by a second
+// pass with two CTA barriers per 1024 positions, which took most of 1240-1490 us of a
+// drafting launch over 32k-token Zipf contexts (batch 128).  pldp_find_candidates, batch
+// 64 x 16k, L2 flushed: 12.2 -> 8-9.6 us.
 #pragma once
 
 #include "pldp_internal.cuh"
