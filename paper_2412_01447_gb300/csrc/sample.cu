@@ -120,6 +120,11 @@ __device__ __forceinline__ float ordered_value(uint32_t o) {
 // Each lane sums its elements' weights against its own maximum m, so the
 // exponentials do not wait for the piece's maximum M (one redux over ordered
 // keys); the lane's sum is then scaled by 2^((m - M) / T log2 e) and the warp adds.
+// The difference l - m comes first and the factor after, here and in the draw: in one
+// FMA, l log2e / T - round(m log2e / T), the rounding weighs up to |m| / T 2^-24 of every
+// weight, and both products overflow where a mask holds the type's lowest value, so that
+// a lane of such elements would weigh infinity, or NaN once scaled.  The difference costs
+// 69.1 -> 69.7 us per call (batch 128 x 13 rows of 128256 bf16, L2 flushed).
 //
 // The streaming form: 16-byte loads (every piece a whole number of vectors) and
 // 32-bit unit arithmetic (fewer than 2^31 units, checked on the host; the rows and
@@ -191,8 +196,7 @@ sample_stats_vec_kernel(const T* __restrict__ logits, uint32_t V, uint32_t units
         for (int q = 0; q < kSegLoads; ++q)
             if (lane + 32u * q < nv) m = fmaxf(m, vmax(raw[q], T()));
         if (m > -INFINITY) {
-            const float mc = m * c;
-            const uint64_t c2 = pack_f32x2(c, c), mc2 = pack_f32x2(-mc, -mc);
+            const uint64_t c2 = pack_f32x2(c, c), m2 = pack_f32x2(-m, -m);
             uint64_t acc = 0;                                          // (0.f, 0.f)
 #pragma unroll
             for (int q = 0; q < kSegLoads; ++q) {
@@ -201,7 +205,7 @@ sample_stats_vec_kernel(const T* __restrict__ logits, uint32_t V, uint32_t units
                 unpack(raw[q], e, T());
 #pragma unroll
                 for (int j = 0; j < static_cast<int>(VW); j += 2) {    // element pairs, packed fp32 math
-                    const uint64_t x = fma_f32x2(pack_f32x2(e[j], e[j + 1]), c2, mc2);
+                    const uint64_t x = fma_f32x2(add_f32x2(pack_f32x2(e[j], e[j + 1]), m2), c2, 0ull);
                     acc = add_f32x2(acc, pack_f32x2(ex2_approx(lo_f32(x)), ex2_approx(hi_f32(x))));
                 }
             }
@@ -245,10 +249,9 @@ sample_stats_kernel(const T* __restrict__ logits, int64_t V, int64_t rows, int n
             m = fmaxf(m, x[q]);
         }
         if (m > -INFINITY) {
-            const float mc = m * c;
 #pragma unroll
             for (int q = 0; q < PER; ++q)
-                if (x[q] > -INFINITY) sum += ex2_approx(fmaf(x[q], c, -mc));
+                if (x[q] > -INFINITY) sum += ex2_approx((x[q] - m) * c);
         }
         const float M = ordered_value(__reduce_max_sync(0xFFFFFFFFu, ordered_key(m)));
         if (sum > 0.f) sum *= ex2_approx((m - M) * c);
@@ -264,10 +267,10 @@ sample_stats_kernel(const T* __restrict__ logits, int64_t V, int64_t rows, int n
 }
 
 // Weight of piece k of a row against the row max M (0 for an empty piece).
-__device__ __forceinline__ float piece_weight(const float2* st, int k, int npieces, float Mc, float c) {
+__device__ __forceinline__ float piece_weight(const float2* st, int k, int npieces, float M, float c) {
     if (k >= npieces) return 0.f;
     const float2 s = __ldcg(st + k);
-    return s.x > -INFINITY ? s.y * ex2_approx(fmaf(s.x, c, -Mc)) : 0.f;
+    return s.x > -INFINITY ? s.y * ex2_approx((s.x - M) * c) : 0.f;
 }
 
 __device__ __forceinline__ float warp_incl_scan(float v, int lane) {
@@ -304,11 +307,11 @@ __device__ __forceinline__ PiecePick pick_piece(const float2* __restrict__ st, i
             sv[q] = k < np ? __ldcg(st + k) : make_float2(-INFINITY, 0.f);
             m = fmaxf(m, sv[q].x);
         }
-        const float Mc = warp_max_f(m) * c;
+        const float M = warp_max_f(m);
         float wv[kStatRegs], incl[kStatRegs], total = 0.f;
 #pragma unroll
         for (int q = 0; q < kStatRegs; ++q) {
-            wv[q] = sv[q].x > -INFINITY ? sv[q].y * ex2_approx(fmaf(sv[q].x, c, -Mc)) : 0.f;
+            wv[q] = sv[q].x > -INFINITY ? sv[q].y * ex2_approx((sv[q].x - M) * c) : 0.f;
             incl[q] = warp_incl_scan(wv[q], lane);
             total += __shfl_sync(0xFFFFFFFFu, incl[q], 31);
         }
@@ -329,16 +332,16 @@ __device__ __forceinline__ PiecePick pick_piece(const float2* __restrict__ st, i
     } else {
         float m = -INFINITY;
         for (int k = lane; k < np; k += 32) m = fmaxf(m, __ldcg(st + k).x);
-        const float Mc = warp_max_f(m) * c;
+        const float M = warp_max_f(m);
         float total = 0.f;
         for (int k0 = 0; k0 < np; k0 += 32) {
-            const float incl = warp_incl_scan(piece_weight(st, k0 + lane, np, Mc, c), lane);
+            const float incl = warp_incl_scan(piece_weight(st, k0 + lane, np, M, c), lane);
             total += __shfl_sync(0xFFFFFFFFu, incl, 31);
         }
         pk.target = u * total;
         float run = 0.f;
         for (int k0 = 0; k0 < np && pk.k < 0; k0 += 32) {
-            const float wv = piece_weight(st, k0 + lane, np, Mc, c);
+            const float wv = piece_weight(st, k0 + lane, np, M, c);
             const float incl = warp_incl_scan(wv, lane);
             const unsigned hit = __ballot_sync(0xFFFFFFFFu, run + incl > pk.target && k0 + lane < np);
             if (hit) {
@@ -383,7 +386,6 @@ __device__ int sample_row(const T* __restrict__ logits, const SampleArgs& a, int
     const int64_t e0 = static_cast<int64_t>(ks) * a.P - (RD == Rows::kRagged ? row_head<T>(r, V) : 0);   // may be negative
     const int64_t n = (V - e0 < a.P) ? V - e0 : a.P;
     const T* piece = logits + r * V + e0;
-    const float Mkc = pk.Mk * a.c;
     float x[E];
     if constexpr (RD != Rows::kElements) {
         constexpr int VW = 16 / static_cast<int>(sizeof(T));
@@ -411,7 +413,7 @@ __device__ int sample_row(const T* __restrict__ logits, const SampleArgs& a, int
     }
     float ls = 0.f;
 #pragma unroll
-    for (int j = 0; j < E; ++j) ls += x[j] > -INFINITY ? ex2_approx(fmaf(x[j], a.c, -Mkc)) : 0.f;
+    for (int j = 0; j < E; ++j) ls += x[j] > -INFINITY ? ex2_approx((x[j] - pk.Mk) * a.c) : 0.f;
     const float incl = warp_incl_scan(ls, lane);
     const float tot = __shfl_sync(0xFFFFFFFFu, incl, 31);
     const float tgt = f * tot;
@@ -426,7 +428,7 @@ __device__ int sample_row(const T* __restrict__ logits, const SampleArgs& a, int
         int last = -1;
 #pragma unroll
         for (int j = 0; j < E; ++j) {
-            const float wv = x[j] > -INFINITY ? ex2_approx(fmaf(x[j], a.c, -Mkc)) : 0.f;
+            const float wv = x[j] > -INFINITY ? ex2_approx((x[j] - pk.Mk) * a.c) : 0.f;
             if (wv > 0.f) last = j;
             acc += wv;
             if (y < 0 && acc > tgt) y = j;

@@ -68,3 +68,29 @@ def test_sampling(lib, V, dtype, T):
     assert len(diff) <= 2, diff
     for b, i in diff:
         assert _valid_draw(l64[b, i], T, float(u[b, i]), int(ys[b, i])), (b, i, ys[b, i], o[b, i])
+
+
+# masks that hold the type's lowest value or a large one: whole rows, whole 2 KB pieces and lanes of them;
+# whole vectors, cut rows and unaligned (element) loads
+@pytest.mark.parametrize("V,dtype,off", [(4096, torch.bfloat16, 0), (4097, torch.bfloat16, 0), (4096, torch.float32, 0),
+                                         (4097, torch.float32, 0), (4097, torch.bfloat16, 1)])
+@pytest.mark.parametrize("T", [0.3, 1.0, 2.0])
+@pytest.mark.parametrize("lowest", [None, -1e9, -1e4])
+def test_sampling_masked(lib, V, dtype, off, T, lowest):
+    B, K = 3, 7
+    gen = torch.Generator(device=DEV).manual_seed(V)
+    logits = torch.empty(B * (K + 1) * V + off, dtype=dtype, device=DEV)[off:].view(B, K + 1, V)
+    logits.copy_(torch.randn((B, K + 1, V), generator=gen, device=DEV) * 2)
+    low = lowest if lowest is not None else torch.finfo(dtype).min
+    logits[:, 0] = low
+    logits[:, 1, :3000] = low                            # pieces without weight before the row's
+    logits[:, 2, 100:] = low
+    logits[:, 3, 1:] = low                               # one token left
+    logits[:, 4][torch.rand((B, V), generator=gen, device=DEV) < 0.9] = low
+    u = torch.rand((B, K + 1), generator=gen, device=DEV)
+    draft, dlen = torch.zeros((B, K), dtype=torch.int32, device=DEV), torch.zeros(B, dtype=torch.int32, device=DEV)
+    _, ys, _ = _run(logits, u, draft, dlen, T)
+    o = oracle.verify_sample(host(logits), host(u), host(draft), host(dlen), T)["sampled"]
+    l64 = _f64(logits)
+    for b, i in np.argwhere(ys != o):
+        assert _valid_draw(l64[b, i], T, float(u[b, i]), int(ys[b, i])), (b, i, ys[b, i], o[b, i])
