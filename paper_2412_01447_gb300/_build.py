@@ -50,18 +50,20 @@ def up_to_date() -> bool:
     return all(os.path.getmtime(p) <= t for p in _deps())
 
 
-def build_calls(force: bool = False) -> str:
+def build_calls(force: bool = False, out: str = CALLS, extra_flags=()) -> str:
     """The binding's native checks and marshalling: a Python extension against the
-    installed torch's headers and libraries (host code only)."""
+    installed torch's headers and libraries (host code only).  A test build goes to
+    another `out` with extra compiler flags."""
     deps = [CALLS_SRC, os.path.join(INCLUDE, "pldp.h"), os.path.abspath(__file__)]
-    if not force and os.path.exists(CALLS) and all(os.path.getmtime(p) <= os.path.getmtime(CALLS) for p in deps):
-        return CALLS
+    if not force and os.path.exists(out) and all(os.path.getmtime(p) <= os.path.getmtime(out) for p in deps):
+        return out
     import torch
     root = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(nvcc())))
-    tmp = CALLS + f".tmp{os.getpid()}"
+    os.makedirs(os.path.dirname(out), exist_ok=True)
+    tmp = out + f".tmp{os.getpid()}"
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *extra_flags,
            "-I", INCLUDE, "-I", os.path.join(root, "include"),
            "-I", os.path.join(root, "include", "torch", "csrc", "api", "include"),
            "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include"), CALLS_SRC, "-o", tmp,
@@ -69,8 +71,8 @@ def build_calls(force: bool = False) -> str:
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"building the binding's native calls failed:\n{r.stdout}\n{r.stderr}")
-    os.replace(tmp, CALLS)
-    return CALLS
+    os.replace(tmp, out)
+    return out
 
 
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:

@@ -42,6 +42,12 @@ struct Library {
     decltype(&pldp_top_heads) top_heads;
 } lib;
 
+#ifdef PLDP_TEST_ANY_DEVICE
+constexpr bool kAnyDevice = true;    // test build: host tensors pass, so that the checks run without a GPU
+#else
+constexpr bool kAnyDevice = false;
+#endif
+
 // Reads arguments; `ok` goes false at the first one that is not what the call wants.
 struct Args {
     bool ok = true;
@@ -57,7 +63,7 @@ struct Args {
             return nullptr;
         }
         const at::Tensor& t = THPVariable_Unpack(o);
-        if (!t.defined() || !t.is_cuda()) {
+        if (!t.defined() || !(kAnyDevice || t.is_cuda())) {
             ok = false;
             return nullptr;
         }
@@ -178,6 +184,15 @@ struct Args {
     }
 };
 
+// The interpreter's lock given up, and taken back however the scope is left.
+struct Unlocked {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+
+// Makes the library's call without the interpreter's lock.  `call` holds values only:
+// asking a tensor anything may raise (data_ptr() does for one without storage), and
+// belongs to the checks before it.
 template <typename F>
 PyObject* finish(const Args& a, F call) {
     if (!a.ok) {
@@ -185,14 +200,16 @@ PyObject* finish(const Args& a, F call) {
         Py_RETURN_NONE;
     }
     pldp_status rc;
-    Py_BEGIN_ALLOW_THREADS
-    rc = call();
-    Py_END_ALLOW_THREADS
+    {
+        const Unlocked unlocked;
+        rc = call();
+    }
     return PyLong_FromLong(rc);
 }
 
 #define PLDP_CALL(name) PyObject* name(PyObject*, PyObject* const* v, Py_ssize_t n) noexcept
-// An exception of the tensor library counts as a check that did not pass.
+// An exception of the tensor library counts as a check that did not pass; the
+// interpreter's lock is held wherever one can arise (see finish).
 #define PLDP_BEGIN(count)              \
     if (n != (count)) Py_RETURN_NONE;  \
     try {                              \
@@ -227,7 +244,8 @@ PLDP_CALL(rank_hidden) {
     PLDP_BEGIN(10)
     const at::Tensor* H = a.hidden(v[0]);
     if (!H) Py_RETURN_NONE;
-    const int64_t B = H->size(0);
+    const void* h = H->data_ptr();
+    const int64_t B = H->size(0), T_cap = H->size(1), d = H->size(2), stride = H->stride(0);
     const pldp_dtype code = a.code(H);
     const int C = a.cols(v[2]);
     const int32_t* L = a.ints(v[1], B);
@@ -241,8 +259,7 @@ PLDP_CALL(rank_hidden) {
     void* s = a.stream(v[9]);
     if (B > INT32_MAX) a.ok = false;
     return finish(a, [&] {
-        return lib.rank_hidden(H->data_ptr(), code, H->size(2), H->stride(0), L, static_cast<int>(B), H->size(1), cand,
-                               cnt, C, thr, sc, best, bs, st, s);
+        return lib.rank_hidden(h, code, d, stride, L, static_cast<int>(B), T_cap, cand, cnt, C, thr, sc, best, bs, st, s);
     });
     PLDP_END
 }
@@ -252,7 +269,9 @@ PLDP_CALL(rank_attention) {
     PLDP_BEGIN(11)
     const at::Tensor* A = a.dims3(v[0]);
     if (!A) Py_RETURN_NONE;
-    const int64_t B = A->size(0);
+    const void* rows = A->data_ptr();
+    const int64_t B = A->size(0), R = A->size(1), T_cap = A->size(2);
+    const int64_t row_stride = A->stride(1), key_stride = A->stride(2), seq_stride = A->stride(0);
     const pldp_dtype code = a.code(A);
     const int C = a.cols(v[2]);
     const int32_t* L = a.ints(v[1], B);
@@ -260,17 +279,17 @@ PLDP_CALL(rank_attention) {
     const int32_t* cnt = a.ints(v[3], B);
     int32_t* best = a.ints(v[4], B);
     const int32_t* ri = a.ints(v[5], -1, true);
-    const int64_t n_sel = ri ? THPVariable_Unpack(v[5]).numel() : A->size(1);
+    const int64_t n_sel = ri ? THPVariable_Unpack(v[5]).numel() : R;
     const int agg = static_cast<int>(a.integer(v[6]));
     float* sc = a.floats(v[7], B * C, true);
     float* bs = a.floats(v[8], B, true);
     uint32_t* st = a.words(v[9], B);
     void* s = a.stream(v[10]);
-    if (B > INT32_MAX || A->size(1) > INT32_MAX || n_sel > INT32_MAX || (v[5] != Py_None && !ri)) a.ok = false;
+    if (B > INT32_MAX || R > INT32_MAX || n_sel > INT32_MAX || (v[5] != Py_None && !ri)) a.ok = false;
     return finish(a, [&] {
-        return lib.rank_attention(A->data_ptr(), code, static_cast<int>(A->size(1)), A->stride(1), A->stride(2), A->stride(0),
-                                  ri, static_cast<int>(n_sel), static_cast<pldp_agg>(agg), L, static_cast<int>(B),
-                                  A->size(2), cand, cnt, C, sc, best, bs, st, s);
+        return lib.rank_attention(rows, code, static_cast<int>(R), row_stride, key_stride, seq_stride, ri,
+                                  static_cast<int>(n_sel), static_cast<pldp_agg>(agg), L, static_cast<int>(B), T_cap, cand,
+                                  cnt, C, sc, best, bs, st, s);
     });
     PLDP_END
 }
@@ -572,7 +591,8 @@ PLDP_CALL(identify_heads) {
     PLDP_BEGIN(8)
     const at::Tensor* A = a.dims3(v[2]);
     if (!A || A->stride(2) != 1) Py_RETURN_NONE;
-    const int64_t B = A->size(0), R = A->size(1);
+    const void* rows = A->data_ptr();
+    const int64_t B = A->size(0), R = A->size(1), row_stride = A->stride(1), seq_stride = A->stride(0);
     const Args::Rows r = a.rows(v[0], B, nullptr);
     if (A->size(2) < r.T_cap || B > INT32_MAX || R > INT32_MAX) a.ok = false;
     const pldp_dtype code = a.code(A);
@@ -583,8 +603,8 @@ PLDP_CALL(identify_heads) {
     uint32_t* st = a.words(v[6], B);
     void* s = a.stream(v[7]);
     return finish(a, [&] {
-        return lib.identify_heads(r.p, r.stride, pos, static_cast<int>(B), r.T_cap, ms, A->data_ptr(), code,
-                                  static_cast<int>(R), A->stride(1), A->stride(0), counts, rs, st, s);
+        return lib.identify_heads(r.p, r.stride, pos, static_cast<int>(B), r.T_cap, ms, rows, code, static_cast<int>(R),
+                                  row_stride, seq_stride, counts, rs, st, s);
     });
     PLDP_END
 }

@@ -1,10 +1,15 @@
 """The binding's native checks (csrc/host_calls.cpp) against the Python ones: the same
 calls are made, with the same results, and what a check refuses is refused the same way."""
+import os
+import subprocess
+import sys
+
 import pytest
 import torch
 
 import paper_2412_01447_gb300 as pk
 import workloads as wl
+from paper_2412_01447_gb300 import _build
 from tests._parity import Buffers, snapshot
 
 DEV = "cuda"
@@ -22,6 +27,51 @@ def test_nothing_is_taken_off_the_device():
     assert c.verify_greedy(None, x, y, y, y, y, None, None, None, None, None, None, None) is None
     with pytest.raises(ValueError):
         c.bind((1, 2))
+
+
+@pytest.fixture(scope="session")
+def any_device():
+    """The native checks built without the device check, so that host tensors reach the
+    rest of them (bound to recorders here, never to the library)."""
+    pk.build()
+    pk._load()
+    return _build.build_calls(out=os.path.join(_build.BUILD_DIR, "any_device", "_pldp_calls.so"),
+                              extra_flags=["-DPLDP_TEST_ANY_DEVICE"])
+
+
+VMAP = """
+import ctypes, importlib.util, sys
+import torch
+spec = importlib.util.spec_from_file_location("_pldp_calls", sys.argv[1])
+c = importlib.util.module_from_spec(spec)
+spec.loader.exec_module(c)
+made = []
+@ctypes.CFUNCTYPE(ctypes.c_int)
+def call():
+    made.append(1)
+    return 0
+c.bind((ctypes.cast(call, ctypes.c_void_p).value,) * 12)
+i = lambda *s: torch.zeros(s, dtype=torch.int32)
+B, C, T = 2, 3, 16
+calls = [lambda x: c.rank_hidden(x, i(B), i(B, C), i(B), i(B), None, None, 0.0, None, 0),
+         lambda x: c.rank_attention(x, i(B), i(B, C), i(B), i(B), None, 0, None, None, None, 0),
+         lambda x: c.identify_heads(i(B, T), i(B), x, i(T), 8, None, None, 0),
+         lambda x: c.verify_greedy(x, i(B, T - 1), i(B), i(B), i(B), i(64), None, None, None, None, None, None, 0)]
+for f in calls:
+    assert f(torch.zeros(B, T, T)) == 0                  # a plain tensor: the call is made
+    n, got = len(made), []
+    torch.vmap(lambda x: (got.append(f(x)), x)[1])(torch.zeros(2, B, T, T))
+    assert got == [None] and len(made) == n, got         # one without storage: left to Python
+print("left to python")
+"""
+
+
+def test_a_tensor_without_storage_is_left_to_python(any_device):
+    """torch.vmap hands a function tensors that pass every check of type, shape and
+    strides and whose data pointer raises: in a child process, since that once raised
+    without the interpreter's lock."""
+    r = subprocess.run([sys.executable, "-c", VMAP, any_device], capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0 and "left to python" in r.stdout, (r.returncode, r.stdout, r.stderr[-2000:])
 
 
 def _steps(buf, inp, w, index, calls):
