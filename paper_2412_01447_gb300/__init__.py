@@ -33,6 +33,7 @@ import ctypes
 import importlib.util
 import os
 import threading
+import warnings
 
 import torch
 
@@ -149,12 +150,18 @@ def _load_calls(lib):
     call's arguments, makes its checks and returns the library's status, or None when a
     check does not pass or an argument is of a kind it does not handle; the Python that
     follows then does the same and words the error."""
-    if not os.path.exists(_build.CALLS):
+    path = _build.calls_path()
+    if not os.path.exists(path):
         return None
-    spec = importlib.util.spec_from_file_location("_pldp_calls", _build.CALLS)
-    m = importlib.util.module_from_spec(spec)
-    spec.loader.exec_module(m)
-    m.bind(tuple(ctypes.cast(getattr(lib, f), ctypes.c_void_p).value for f in _CALLS))
+    try:
+        spec = importlib.util.spec_from_file_location("_pldp_calls", path)
+        m = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(m)
+        m.bind(tuple(ctypes.cast(getattr(lib, f), ctypes.c_void_p).value for f in _CALLS))
+    except Exception as e:                               # the Python below makes every call by itself
+        warnings.warn(f"{os.path.basename(path)} does not load, the binding's calls go through ctypes: {e}",
+                      RuntimeWarning, stacklevel=2)
+        return None
     return m
 
 

@@ -12,13 +12,13 @@ import os
 import shutil
 import subprocess
 import sysconfig
+import warnings
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(PKG, "libpldp.so")
-CALLS = os.path.join(PKG, "_pldp_calls.so")
 CALLS_SRC = os.path.join(CSRC, "host_calls.cpp")
 BUILD_DIR = os.path.join(PKG, "_build")
 
@@ -50,10 +50,20 @@ def up_to_date() -> bool:
     return all(os.path.getmtime(p) <= t for p in _deps())
 
 
-def build_calls(force: bool = False, out: str = CALLS, extra_flags=()) -> str:
+def calls_path() -> str:
+    """The binding's native calls, by the torch and the Python that they are for: the
+    extension reads tensors through accessors compiled into it, so one built against
+    another torch would read their fields in the wrong places."""
+    import torch
+    return os.path.join(PKG, f"_pldp_calls.torch{torch.__version__}-cxx{int(torch._C._GLIBCXX_USE_CXX11_ABI)}"
+                             f"{sysconfig.get_config_var('EXT_SUFFIX')}")
+
+
+def build_calls(force: bool = False, out: str | None = None, extra_flags=()) -> str:
     """The binding's native checks and marshalling: a Python extension against the
     installed torch's headers and libraries (host code only).  A test build goes to
     another `out` with extra compiler flags."""
+    out = out or calls_path()
     deps = [CALLS_SRC, os.path.join(INCLUDE, "pldp.h"), os.path.abspath(__file__)]
     if not force and os.path.exists(out) and all(os.path.getmtime(p) <= os.path.getmtime(out) for p in deps):
         return out
@@ -75,9 +85,20 @@ def build_calls(force: bool = False, out: str = CALLS, extra_flags=()) -> str:
     return out
 
 
+def _build_calls_if_possible(force: bool = False) -> None:
+    """build_calls where a C++ compiler and the headers of torch and Python are found; the
+    ctypes form of every call needs none of them."""
+    try:
+        build_calls(force)
+    except Exception as e:
+        if os.path.exists(calls_path()):
+            os.remove(calls_path())                   # stale: of another state of the sources
+        warnings.warn(f"the binding's calls go through ctypes: {e}", RuntimeWarning, stacklevel=2)
+
+
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     if not force and up_to_date():
-        build_calls()
+        _build_calls_if_possible()
         return LIB
     os.makedirs(BUILD_DIR, exist_ok=True)
     cc = nvcc()
@@ -94,7 +115,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
         return obj
 
     with cf.ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 1)) as ex:
-        calls = ex.submit(build_calls, force)
+        calls = ex.submit(_build_calls_if_possible, force)
         objs = list(ex.map(compile_one, sources()))
         calls.result()
     tmp = LIB + f".tmp{os.getpid()}"

@@ -39,6 +39,38 @@ def any_device():
                               extra_flags=["-DPLDP_TEST_ANY_DEVICE"])
 
 
+def test_a_build_belongs_to_its_torch_and_python(monkeypatch):
+    """The extension of another torch or Python is not taken for this one's."""
+    mine = _build.calls_path()
+    monkeypatch.setattr(torch, "__version__", "0.0.0+other")
+    assert _build.calls_path() != mine
+    monkeypatch.undo()
+    monkeypatch.setattr(_build.sysconfig, "get_config_var", lambda name: ".cpython-00-other.so")
+    assert _build.calls_path() != mine
+
+
+def test_the_library_does_not_need_the_extension(monkeypatch, tmp_path):
+    """Without a C++ compiler the library is built and linked all the same and an extension
+    of older sources goes; one that does not load is left out."""
+    pk.build()
+    path = tmp_path / "_pldp_calls.so"
+    monkeypatch.setattr(_build, "calls_path", lambda: str(path))
+    path.write_bytes(b"not a library")
+    lib = pk._load()
+    with pytest.warns(RuntimeWarning, match="ctypes"):
+        assert pk._load_calls(lib) is None
+    monkeypatch.setenv("CXX", str(tmp_path / "no-such-compiler"))
+    os.utime(path, (1, 1))
+    with pytest.warns(RuntimeWarning, match="ctypes"):
+        _build.build()
+    assert not path.exists() and pk._load_calls(lib) is None
+    monkeypatch.setattr(_build, "LIB", str(tmp_path / "libpldp.so"))
+    monkeypatch.setattr(_build, "BUILD_DIR", str(tmp_path / "_build"))
+    monkeypatch.setattr(_build, "sources", lambda: [os.path.join(_build.CSRC, "abi.cu")])
+    with pytest.warns(RuntimeWarning, match="ctypes"):
+        assert os.path.exists(_build.build())
+
+
 VMAP = """
 import ctypes, importlib.util, sys
 import torch
