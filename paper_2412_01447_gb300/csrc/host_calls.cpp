@@ -170,6 +170,7 @@ struct Args {
         if (PyLong_CheckExact(o)) {
             void* s = PyLong_AsVoidPtr(o);
             if (s != nullptr || !PyErr_Occurred()) return s;
+            PyErr_Clear();                                     // out of range: Python's to take or to refuse
         }
         ok = false;                                            // a stream object, which Python unwraps
         return nullptr;

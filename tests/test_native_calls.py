@@ -1,9 +1,14 @@
 """The binding's native checks (csrc/host_calls.cpp) against the Python ones: the same
 calls are made, with the same results, and what a check refuses is refused the same way."""
+import ctypes
+import importlib.util
+import inspect
 import os
 import subprocess
 import sys
+import types
 
+import numpy as np
 import pytest
 import torch
 
@@ -104,6 +109,142 @@ def test_a_tensor_without_storage_is_left_to_python(any_device):
     without the interpreter's lock."""
     r = subprocess.run([sys.executable, "-c", VMAP, any_device], capture_output=True, text=True, timeout=600)
     assert r.returncode == 0 and "left to python" in r.stdout, (r.returncode, r.stdout, r.stderr[-2000:])
+
+
+class Recorder:
+    """The library's entry points, each writing down the arguments it is called with."""
+
+    def __init__(self, lib):
+        self.made, self.rc, self.fns = [], 0, {}
+        for f in pk._CALLS:
+            self.fns[f] = ctypes.CFUNCTYPE(ctypes.c_int, *getattr(lib, f).argtypes)(self._entry(f))
+        self.addresses = tuple(ctypes.cast(self.fns[f], ctypes.c_void_p).value for f in pk._CALLS)
+
+    def _entry(self, name):
+        def entry(*args):
+            self.made.append((name, *(bytes(a.contents) if hasattr(a, "contents") else repr(a) for a in args)))
+            return self.rc
+        return entry
+
+    def pldp_last_error(self):
+        return b"refused"
+
+    def __getattr__(self, name):
+        return self.fns[name]
+
+
+B, C, K, V, T, D, R = 3, 5, 4, 16, 40, 8, 6
+
+
+def _i(*shape):
+    return torch.zeros(shape, dtype=torch.int32)
+
+
+def _f(*shape, dtype=torch.float32):
+    return torch.zeros(shape, dtype=dtype)
+
+
+def _call_arguments():
+    """A call of every function with all of its arguments, and the same without the optional ones."""
+    H, A = _f(B, T, D, dtype=torch.bfloat16), _f(B, R, T)
+    lists = dict(cand_pos=_i(B, C), cand_count=_i(B))
+    ctx = dict(ids=_i(B, T + 4)[:, :T], seq_len=_i(B))
+    opt = dict(status=_i(B), stream=7)
+    find = dict(ngram_min=1, ngram_max=3, match_len=_i(B), **lists)
+    both = dict(H=H, best_h=_i(B), h_scores=_f(B, C), best_h_score=_f(B), threshold=0.25, A=A, best_a=_i(B),
+                row_idx=_i(2), agg=1, a_scores=_f(B, C), best_a_score=_f(B), draft_from="attention", status=_i(B), T_cap=T - 8)
+    ver = dict(logits=_f(B, K + 1, V, dtype=torch.bfloat16), draft=_i(B, K), draft_len=_i(B), accept_len=_i(B),
+               next_token=_i(B), workspace=_f(64))
+    app = dict(ids=ctx["ids"], seq_len=ctx["seq_len"], kv_keep_len=_i(B), T_cap=T - 8, **opt)
+    nxt = dict(next_draft=_i(B, K), next_draft_len=_i(B), index=_f(64), kv_keep_len=_i(B), stream=7, **ctx, **find, **both)
+    u = dict(uniforms=_f(B, K + 1), temperature=0.7, sampled=_i(B, K + 1))
+    full = {
+        "pldp_find_candidates": dict(**ctx, **find, **opt, T_cap=T - 8),
+        "pldp_rank_hidden": dict(H=H, seq_len=_i(B), **lists, best_pos=_i(B), scores=_f(B, C), best_score=_f(B),
+                                 threshold=0.25, **opt),
+        "pldp_rank_attention": dict(A=A.transpose(1, 2).contiguous().transpose(1, 2), seq_len=_i(B), **lists, best_pos=_i(B),
+                                    row_idx=_i(2), agg=1, scores=_f(B, C), best_score=_f(B), **opt),
+        "pldp_extract_draft": dict(**ctx, best_pos=_i(B), draft=_i(B, K), draft_len=_i(B), T_cap=T - 8, stream=7),
+        "pldp_draft_step": dict(**ctx, **find, K=K, draft=_i(B, K), draft_len=_i(B), workspace=_f(64), stream=7, index=_f(64),
+                                V=V, **both),
+        "pldp_index_build": dict(**ctx, V=V, index=_f(64), T_cap=T - 8, **opt),
+        "pldp_verify_greedy": dict(**ver, argmax=_i(B, K + 1), **app),
+        "pldp_verify_greedy_draft": dict(**ver, argmax=_i(B, K + 1), **nxt),
+        "pldp_verify_sample": dict(**ver, **u, **app),
+        "pldp_verify_sample_draft": dict(**ver, **u, **nxt),
+        "pldp_identify_heads": dict(ids=ctx["ids"], pos=_i(B), A=A, counts=_i(R), max_suffix=9, r_star=_i(B), **opt),
+        "pldp_top_heads": dict(counts=_i(R), k=2, row_idx=_i(2), stream=7),
+    }
+    assert set(full) == set(pk._CALLS)
+    needed = {f: [p.name for p in inspect.signature(getattr(pk, f)).parameters.values()
+                  if p.default is p.empty and p.kind != p.VAR_KEYWORD] for f in full}
+    plain = {f: {**{k: a[k] for k in needed[f]}, "stream": 0, **({"H": H, "best_h": a["best_h"]} if "best_h" in a else {})}
+             for f, a in full.items()}
+    return full, plain
+
+
+def _variants(x):
+    """Other things in the place of an argument: kinds, sizes, strides and ranges that a check is for."""
+    if isinstance(x, torch.Tensor):
+        yield from (None, 3, [1], x.numpy() if x.dtype != torch.bfloat16 else 1.5, x.long(), x.to(torch.float16), x.float(),
+                    x.to(torch.bfloat16), x.to(torch.uint32) if x.dtype == torch.int32 else x.double(), x[:-1], x[..., :-1],
+                    x[..., :-1].contiguous(), x.flatten(), x.unsqueeze(0), torch.stack([x, x], -1)[..., 0],
+                    torch.cat([x, x]), torch.cat([x, x], -1), torch.empty(0, dtype=x.dtype), x.new_zeros(()))
+        if x.dim() > 1:
+            yield from (x.transpose(-1, -2), x.transpose(0, 1), x[:, :-1], x[:, :-1].contiguous(), x[:, 1:], torch.cat([x, x], 1),
+                        x[:1].expand(x.shape))
+        if x.is_floating_point():
+            yield torch.nn.Parameter(x)
+    elif isinstance(x, str):
+        yield from ("hidden", "x", 0, 1, 2, True, None, np.int64(1), [])
+    else:
+        yield from (None, 0, 1, -1, 5, T, T + 1, 2**31 - 1, 2**31, -2**31, -2**31 - 1, 2**40, 2**63, -2**70, 0.0, 1.0, 1.5,
+                    float("nan"), float("-inf"), 1e300, True, "1", np.int32(2), np.float32(0.5))
+
+
+def test_native_and_python_checks_agree(any_device, monkeypatch):
+    """Every argument of every call in turn replaced by other things: the native form makes
+    the call that the Python form makes, argument for argument, or leaves it to Python.
+    Without a GPU: host tensors in both forms, the entry points replaced."""
+    spec = importlib.util.spec_from_file_location("_pldp_calls", any_device)
+    native = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(native)
+    rec = Recorder(pk._load())
+    native.bind(rec.addresses)
+    monkeypatch.setattr(pk, "_load", lambda: rec)
+    monkeypatch.setattr(torch.Tensor, "is_cuda", True, raising=False)
+
+    def outcome(f, args, calls):
+        monkeypatch.setattr(pk, "_calls", calls)
+        rec.made.clear()
+        try:
+            getattr(pk, f)(**args)
+            return list(rec.made)
+        except Exception as e:
+            return [*rec.made, type(e), str(e)]
+
+    def agree(f, args, what):
+        a, b = outcome(f, args, native), outcome(f, args, None)
+        assert a == b, (f, what, a, b)
+        return a
+
+    for arguments in _call_arguments():
+        for f, args in arguments.items():
+            taken = getattr(native, f[5:])
+            made = agree(f, args, "as it is")
+            assert len(made) == 1 and made[0][0] == f, made
+            spy = types.SimpleNamespace(**{f[5:]: lambda *a: seen.append(taken(*a)) or seen[-1]})
+            seen = []
+            outcome(f, args, spy)
+            assert seen == [0], (f, "not taken natively")
+            rec.rc = 3
+            assert agree(f, args, "refused by the library")[1] is pk.PldpError
+            rec.rc = 0
+            for name, x in args.items():
+                for i, y in enumerate(_variants(x)):
+                    agree(f, {**args, name: y}, (name, i, y))
+            agree(f, {k: v for k, v in args.items() if k not in ("best_h", "best_a", "V")}, "outputs missing")
+            agree(f, {**args, "no_such": 1}, "a keyword it does not have")
 
 
 def _steps(buf, inp, w, index, calls):
