@@ -183,9 +183,9 @@ __device__ __forceinline__ SegKeys ragged_argmax(const T* __restrict__ logits, u
         uint4 x[kSegLoads];
 #pragma unroll
         for (int u = 0; u < kSegLoads; ++u) x[u] = ld_stream16(p + s0 + lane + 32 * u);
-        float m = vmax(x[0], T());
+        float m = -INFINITY;                                   // a lane of NaNs offers this, never a NaN
 #pragma unroll
-        for (int u = 1; u < kSegLoads; ++u) m = fmaxf(m, vmax(x[u], T()));
+        for (int u = 0; u < kSegLoads; ++u) m = fmaxf(m, vmax(x[u], T()));
         const uint32_t ok = ordered_key(m);
         const uint32_t wk = __reduce_max_sync(0xFFFFFFFFu, ok);
         uint32_t idx = 0xFFFFFFFFu;
@@ -195,6 +195,7 @@ __device__ __forceinline__ SegKeys ragged_argmax(const T* __restrict__ logits, u
                 if (idx == 0xFFFFFFFFu && vmax(x[u], T()) == m) idx = rem + (lane + 32 * u) * VW + vfirst(x[u], m, T());
         }
         idx = __reduce_min_sync(0xFFFFFFFFu, idx);
+        if (wk == ordered_key(-INFINITY)) idx = rem;           // nothing above -inf: the first element
         return SegKeys{pack_ordered(wk, idx), 0ull};
     }
     const uint32_t bnd = V - rem;                              // first element of the next row, from the segment's start

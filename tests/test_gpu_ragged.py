@@ -46,6 +46,34 @@ def test_greedy(lib, V, dtype, B, K):
         assert not ws.any()
 
 
+# NaN is no maximum: whole rows, whole lanes (32 bf16 or 16 fp32 a segment) and all but a
+# few elements of a row; the streaming path against the element loads, which take one
+# element at a time
+@pytest.mark.parametrize("V,dtype", [(1025, torch.bfloat16), (5003, torch.bfloat16), (5003, torch.float32)])
+def test_greedy_nan(lib, V, dtype):
+    B, K = 6, 7
+    gen = torch.Generator(device=DEV).manual_seed(V)
+    logits = torch.randn((B, K + 1, V), generator=gen, device=DEV).to(dtype)
+    logits[0] = float("nan")
+    logits[1, :, 3:] = float("nan")
+    logits[2] = torch.where(torch.rand((K + 1, V), generator=gen, device=DEV) < 0.999, float("nan"), -3.0).to(dtype)
+    logits[3] = torch.where(torch.rand((K + 1, V), generator=gen, device=DEV) < 0.5, float("nan"), float("-inf")).to(dtype)
+    logits[4, :, : V // 2] = float("nan")
+    draft = torch.zeros((B, K), dtype=torch.int32, device=DEV)
+    dlen = torch.zeros(B, dtype=torch.int32, device=DEV)
+    shifted = torch.empty(logits.numel() + 1, dtype=dtype, device=DEV)[1:].reshape(logits.shape)   # unaligned logits
+    shifted.copy_(logits)
+    got = []
+    for lg in (logits, shifted):
+        ws = torch.zeros(pk.pldp_verify_workspace_size(B, K, V), dtype=torch.uint8, device=DEV)
+        am = torch.full((B, K + 1), -7, dtype=torch.int32, device=DEV)
+        acc, nxt = torch.zeros_like(dlen), torch.zeros_like(dlen)
+        pk.pldp_verify_greedy(lg, draft, dlen, acc, nxt, ws, argmax=am)
+        got.append(host(am))
+    assert np.array_equal(got[0], got[1])
+    assert (got[0] >= 0).all() and (got[0][0] == 0).all()
+
+
 # a last piece with and without room for the elements that a cut row start moves there
 # (1017 and 1021 of 1024, 509 and 510 of 512), rows shorter than a vector, several pieces
 @pytest.mark.parametrize("V,dtype", [(3, torch.bfloat16), (1017, torch.bfloat16), (1021, torch.bfloat16),
