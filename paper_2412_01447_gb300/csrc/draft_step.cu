@@ -104,6 +104,7 @@ struct DraftParams {
     int32_t* draft;
     int32_t* draft_len;
     uint32_t* status;
+    int B;
     struct DeferSlot* defer;   // [B + 1], all zero between calls; null: nothing is deferred
 };
 
@@ -113,9 +114,19 @@ struct DraftParams {
 struct alignas(16) DeferSlot {
     unsigned long long h, a;
     unsigned pending, done;
-    unsigned pad[2];
+    unsigned decided;          // slot B, indexed drafting: sequences decided on, and kDeferred times those left
+    unsigned pad;
 };
+constexpr unsigned kDeferred = 1u << 16;                       // (at most 65535 sequences)
 static_assert(sizeof(DeferSlot) == 32 && 2 * sizeof(DeferSlot) <= kSeqWs, "B + 1 slots fit the workspace");
+
+// One thread, once per sequence and launch of an indexed drafting kernel: whether the
+// sequence's `pending` candidates (0: none) are left to score_deferred_kernel.
+__device__ __forceinline__ void decide(const DraftParams& p, int b, unsigned pending) {
+    if (p.defer == nullptr) return;
+    if (pending != 0) p.defer[b].pending = pending;
+    atomicAdd(&p.defer[p.B].decided, pending != 0 ? 1u + kDeferred : 1u);
+}
 
 template <int NB>
 __device__ __forceinline__ float (&part_buf(float (&part)[kMaxScoreBatch][kWarps][4]))[NB][kWarps][4] {
@@ -460,8 +471,18 @@ __device__ __forceinline__ void write_counts(const DraftParams& p, int b, int ns
 // The same work by the sequences' own CTAs (up to 8, one in the indexed kernels) took
 // 100-400 us of a drafting launch on Zipf contexts while the other SMs were idle: drafting
 // batch 128 x 32k 125-190 -> 30 us (28 now); index build + 8 fused steps of it 6083 -> 1400
-// us (1100 now).  A batch without deferred sequences pays the empty launch, 1-2 us.
-template <typename TH>
+// us (1100 now).
+//
+// A batch without deferred sequences (uniform contexts, where x_t occurs a few times) pays
+// for the launch all the same, most of it the boundary between two kernels: fused step of
+// batch 128 x 32k uniform tokens 74.7 us without it, 76.5 with a grid of one CTA, 76.8 with
+// every CTA waiting for the drafting kernel and then finding nothing.  COUNTED (behind
+// indexed drafting, which counts the sequences it has decided on): when all are and none
+// is left, every CTA but the first leaves before the wait, 76.4; the first stays until the
+// drafting kernel is complete, since the stream's next work relies on this launch for that.
+// Behind the scanning kernel the counts cost as much as they gave (draft_step, 2 x 128k
+// Zipf tokens, 12.2 -> 12.4 us).
+template <typename TH, bool COUNTED>
 __global__ void __launch_bounds__(kThreads, 2) score_deferred_kernel(const DraftParams p, int B) {
     constexpr bool HAS_H = !std::is_same<TH, NoHidden>::value;
     __shared__ int n_of[kThreads];                                // deferred candidates of this tile's sequences
@@ -470,6 +491,10 @@ __global__ void __launch_bounds__(kThreads, 2) score_deferred_kernel(const Draft
     __shared__ unsigned long long wkey[2][kWarps];
     __shared__ float wnq[kWarps];
     __shared__ int last;
+    if constexpr (COUNTED) {
+        const bool none = threadIdx.x == 0 && ld_relaxed(&p.defer[B].decided) == static_cast<unsigned>(B);
+        if (__syncthreads_or(none) && blockIdx.x != 0) return;
+    }
     pdl_enter();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     DeferSlot* slots = p.defer;
@@ -494,7 +519,10 @@ __global__ void __launch_bounds__(kThreads, 2) score_deferred_kernel(const Draft
         all += wsum[w];
         heavy += n_of[w];
     }
-    if (all == 0) return;
+    if (all == 0) {
+        if (COUNTED && blockIdx.x == 0 && tid == 0) slots[B].decided = 0;
+        return;
+    }
     // The last CTA to have read every `pending` clears them on its way out: known at once
     // when they are one tile, else after the last tile.
     bool clears = false;
@@ -614,7 +642,10 @@ __global__ void __launch_bounds__(kThreads, 2) score_deferred_kernel(const Draft
     }
     if (!__syncthreads_or(clears)) return;
     for (int b = tid; b < B; b += kThreads) slots[b].pending = 0;
-    if (tid == 0) slots[B].done = 0;
+    if (tid == 0) {
+        slots[B].done = 0;
+        if (COUNTED) slots[B].decided = 0;
+    }
 }
 
 // What the rescan keeps per warp: every round's longest match and its mask (see
@@ -986,6 +1017,7 @@ __device__ __forceinline__ void index_draft(const DraftParams& p, const IndexVie
     bad = __syncthreads_or(bad) != 0;
     if (!valid) {
         no_draft<HAS_H>(p, b);
+        if (tid == 0) decide(p, b, 0);
         return;
     }
     // usable: the index covers a prefix of the context; small: what was appended fits the CTA
@@ -1137,12 +1169,11 @@ __device__ __forceinline__ void index_draft(const DraftParams& p, const IndexVie
     }
 
     const int n = spec ? nocc : (total < p.C_cap ? total : p.C_cap);
-    if (p.defer != nullptr && n > kCtaPasses * NB) {
+    const bool deferred = p.defer != nullptr && n > kCtaPasses * NB;
+    if (tid == 0) decide(p, b, deferred ? static_cast<unsigned>(n) : 0u);
+    if (deferred) {
         if (mine) index_put(ix, b, mytok, myslot, il + tid);      // the slot taken above
-        if (tid == 0) {
-            counts(nstar, total);
-            p.defer[b].pending = static_cast<unsigned>(n);
-        }
+        if (tid == 0) counts(nstar, total);
         return;
     }
     {
@@ -1409,14 +1440,14 @@ inline IndexView index_view(void* base, int B, int V) {
 // may have to leave some: then its launch is followed by score_deferred_kernel's.
 inline bool may_defer(const DraftParams& p, int64_t here) { return p.C_cap > here && p.T_cap > here; }
 
-template <typename TH>
+template <typename TH, bool COUNTED>
 pldp_status launch_deferred(const DraftParams& p, int B, cudaStream_t s, const char* what) {
-    int64_t blocks = resident_blocks(reinterpret_cast<const void*>(&score_deferred_kernel<TH>), kThreads, 0);
+    int64_t blocks = resident_blocks(reinterpret_cast<const void*>(&score_deferred_kernel<TH, COUNTED>), kThreads, 0);
     const int64_t most = p.C_cap < p.T_cap ? p.C_cap : p.T_cap;               // candidates of a sequence
     const int64_t need = (most + kWarps - 1) / kWarps * B;                    // units of one per warp
     if (blocks > need) blocks = need;
-    const cudaError_t e = launch_pdl(score_deferred_kernel<TH>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, s,
-                                     0, p, B);
+    const cudaError_t e = launch_pdl(score_deferred_kernel<TH, COUNTED>, dim3(static_cast<unsigned>(blocks)),
+                                     dim3(kThreads), 0, s, 0, p, B);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "%s: launch failed: %s", what, cudaGetErrorString(e));
     return PLDP_OK;
 }
@@ -1432,7 +1463,7 @@ pldp_status launch_t(const DraftParams& p0, int B, cudaStream_t s) {
     const cudaError_t e = launch_pdl(draft_step_kernel<TH, IVEC>, dim3(static_cast<unsigned>(B) * CL), dim3(kThreads), 0,
                                      s, CL > 1 ? CL : 0, p, CL, chunk);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "draft_step: launch failed: %s", cudaGetErrorString(e));
-    return p.defer ? launch_deferred<TH>(p, B, s, "draft_step") : PLDP_OK;
+    return p.defer ? launch_deferred<TH, false>(p, B, s, "draft_step") : PLDP_OK;
 }
 
 template <typename TH, bool IVEC>
@@ -1442,7 +1473,7 @@ pldp_status launch_index_t(const DraftParams& p0, const IndexView& ix, int B, cu
     cudaError_t e = launch_pdl(draft_index_kernel<TH, IVEC>, dim3(static_cast<unsigned>(B)), dim3(kThreads), 0, s, 0,
                                p, ix);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "draft_step (indexed): launch failed: %s", cudaGetErrorString(e));
-    return p.defer ? launch_deferred<TH>(p, B, s, "draft_step (indexed)") : PLDP_OK;
+    return p.defer ? launch_deferred<TH, true>(p, B, s, "draft_step (indexed)") : PLDP_OK;
 }
 
 template <typename TH>
@@ -1554,6 +1585,7 @@ pldp_status prepare_draft(const pldp_draft_step_args* a, const char* what, Draft
     p.draft = a->draft;
     p.draft_len = a->draft_len;
     p.status = a->status;
+    p.B = B;
     p.defer = has_ix ? nullptr : reinterpret_cast<DeferSlot*>(a->workspace);
     ivec = aligned16(a->ids) && a->ids_stride % 4 == 0 && a->T_cap % 4 == 0;
     return PLDP_OK;
@@ -1567,7 +1599,7 @@ pldp_status launch_verify_draft_t(const VerifyArgs& va, const DraftParams& p0, c
     const cudaError_t e = launch_pdl(verify_draft_kernel<TH, IVEC>, dim3(static_cast<unsigned>(B)), dim3(kThreads), 0,
                                      s, 0, va, p, ix);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "verify_draft: launch failed: %s", cudaGetErrorString(e));
-    return p.defer ? launch_deferred<TH>(p, B, s, "verify_draft") : PLDP_OK;
+    return p.defer ? launch_deferred<TH, true>(p, B, s, "verify_draft") : PLDP_OK;
 }
 
 template <typename TH>

@@ -134,6 +134,13 @@ __device__ __forceinline__ uint4 ld_stream16(const void* p) {
     return r;
 }
 
+// A word that other CTAs may be adding to.
+__device__ __forceinline__ unsigned ld_relaxed(const unsigned* p) {
+    unsigned r;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(r) : "l"(p) : "memory");
+    return r;
+}
+
 // ---------------------------------------------------------------------------
 // mbarrier + bulk async copy (global -> this CTA's shared memory)
 // ---------------------------------------------------------------------------

@@ -84,3 +84,36 @@ def test_many_candidates(lib, T, V, B, d, R, agg, dtype, ngram):
         _compare(out[-1], ids, lens, H, A, None, agg, ngram, C, K, "hidden")
     for k in ("cand", "scores_h", "scores_a", "best_h", "best_a", "draft"):
         assert np.array_equal(out[0][k], out[1][k], equal_nan=True), k
+
+
+# calls that leave some, all or none of their sequences to the deferred launch, in turn on the
+# same scratch, invalid lengths among them: every call's results are its own and the scratch
+# is left zeroed (one sequence, one tile of the deferred launch and several, grids of one wave
+# of drafting CTAs and more)
+@pytest.mark.parametrize("B,T", [(1, 3000), (37, 2000), (256, 600), (700, 600)])
+def test_deferred_in_turn(lib, B, T):
+    K, C, V, d = 5, 256, 600, 64
+    rng = np.random.default_rng(B)
+    gen = torch.Generator(device=DEV).manual_seed(B)
+    H = torch.randn((B, T, d), generator=gen, device=DEV).to(torch.bfloat16)
+    buf = Buffers(B, K, 8, C, DEV)
+    index = torch.empty(pk.pldp_index_size(B, V), dtype=torch.uint8, device=DEV)
+    slots = index.numel() - (32 * (B + 1) + 255) // 256 * 256
+    for heavy in (0.0, 1.0, 0.0, 0.3, 0.0, 0.02):
+        ids = rng.integers(0, V, size=(B, T)).astype(np.int32)
+        lens = np.full(B, T, np.int32)
+        for b in np.nonzero(rng.random(B) < heavy)[0]:
+            ids[b, rng.integers(0, T, size=T // 4)] = ids[b, T - 1]
+        if B > 1:
+            lens[rng.integers(0, B)] = T + 1
+            lens[rng.integers(0, B)] = rng.integers(0, 3)
+        L = i32(lens)
+        pk.pldp_index_build(i32(ids), L, V, index)
+        for ix in (None, index):
+            out = buf if ix is None else Buffers(B, K, 8, C, DEV)
+            out.status.zero_()
+            pk.pldp_draft_step(i32(ids), L, 1, 3, out.cand, out.cnt, out.ml, K, out.draft, out.dlen,
+                               None if ix is not None else buf.dws, H=H, best_h=out.best_h, h_scores=out.scores_h,
+                               best_h_score=out.bscore_h, status=out.status, index=ix, V=V)
+            _compare(snapshot(out), ids, lens, H, None, None, 0, (1, 3), C, K, "hidden")
+            assert not buf.dws.any() and not index[slots:slots + 32 * (B + 1)].any()
