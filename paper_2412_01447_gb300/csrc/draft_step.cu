@@ -943,7 +943,7 @@ constexpr int kDraftWin = 32;                      // draft tokens staged per oc
 static_assert(kEntryWords * 4 == 64 && kEntryWords <= 32, "an entry is 64 bytes, a word per lane");
 
 struct IndexView {
-    DeferSlot* defer;   // [B + 1], after the entries
+    DeferSlot* defer;   // [B + 1], after the entries; null where the memory ends with these
     int32_t* ilen;      // [B]
     int32_t* flags;     // [B], build scratch
     int32_t* entries;   // [B][V][kEntryWords]
@@ -1364,8 +1364,10 @@ index_build_kernel(const int32_t* __restrict__ ids, int64_t ids_stride, const in
     const int64_t t = valid ? L - 1 : 0;
     if (rank == 0 && tid == 0) {
         ix.flags[b] = 0;
-        ix.defer[b] = DeferSlot{};
-        if (b == 0) ix.defer[B] = DeferSlot{};
+        if (ix.defer != nullptr) {
+            ix.defer[b] = DeferSlot{};
+            if (b == 0) ix.defer[B] = DeferSlot{};
+        }
     }
     const int step = S * kBuildThreads, first = rank * kBuildThreads + tid;
     uint4* entries = reinterpret_cast<uint4*>(index_entry(ix, b, 0));   // four vectors each
@@ -1415,7 +1417,8 @@ index_build_kernel(const int32_t* __restrict__ ids, int64_t ids_stride, const in
 }
 
 // Byte offsets of the index parts (ilen, flags, entries, the drafting calls' scratch),
-// 256-byte aligned.
+// 256-byte aligned.  Memory without the last part (an index was its first `defer` bytes
+// before deferred scoring was there) does too: its sequences score their own candidates.
 struct IndexLayout {
     size_t ilen, flags, entries, defer, total;
 };
@@ -1429,10 +1432,10 @@ inline IndexLayout index_layout(int B, int V) {
     l.total = l.defer + up((static_cast<size_t>(B) + 1) * sizeof(DeferSlot));
     return l;
 }
-inline IndexView index_view(void* base, int B, int V) {
+inline IndexView index_view(void* base, size_t bytes, int B, int V) {
     const IndexLayout l = index_layout(B, V);
     char* c = static_cast<char*>(base);
-    return IndexView{reinterpret_cast<DeferSlot*>(c + l.defer), reinterpret_cast<int32_t*>(c + l.ilen),
+    return IndexView{bytes < l.total ? nullptr : reinterpret_cast<DeferSlot*>(c + l.defer), reinterpret_cast<int32_t*>(c + l.ilen),
                      reinterpret_cast<int32_t*>(c + l.flags), reinterpret_cast<int32_t*>(c + l.entries), V};
 }
 
@@ -1537,10 +1540,10 @@ pldp_status prepare_draft(const pldp_draft_step_args* a, const char* what, Draft
     has_ix = a->index != nullptr;
     if (a->index) {
         if (a->V < 1) return fail(PLDP_ERR_INVALID_ARG, "%s: V < 1 with an index", what);
-        const size_t need = index_layout(B, a->V).total;
+        const size_t need = index_layout(B, a->V).defer;
         if (a->index_bytes < need || !aligned16(a->index))
             return fail(PLDP_ERR_INVALID_ARG, "%s: index needs %zu bytes, 16-byte aligned", what, need);
-        ixv = index_view(a->index, B, a->V);
+        ixv = index_view(a->index, a->index_bytes, B, a->V);
     } else if (!a->workspace || a->workspace_bytes < static_cast<size_t>(B) * kSeqWs || !aligned16(a->workspace)) {
         return fail(PLDP_ERR_INVALID_ARG, "%s: workspace needs %zu bytes, 16-byte aligned", what,
                     static_cast<size_t>(B) * kSeqWs);
@@ -1720,11 +1723,11 @@ extern "C" PLDP_API pldp_status pldp_index_build(const int32_t* ids, int64_t ids
     if (ids_stride < T_cap) return fail(PLDP_ERR_INVALID_ARG, "index_build: ids_stride < T_cap");
     if (B == 0) return PLDP_OK;
     if (!ids || !seq_len || !index) return fail(PLDP_ERR_INVALID_ARG, "index_build: null pointer");
-    const size_t need = index_layout(B, V).total;
+    const size_t need = index_layout(B, V).defer;
     if (index_bytes < need || !aligned16(index))
         return fail(PLDP_ERR_INVALID_ARG, "index_build: index needs %zu bytes, 16-byte aligned", need);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const IndexView ix = index_view(index, B, V);
+    const IndexView ix = index_view(index, index_bytes, B, V);
     // a cluster of 8 where its CTAs have a few entries or positions a thread
     const int64_t work = T_cap > V ? T_cap : V;
     int64_t S = work / (4 * kBuildThreads);

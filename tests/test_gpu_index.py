@@ -185,3 +185,31 @@ def test_build_over_garbage(lib, B, T, V):
                 assert np.array_equal(np.sort(e[b, v, 1:1 + at.size]), at), (b, v)
             else:
                 assert np.isin(e[b, v, 1:], at).all(), (b, v)
+
+
+# an index was B * V * 64 bytes and a line per 64 sequences before the scratch of deferred
+# scoring came behind them: memory of that size still does, with the same results
+def test_index_without_scratch(lib):
+    B, T, V, K, C, d = 5, 3000, 40, 6, 512, 64
+    rng = np.random.default_rng(3)
+    ids = (rng.zipf(1.5, size=(B, T)) % V).astype(np.int32)
+    L = i32(np.full(B, T, np.int32))
+    gen = torch.Generator(device=DEV).manual_seed(5)
+    H = torch.randn((B, T, d), generator=gen, device=DEV).to(torch.bfloat16)
+    short = 2 * 256 + B * V * 64
+    out = []
+    for size in (short, pk.pldp_index_size(B, V)):
+        memory = torch.full((size + 256,), 0x5a, dtype=torch.uint8, device=DEV)
+        index = memory[:size]
+        pk.pldp_index_build(i32(ids), L, V, index)
+        buf = Buffers(B, K, 8, C, DEV)
+        pk.pldp_draft_step(i32(ids), L, 1, 3, buf.cand, buf.cnt, buf.ml, K, buf.draft, buf.dlen, None, H=H,
+                           best_h=buf.best_h, h_scores=buf.scores_h, best_h_score=buf.bscore_h, status=buf.status,
+                           index=index, V=V)
+        out.append(snapshot(buf))
+        assert (memory[size:] == 0x5a).all()
+    assert out[0]["cnt"].max() > 8                       # some sequences would be deferred
+    for k in out[0]:
+        assert np.array_equal(out[0][k], out[1][k], equal_nan=out[0][k].dtype.kind == "f"), k
+    with pytest.raises(pk.PldpError, match="index needs"):
+        pk.pldp_index_build(i32(ids), L, V, torch.empty(short - 1, dtype=torch.uint8, device=DEV))
