@@ -15,10 +15,11 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
-# 2 KB is the shortest row of the streaming pass (1024 bf16, 512 fp32)
+# 2 KB is the shortest row of the streaming pass (1024 bf16, 512 fp32); every remainder of a vector
 @pytest.mark.parametrize("V,dtype", [(1023, torch.bfloat16), (1025, torch.bfloat16), (1031, torch.bfloat16),
                                      (2049, torch.bfloat16), (32001, torch.bfloat16), (511, torch.float32),
-                                     (513, torch.float32), (1026, torch.float32), (32003, torch.float32)])
+                                     (513, torch.float32), (1026, torch.float32), (32003, torch.float32)]
+                         + [(V + r, torch.bfloat16) for V in (1024, 2048) for r in range(2, 7)])
 @pytest.mark.parametrize("B,K", [(1, 1), (5, 7), (64, 10)])
 def test_greedy(lib, V, dtype, B, K):
     rng = np.random.default_rng(V + B)
@@ -44,6 +45,10 @@ def test_greedy(lib, V, dtype, B, K):
         assert np.array_equal(host(am), o["argmax"])
         assert np.array_equal(host(acc), o["accept_len"]) and np.array_equal(host(nxt), o["next_token"])
         assert not ws.any()
+
+
+def test_greedy_wide(lib):
+    test_greedy(lib, 128255, torch.bfloat16, 2, 12)
 
 
 # NaN is no maximum: whole rows, whole lanes (32 bf16 or 16 fp32 a segment) and all but a
@@ -78,7 +83,8 @@ def test_greedy_nan(lib, V, dtype):
 # (1017 and 1021 of 1024, 509 and 510 of 512), rows shorter than a vector, several pieces
 @pytest.mark.parametrize("V,dtype", [(3, torch.bfloat16), (1017, torch.bfloat16), (1021, torch.bfloat16),
                                      (2041, torch.bfloat16), (32001, torch.bfloat16), (509, torch.float32),
-                                     (510, torch.float32), (32003, torch.float32)])
+                                     (510, torch.float32), (32003, torch.float32), (128255, torch.bfloat16)]
+                         + [(1024 + r, torch.bfloat16) for r in range(1, 8)])
 @pytest.mark.parametrize("T", [0.6, 1.0])
 def test_sampling(lib, V, dtype, T):
     B, K = 5, 12
