@@ -1340,21 +1340,45 @@ __global__ void __launch_bounds__(kThreads, 1) verify_draft_kernel(const VerifyA
 // below the count), which is all that most entries of a vocabulary ever see.
 //
 // What bounds it: the clearing, V * 32 bytes a sequence (525 MB at batch 128, V = 128256:
-// 85 us alone), and the atomics, whose entries leave L2 again when many sequences are
-// under way.  A memset of everything (1.05 GB, 155 us), a kernel that inserted (83 us) and
-// one that wrote the lengths took 230-240 us there, 207 us now; batch 16 x 8k, V = 128256:
-// 64 -> 28 us; batch 64 x 16k, V = 32000: 69 -> 38 us; batch 1 x 4k: 19.5 -> 13 us.
+// 85 us alone), and the atomics: those of a text's frequent tokens take turns on a few
+// entries, and entries that have left L2 come back from memory.  Batch 16 x 8k,
+// V = 128256: 64 -> 28 us against a memset of everything, a kernel that inserted and one
+// that wrote the lengths; batch 64 x 16k, V = 32000: 69 -> 38 us; batch 1 x 4k: 19.5 -> 13 us.
+//
+// More sequences than clusters of 8 at once and entries beyond what L2 holds of those under
+// way: one launch clears them all at the memory's rate, and smaller clusters insert all the
+// sequences in one wave.  By clusters of 8 that clear and insert in turn, a few sequences at
+// a time, each wave waited for its frequent tokens.  Batch 128 x 32k, V = 128256, against
+// those and (in brackets) the three kernels: Zipf tokens whose ids are in the order of their
+// frequency, as a tokenizer's roughly are, 272 -> 203 (243) us, named at random 233 -> 186
+// (230), uniform tokens 207 -> 236 (306); 200 x 4k, V = 152000, 226 -> 184 (290); 300 x 16k,
+// V = 128256, in order 463 -> 344 (435).
 constexpr int kBuildThreads = 1024;
 constexpr int kBuildLoads = 4;                     // positions in flight per thread
-// Tokens cleared and counted at a time, when there are more sequences than clusters at
-// once: entries then wait less long for their positions (228 -> 207 us at the first size
-// above; 16384 gave 197, and 45 for 28 us at the second, where one pass is best).
+constexpr int kClearThreads = 512;
+// Tokens counted (and cleared) at a time, when there are more sequences than clusters at
+// once: entries then wait less long for their positions.  Inserting alone, uniform tokens at
+// the first size above: 248 us against 266 by 65536 (Zipf in order 217 / 205).  With the
+// clearing, batch 128 x 32k, V = 50257, Zipf: 147 / 131 us against 164 / 152 in one pass.
 constexpr int64_t kBuildTokens = 32768;
+// The largest vocabulary whose entries the clusters clear themselves: batch 128 x 32k,
+// V = 50257, Zipf 137 / 127 us (cleared first 133 / 127), uniform 127 (188); the same of
+// V = 66000, Zipf 184 / 166 us (148 / 143), uniform 150 (205); 64 x 16k, V = 100000, Zipf
+// 90 / 80 us (80 / 84), uniform 80 (84).
+constexpr int kBuildClearTokens = 65536;
+
+__global__ void __launch_bounds__(kClearThreads) index_clear_kernel(uint4* __restrict__ entries, int64_t sectors) {
+    pdl_enter();
+    const int64_t step = static_cast<int64_t>(gridDim.x) * kClearThreads;
+#pragma unroll 4
+    for (int64_t u = static_cast<int64_t>(blockIdx.x) * kClearThreads + threadIdx.x; u < 2 * sectors; u += step)
+        entries[(u >> 1) * (kEntryWords / 4) + (u & 1)] = make_uint4(0u, 0u, 0u, 0u);
+}
 
 __global__ void __launch_bounds__(kBuildThreads, 2)
 index_build_kernel(const int32_t* __restrict__ ids, int64_t ids_stride, const int32_t* __restrict__ seq_len, int B,
                    int64_t T_cap, IndexView ix, uint32_t* __restrict__ status, int S,
-                   int64_t tokens) {
+                   int64_t tokens, bool clear) {
     pdl_enter();
     const int b = blockIdx.x / S;
     const int rank = blockIdx.x - b * S;
@@ -1375,9 +1399,10 @@ index_build_kernel(const int32_t* __restrict__ ids, int64_t ids_stride, const in
     bool bad = false;                              // a token the index cannot hold
     for (int64_t v0 = 0; v0 < ix.V; v0 += tokens) {                    // cluster-uniform
         const int64_t v1 = v0 + tokens < ix.V ? v0 + tokens : ix.V;
+        if (clear)
 #pragma unroll 4
-        for (int64_t u = 2 * v0 + first; u < 2 * v1; u += step)
-            entries[(u >> 1) * (kEntryWords / 4) + (u & 1)] = make_uint4(0u, 0u, 0u, 0u);   // a sector per two lanes
+            for (int64_t u = 2 * v0 + first; u < 2 * v1; u += step)
+                entries[(u >> 1) * (kEntryWords / 4) + (u & 1)] = make_uint4(0u, 0u, 0u, 0u);   // a sector per two lanes
         if (S > 1) {
             cluster_arrive();
             cluster_wait();
@@ -1732,11 +1757,18 @@ extern "C" PLDP_API pldp_status pldp_index_build(const int32_t* ids, int64_t ids
     const int64_t work = T_cap > V ? T_cap : V;
     int64_t S = work / (4 * kBuildThreads);
     S = S < 1 ? 1 : (S > kScanMaxCluster ? kScanMaxCluster : S);
-    const int64_t at_once = resident_blocks(reinterpret_cast<const void*>(&index_build_kernel), kBuildThreads, 0) / S;
-    const int64_t tokens = B > at_once ? kBuildTokens : V;
+    const int64_t ctas = resident_blocks(reinterpret_cast<const void*>(&index_build_kernel), kBuildThreads, 0);
+    const int64_t tokens = B > ctas / S ? kBuildTokens : V;
+    const bool clear_first = B > ctas / S && V > kBuildClearTokens;
+    if (clear_first) {
+        while (S > 1 && B * S > ctas) S /= 2;                    // all sequences at once
+        const cudaError_t e = launch_pdl(index_clear_kernel, dim3(8 * sm_count()), dim3(kClearThreads), 0, s, 0,
+                                         reinterpret_cast<uint4*>(ix.entries), static_cast<int64_t>(B) * V);
+        if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "index_build: launch failed: %s", cudaGetErrorString(e));
+    }
     const cudaError_t e = launch_pdl(index_build_kernel, dim3(static_cast<unsigned>(B * S)), dim3(kBuildThreads), 0, s,
                                      S > 1 ? static_cast<int>(S) : 0, ids, ids_stride, seq_len, B, T_cap, ix, status,
-                                     static_cast<int>(S), tokens);
+                                     static_cast<int>(S), tokens, !clear_first);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "index_build: launch failed: %s", cudaGetErrorString(e));
     return PLDP_OK;
 }

@@ -154,8 +154,10 @@ def test_indexed_decode_loop(lib):
 
 # the index built over memory that holds anything: one CTA a sequence and a cluster, one
 # pass over the vocabulary and several (more sequences than clusters at once), entries that
-# fill and overflow, invalid lengths and tokens out of range
-@pytest.mark.parametrize("B,T,V", [(3, 700, 40), (2, 5000, 9000), (60, 9000, 70001), (45, 300, 40000)])
+# fill and overflow, invalid lengths and tokens out of range; entries cleared by the clusters that
+# insert (up to 65536 tokens) and by a launch of its own, then one CTA a sequence and several
+@pytest.mark.parametrize("B,T,V", [(3, 700, 40), (2, 5000, 9000), (60, 9000, 70001), (45, 300, 40000),
+                                   (40, 300, 65536), (160, 300, 65537), (100, 2000, 65540)])
 def test_build_over_garbage(lib, B, T, V):
     rng = np.random.default_rng(B + V)
     ids = (rng.zipf(1.3, size=(B, T)) % V).astype(np.int32)
