@@ -17,6 +17,7 @@ namespace {
 constexpr int kThreads = kRankThreads;
 constexpr int kMaxCluster = 8;                // portable
 constexpr int kWideCluster = 16;
+constexpr int kLongList = 512;                // candidates (see pick_split_hidden)
 constexpr size_t kMaxQueryBytes = 196608;     // d * sizeof(dtype) limit
 constexpr int kMaxSelRows = 8192;             // row_idx entries staged in shared memory
 
@@ -351,19 +352,37 @@ rank_attention_kernel(const void* __restrict__ A, bool a_bf16, int R, int64_t ro
 // CTAs per sequence: as many as the kernel's resident CTA slots allow for the
 // batch (all of its CTAs in one wave), up to a cluster of 8, never more than the
 // candidate capacity.  `kernel` is the variant launched when S > 1.
-//
-// wide: up to a cluster of 16, where the slots allow it and most of the batch's clusters
-// are resident at once.  The sequence with the most candidates sets the time of Eq. 3's
-// call: 1024 of them (batch 16 x 32k Zipf tokens, unigram match) took 43.4 us with 8 CTAs
-// and one candidate per warp, 30.1 us with two per warp, 18.0 us with 16 CTAs.  Eq. 2
-// stays at 8: 16 gave it 8.8 -> 7.2 us there, but 9.3 -> 10.2 us with one candidate a
-// sequence after an L2 flush.
-int pick_split(int B, int C_cap, const void* kernel, size_t smem, bool wide = false) {
+int pick_split(int B, int C_cap, const void* kernel, size_t smem) {
     int s = resident_blocks(kernel, kThreads, smem) / (B > 0 ? B : 1);
     if (s > C_cap) s = C_cap;
-    if (s > kMaxCluster)
-        s = wide && s >= kWideCluster && 4 * resident_clusters(kernel, kThreads, smem, kWideCluster) >= 3 * B ? kWideCluster
-                                                                                                             : kMaxCluster;
+    return s < 1 ? 1 : (s > kMaxCluster ? kMaxCluster : s);
+}
+
+// The same for Eq. 3: the largest clusters, of up to 16, that are all resident at once.
+// Clusters do not straddle the parts of the GPU that hold them, so fewer fit than the
+// slots have room for (14 of 16 CTAs, 19 of 13, 97 of 3), and a call that needs a second
+// wave of them takes 2 us more, which is half of its time where a sequence has a few
+// candidates: batch 40, clusters of 7 and of 6, 6.6 and 4.5 us (lists of 256: 10.6 and
+// 11.1); batch 100, of 3 and of 2, 6.6 and 4.6 us (lists of 64: 12.8 both); batch 24, of 8
+// and of 10, 4.5 us both (lists of 256: 10.3 and 8.2).  Past the portable 8 an exact fit is
+// not taken: batch 19, clusters of 13, 5.7 us, of 12 4.5.
+//
+// Long lists (kLongList candidates or more fit): clusters of 16 though a quarter of the
+// batch's come in a second wave, since the sequence with the most candidates sets the time
+// of the call: 1024 of them (batch 16 x 32k Zipf tokens, unigram match) took 43.4 us with 8
+// CTAs and one candidate per warp, 30.1 us with two per warp, 18.0 us with 16 CTAs, 21 us
+// with 13; where every list is short the second wave is 6.6 for 4.7 us.
+//
+// Eq. 2 stays at 8: 16 gave it 8.8 -> 7.2 us on the lists of 1024, but 9.3 -> 10.2 us with
+// one candidate a sequence after an L2 flush.
+int pick_split_hidden(int B, int C_cap, const void* kernel, size_t smem) {
+    int s = resident_blocks(kernel, kThreads, smem) / (B > 0 ? B : 1);
+    if (s > C_cap) s = C_cap;
+    if (s >= kWideCluster) {
+        s = kWideCluster;
+        if (C_cap >= kLongList && 4 * resident_clusters(kernel, kThreads, smem, s) >= 3 * B) return s;
+    }
+    while (s > 1 && resident_clusters(kernel, kThreads, smem, s) < B + (s > kMaxCluster ? 1 : 0)) --s;
     return s < 1 ? 1 : s;
 }
 
@@ -526,8 +545,8 @@ extern "C" PLDP_API pldp_status pldp_rank_hidden(const void* H, pldp_dtype dtype
     const bool vec = aligned16(H) && (d * es) % 16 == 0 && (seq_stride * es) % 16 == 0;
     const size_t smem = (static_cast<size_t>(d) * es + 127) / 128 * 128;
     // (every variant fits as many CTAs an SM as this one)
-    const int S = pick_split(B, C_cap, reinterpret_cast<const void*>(&rank_hidden_kernel<__nv_bfloat16, true, true>),
-                             smem, true);
+    const int S = pick_split_hidden(B, C_cap,
+                                    reinterpret_cast<const void*>(&rank_hidden_kernel<__nv_bfloat16, true, true>), smem);
     cudaError_t e;
     if (dtype == PLDP_BF16) {
         const __nv_bfloat16* h = static_cast<const __nv_bfloat16*>(H);
