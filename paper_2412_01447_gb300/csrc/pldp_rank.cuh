@@ -199,12 +199,13 @@ __device__ __forceinline__ int64_t cand_at(const int32_t* __restrict__ cands, co
 
 // Eq. 3 with one warp per candidate (G = 1): warp `slot` scores candidates slot,
 // slot + P, ... of this CTA on its own, two at a time: each 16 bytes of the query row
-// are read and widened once for both, its norm is summed once for all, and 16 loads of
-// 16 bytes are in flight per lane.  The rows of the next pair head for L2 meanwhile.  The
+// are read and widened once for both, its norm is summed once for all, and 2 U loads of
+// 16 bytes are in flight per lane (U = 8, or 4 where three CTAs share an SM: the same sums
+// in the same order).  The rows of the next pair head for L2 meanwhile.  The
 // positions are read 32 candidates at a time, a lane each.  510 candidates per sequence
 // (batch 128, 535 MB of random 8 KB rows of a 34 GB tensor, L2 flushed): 107 -> 100 us,
 // 5.3 TB/s; 128 per sequence: 41.7 -> 37.5 us.
-template <typename T, bool CANDS_SHARED>
+template <typename T, bool CANDS_SHARED, int U>
 __device__ __forceinline__ void hidden_rank_warp(const T* __restrict__ hb, int64_t d, int64_t t,
                                                  const int32_t* __restrict__ cands, int S, int rank,
                                                  const int32_t* jpre, const T* q_sh, uint64_t* bar, bool q_pending,
@@ -233,10 +234,10 @@ __device__ __forceinline__ void hidden_rank_warp(const T* __restrict__ hb, int64
         const T* r0 = hb + (ok0 ? j0 - 1 : 0) * d;        // H_{j-1}
         const T* r1 = hb + (ok1 ? j1 - 1 : 0) * d;
         uint64_t dot0 = 0, na0 = 0, dot1 = 0, na1 = 0;
-        for (int c0 = lane; c0 < nch; c0 += 32 * kRowUnroll) {
-            uint4 a0[kRowUnroll], a1[kRowUnroll];
+        for (int c0 = lane; c0 < nch; c0 += 32 * U) {
+            uint4 a0[U], a1[U];
 #pragma unroll
-            for (int u = 0; u < kRowUnroll; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const int c = c0 + 32 * u;
                 if (ok0 && c < nch) a0[u] = ld_stream16(r0 + static_cast<int64_t>(c) * E);
                 if (ok1 && c < nch) a1[u] = ld_stream16(r1 + static_cast<int64_t>(c) * E);
@@ -255,7 +256,7 @@ __device__ __forceinline__ void hidden_rank_warp(const T* __restrict__ hb, int64
             }
             if (timed_out) break;
 #pragma unroll
-            for (int u = 0; u < kRowUnroll; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const int c = c0 + 32 * u;
                 if (c < nch) {
                     const uint4 q = *reinterpret_cast<const uint4*>(q_sh + static_cast<int64_t>(c) * E);
@@ -299,7 +300,7 @@ __device__ __forceinline__ void hidden_rank_warp(const T* __restrict__ hb, int64
 // batch's positions.  Returns with sh.err set if the query never arrived.
 // With CANDS_SHARED the candidate list is in shared memory (else global, read
 // through L2 since other CTAs of the cluster may have just written it).
-template <typename T, bool VEC, bool CANDS_SHARED = false>
+template <typename T, bool VEC, bool CANDS_SHARED = false, int U = kRowUnroll>
 __device__ __forceinline__ void hidden_rank_cta(const T* __restrict__ hb, int64_t d, int64_t t,
                                                 const int32_t* __restrict__ cands, int n, int S,
                                                 int rank, const int32_t* jpre, const T* q_sh,
@@ -310,7 +311,7 @@ __device__ __forceinline__ void hidden_rank_cta(const T* __restrict__ hb, int64_
     const Batch bt = batch_shape(n, S, rank, wg);
     if constexpr (VEC) {
         if (bt.G == 1) {                                  // one warp per candidate: no barriers
-            hidden_rank_warp<T, CANDS_SHARED>(hb, d, t, cands, S, rank, jpre, q_sh, bar, q_pending, threshold,
+            hidden_rank_warp<T, CANDS_SHARED, U>(hb, d, t, cands, S, rank, jpre, q_sh, bar, q_pending, threshold,
                                               scores_row, sh, bt);
             wg.sync();
             return;

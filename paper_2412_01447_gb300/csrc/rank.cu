@@ -17,7 +17,7 @@ namespace {
 constexpr int kThreads = kRankThreads;
 constexpr int kMaxCluster = 8;                // portable
 constexpr int kWideCluster = 16;
-constexpr int kLongList = 512;                // candidates (see pick_split_hidden)
+constexpr int64_t kLongList = 4 << 20;        // bytes of candidate rows (see pick_split_hidden)
 constexpr size_t kMaxQueryBytes = 196608;     // d * sizeof(dtype) limit
 constexpr int kMaxSelRows = 8192;             // row_idx entries staged in shared memory
 
@@ -87,8 +87,10 @@ __device__ __forceinline__ void prefetch_first(RankShared& sh, const int32_t* ca
     }
 }
 
-template <typename T, bool VEC, bool CLUSTER>
-__global__ void __launch_bounds__(kThreads, 2)
+// PER_SM CTAs an SM: 2 with 16 loads in flight per lane where a warp takes two candidates,
+// or 3 with 8 (see pick_split_hidden).
+template <typename T, bool VEC, bool CLUSTER, int PER_SM>
+__global__ void __launch_bounds__(kThreads, PER_SM)
 rank_hidden_kernel(const T* __restrict__ H, int64_t d, int64_t seq_stride,
                    const int32_t* __restrict__ seq_len, int64_t T_cap,
                    const int32_t* __restrict__ cand_pos, const int32_t* __restrict__ cand_count,
@@ -147,7 +149,7 @@ rank_hidden_kernel(const T* __restrict__ H, int64_t d, int64_t seq_stride,
         }
     }
     __syncthreads();               // mbarrier initialised; shared state visible
-    hidden_rank_cta<T, VEC>(hb, d, t, cand_pos + static_cast<int64_t>(b) * C_cap, n, S, rank, sh.jpre,
+    hidden_rank_cta<T, VEC, false, PER_SM == 2 ? 8 : 4>(hb, d, t, cand_pos + static_cast<int64_t>(b) * C_cap, n, S, rank, sh.jpre,
                             q_sh, wait_bar, need_query && VEC, threshold,
                             scores ? scores + static_cast<int64_t>(b) * C_cap : nullptr, sh);
     if constexpr (VEC) {
@@ -367,7 +369,7 @@ int pick_split(int B, int C_cap, const void* kernel, size_t smem) {
 // and of 10, 4.5 us both (lists of 256: 10.3 and 8.2).  Past the portable 8 an exact fit is
 // not taken: batch 19, clusters of 13, 5.7 us, of 12 4.5.
 //
-// Long lists (kLongList candidates or more fit): clusters of 16 though a quarter of the
+// Long lists (room for kLongList bytes of rows): clusters of 16 though a quarter of the
 // batch's come in a second wave, since the sequence with the most candidates sets the time
 // of the call: 1024 of them (batch 16 x 32k Zipf tokens, unigram match) took 43.4 us with 8
 // CTAs and one candidate per warp, 30.1 us with two per warp, 18.0 us with 16 CTAs, 21 us
@@ -375,15 +377,40 @@ int pick_split(int B, int C_cap, const void* kernel, size_t smem) {
 //
 // Eq. 2 stays at 8: 16 gave it 8.8 -> 7.2 us on the lists of 1024, but 9.3 -> 10.2 us with
 // one candidate a sequence after an L2 flush.
-int pick_split_hidden(int B, int C_cap, const void* kernel, size_t smem) {
+//
+// Two kernels, two CTAs an SM or three: the one whose grid fills the larger share of its
+// slots, and on long lists also where they are equal, since more of the smaller CTAs are
+// then under way per sequence.  Lists of 64, two and three CTAs an SM: batch 64 9.0 / 10.3
+// us, 100 12.9 / 11.7, 120 13.3 / 15.3, 160 18.7 / 14.9, 200 19.5 / 15.7, 300 12.9 / 15.1;
+// lists of 1024: batch 100 35.3 / 25.7, 128 110 / 101, 200 38.5 / 28.0 us (with a warp's
+// candidates one at a time, three CTAs an SM: 30.1, 126, 31.9).
+struct HiddenSplit {
+    int S;         // CTAs a sequence
+    int per_sm;    // 2 or 3
+};
+
+int fit_clusters(int B, int C_cap, const void* kernel, size_t smem) {
     int s = resident_blocks(kernel, kThreads, smem) / (B > 0 ? B : 1);
     if (s > C_cap) s = C_cap;
-    if (s >= kWideCluster) {
-        s = kWideCluster;
-        if (C_cap >= kLongList && 4 * resident_clusters(kernel, kThreads, smem, s) >= 3 * B) return s;
-    }
+    if (s > kWideCluster) s = kWideCluster;
     while (s > 1 && resident_clusters(kernel, kThreads, smem, s) < B + (s > kMaxCluster ? 1 : 0)) --s;
     return s < 1 ? 1 : s;
+}
+
+HiddenSplit pick_split_hidden(int B, int C_cap, int64_t row_bytes, const void* two, const void* three, size_t smem) {
+    const bool long_list = C_cap * row_bytes >= kLongList;
+    const int64_t slots2 = resident_blocks(two, kThreads, smem), slots3 = resident_blocks(three, kThreads, smem);
+    if (long_list && C_cap >= kWideCluster && slots2 / B >= kWideCluster &&
+        4 * resident_clusters(two, kThreads, smem, kWideCluster) >= 3 * B)
+        return {kWideCluster, 2};
+    const int s2 = fit_clusters(B, C_cap, two, smem);
+    if (slots3 <= slots2 || slots2 < 1) return {s2, 2};
+    const int s3 = fit_clusters(B, C_cap, three, smem);
+    const int64_t n2 = static_cast<int64_t>(B) * s2, n3 = static_cast<int64_t>(B) * s3;
+    const int64_t room2 = (n2 + slots2 - 1) / slots2 * slots2, room3 = (n3 + slots3 - 1) / slots3 * slots3;   // whole waves
+    const int64_t fill2 = n2 * room3, fill3 = n3 * room2;
+    if (fill3 > fill2 || (fill3 == fill2 && long_list)) return {s3, 3};
+    return {s2, 2};
 }
 
 template <typename K, typename... Args>
@@ -414,17 +441,17 @@ cudaError_t launch_rank(K kernel, int B, int S, size_t smem, void* stream, Args.
     return cudaLaunchKernelEx(&cfg, kernel, args..., S);
 }
 
-template <typename T, bool VEC>
+template <typename T, bool VEC, int PER_SM>
 cudaError_t launch_hidden(int B, int S, size_t smem, void* stream, const T* h, int64_t d,
                           int64_t seq_stride, const int32_t* seq_len, int64_t T_cap,
                           const int32_t* cand_pos, const int32_t* cand_count, int C_cap,
                           float threshold, float* scores, int32_t* best_pos, float* best_score,
                           uint32_t* status) {
     if (S > 1)
-        return launch_rank(rank_hidden_kernel<T, VEC, true>, B, S, smem, stream, h, d, seq_stride,
+        return launch_rank(rank_hidden_kernel<T, VEC, true, PER_SM>, B, S, smem, stream, h, d, seq_stride,
                            seq_len, T_cap, cand_pos, cand_count, C_cap, threshold, scores, best_pos,
                            best_score, status);
-    return launch_rank(rank_hidden_kernel<T, VEC, false>, B, S, smem, stream, h, d, seq_stride,
+    return launch_rank(rank_hidden_kernel<T, VEC, false, PER_SM>, B, S, smem, stream, h, d, seq_stride,
                        seq_len, T_cap, cand_pos, cand_count, C_cap, threshold, scores, best_pos,
                        best_score, status);
 }
@@ -544,27 +571,20 @@ extern "C" PLDP_API pldp_status pldp_rank_hidden(const void* H, pldp_dtype dtype
 
     const bool vec = aligned16(H) && (d * es) % 16 == 0 && (seq_stride * es) % 16 == 0;
     const size_t smem = (static_cast<size_t>(d) * es + 127) / 128 * 128;
-    // (every variant fits as many CTAs an SM as this one)
-    const int S = pick_split_hidden(B, C_cap,
-                                    reinterpret_cast<const void*>(&rank_hidden_kernel<__nv_bfloat16, true, true>), smem);
+    // (the other types fit as many CTAs an SM)
+    const HiddenSplit sp =
+        pick_split_hidden(B, C_cap, d * static_cast<int64_t>(es),
+                          reinterpret_cast<const void*>(&rank_hidden_kernel<__nv_bfloat16, true, true, 2>),
+                          reinterpret_cast<const void*>(&rank_hidden_kernel<__nv_bfloat16, true, true, 3>), smem);
     cudaError_t e;
-    if (dtype == PLDP_BF16) {
-        const __nv_bfloat16* h = static_cast<const __nv_bfloat16*>(H);
-        e = vec ? launch_hidden<__nv_bfloat16, true>(B, S, smem, stream, h, d, seq_stride, seq_len, T_cap,
-                                                     cand_pos, cand_count, C_cap, threshold, scores,
-                                                     best_pos, best_score, status)
-                : launch_hidden<__nv_bfloat16, false>(B, S, smem, stream, h, d, seq_stride, seq_len,
-                                                      T_cap, cand_pos, cand_count, C_cap, threshold,
-                                                      scores, best_pos, best_score, status);
-    } else {
-        const float* h = static_cast<const float*>(H);
-        e = vec ? launch_hidden<float, true>(B, S, smem, stream, h, d, seq_stride, seq_len, T_cap,
-                                             cand_pos, cand_count, C_cap, threshold, scores, best_pos,
-                                             best_score, status)
-                : launch_hidden<float, false>(B, S, smem, stream, h, d, seq_stride, seq_len, T_cap,
-                                              cand_pos, cand_count, C_cap, threshold, scores, best_pos,
-                                              best_score, status);
-    }
+#define PLDP_HIDDEN_LAUNCH(T, V, N)                                                                                    \
+    launch_hidden<T, V, N>(B, sp.S, smem, stream, static_cast<const T*>(H), d, seq_stride, seq_len, T_cap, cand_pos, \
+                           cand_count, C_cap, threshold, scores, best_pos, best_score, status)
+#define PLDP_HIDDEN_TYPE(T) \
+    (!vec ? PLDP_HIDDEN_LAUNCH(T, false, 2) : sp.per_sm == 3 ? PLDP_HIDDEN_LAUNCH(T, true, 3) : PLDP_HIDDEN_LAUNCH(T, true, 2))
+    e = dtype == PLDP_BF16 ? PLDP_HIDDEN_TYPE(__nv_bfloat16) : PLDP_HIDDEN_TYPE(float);
+#undef PLDP_HIDDEN_TYPE
+#undef PLDP_HIDDEN_LAUNCH
     if (e != cudaSuccess)
         return fail(PLDP_ERR_CUDA, "rank_hidden: launch failed: %s", cudaGetErrorString(e));
     return PLDP_OK;
