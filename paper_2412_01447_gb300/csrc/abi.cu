@@ -64,7 +64,7 @@ int resident_clusters(const void* kernel, int threads, size_t smem, int size) {
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
     if (size > 8) cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (smem > 48 * 1024)
+    if (smem > kOptInShared)
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;

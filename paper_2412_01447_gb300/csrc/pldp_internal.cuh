@@ -23,6 +23,10 @@ int resident_blocks(const void* kernel, int threads, size_t smem);
 // Clusters of `size` CTAs of `kernel` that fit at once; 0 when it takes none (cached).
 int resident_clusters(const void* kernel, int threads, size_t smem, int size);
 
+// Dynamic shared memory above which a kernel opts in to more: its static shared memory counts
+// toward the 48 KB that it has otherwise.
+constexpr size_t kOptInShared = 40 * 1024;
+
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // ---------------------------------------------------------------------------

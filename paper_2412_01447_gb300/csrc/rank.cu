@@ -429,7 +429,7 @@ cudaError_t launch_rank(K kernel, int B, int S, size_t smem, void* stream, Args.
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = S > 1 ? 2 : 1;
-    if (smem > 48 * 1024) {
+    if (smem > kOptInShared) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(smem));
         if (e != cudaSuccess) return e;

@@ -94,3 +94,23 @@ def test_paired_candidates(lib, B, n, d, dtype):
     check_scores(host(sc), o_s, host(cnt), n)
     check_choice(host(best), o_b, o_s, host(cand), host(cnt), n)
     assert not st.any()
+
+
+# the dynamic shared memory of a call and the kernel's own, around the 48 KB that need no opt-in
+@pytest.mark.parametrize("d", [24448, 24512, 24576, 24584])
+def test_rows_around_48_kb(lib, d):
+    B, T, C = 3, 40, 9
+    gen = torch.Generator(device=DEV).manual_seed(d)
+    H = torch.randn((B, T, d), generator=gen, device=DEV).to(torch.bfloat16)
+    cand = torch.arange(2, 2 + C, dtype=torch.int32, device=DEV).repeat(B, 1)
+    cnt, L = torch.full((B,), C, dtype=torch.int32, device=DEV), torch.full((B,), T, dtype=torch.int32, device=DEV)
+    sc, best = torch.zeros((B, C), device=DEV), torch.zeros(B, dtype=torch.int32, device=DEV)
+    lib.pldp_rank_hidden(H, L, cand, cnt, best, scores=sc)
+    o_s, o_b, _ = oracle.rank_hidden(host(H), host(L), host(cand), host(cnt))
+    check_scores(host(sc), o_s, host(cnt), C)
+    check_choice(host(best), o_b, o_s, host(cand), host(cnt), C)
+    lib.pldp_rank_hidden_avg(H[..., :d // 2].contiguous(), L, cand, cnt, best, 2, scores=sc)   # fp32 sums of its rows
+    assert not sc.isnan().any() and (best >= 2).all()
+    A = torch.rand((B, d // 4, T), generator=gen, device=DEV)                                  # 8 bytes a selected row
+    lib.pldp_rank_attention(A, L, cand, cnt, best, scores=sc)
+    assert np.array_equal(host(sc), host(A.amax(1).gather(1, cand.long())))
