@@ -19,7 +19,9 @@ DEV = "cuda"
 @pytest.mark.parametrize("V,dtype", [(1023, torch.bfloat16), (1025, torch.bfloat16), (1031, torch.bfloat16),
                                      (2049, torch.bfloat16), (32001, torch.bfloat16), (511, torch.float32),
                                      (513, torch.float32), (1026, torch.float32), (32003, torch.float32)]
-                         + [(V + r, torch.bfloat16) for V in (1024, 2048) for r in range(2, 7)])
+                         + [(V + r, torch.bfloat16) for V in (1024, 2048) for r in range(2, 7)]
+                         # fp32: element loads up to 32 MB, or 16 MB of rows of 192 KB
+                         + [(12001, torch.float32), (12002, torch.float32)])
 @pytest.mark.parametrize("B,K", [(1, 1), (5, 7), (64, 10)])
 def test_greedy(lib, V, dtype, B, K):
     rng = np.random.default_rng(V + B)
@@ -47,16 +49,17 @@ def test_greedy(lib, V, dtype, B, K):
         assert not ws.any()
 
 
-def test_greedy_wide(lib):
-    test_greedy(lib, 128255, torch.bfloat16, 2, 12)
+@pytest.mark.parametrize("B,K,dtype", [(2, 12, torch.bfloat16), (3, 10, torch.float32), (3, 13, torch.float32)])
+def test_greedy_wide(lib, B, K, dtype):
+    test_greedy(lib, 128255, dtype, B, K)
 
 
 # NaN is no maximum: whole rows, whole lanes (32 bf16 or 16 fp32 a segment) and all but a
 # few elements of a row; the streaming path against the element loads, which take one
 # element at a time
-@pytest.mark.parametrize("V,dtype", [(1025, torch.bfloat16), (5003, torch.bfloat16), (5003, torch.float32)])
-def test_greedy_nan(lib, V, dtype):
-    B, K = 6, 7
+@pytest.mark.parametrize("V,dtype,B", [(1025, torch.bfloat16, 6), (5003, torch.bfloat16, 6), (5003, torch.float32, 220)])
+def test_greedy_nan(lib, V, dtype, B):
+    K = 7
     gen = torch.Generator(device=DEV).manual_seed(V)
     logits = torch.randn((B, K + 1, V), generator=gen, device=DEV).to(dtype)
     logits[0] = float("nan")
