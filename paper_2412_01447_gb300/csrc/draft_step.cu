@@ -106,6 +106,7 @@ struct DraftParams {
     uint32_t* status;
     int B;
     struct DeferSlot* defer;   // [B + 1], all zero between calls; null: nothing is deferred
+    bool count;                // the sequences decided on are counted (see score_deferred_kernel)
 };
 
 // What the drafting kernels leave to score_deferred_kernel: `pending` candidates of a
@@ -125,7 +126,7 @@ static_assert(sizeof(DeferSlot) == 32 && 2 * sizeof(DeferSlot) <= kSeqWs, "B + 1
 __device__ __forceinline__ void decide(const DraftParams& p, int b, unsigned pending) {
     if (p.defer == nullptr) return;
     if (pending != 0) p.defer[b].pending = pending;
-    atomicAdd(&p.defer[p.B].decided, pending != 0 ? 1u + kDeferred : 1u);
+    if (p.count) atomicAdd(&p.defer[p.B].decided, pending != 0 ? 1u + kDeferred : 1u);
 }
 
 template <int NB>
@@ -477,11 +478,12 @@ __device__ __forceinline__ void write_counts(const DraftParams& p, int b, int ns
 // for the launch all the same, most of it the boundary between two kernels: fused step of
 // batch 128 x 32k uniform tokens 74.7 us without it, 76.5 with a grid of one CTA, 76.8 with
 // every CTA waiting for the drafting kernel and then finding nothing.  COUNTED (behind
-// indexed drafting, which counts the sequences it has decided on): when all are and none
-// is left, every CTA but the first leaves before the wait, 76.4; the first stays until the
-// drafting kernel is complete, since the stream's next work relies on this launch for that.
-// Behind the scanning kernel the counts cost as much as they gave (draft_step, 2 x 128k
-// Zipf tokens, 12.2 -> 12.4 us).
+// indexed drafting of more sequences than half the SMs, which counts those it has decided
+// on): when all are and none is left, every CTA but the first leaves before the wait, 76.4;
+// the first stays until the drafting kernel is complete, since the stream's next work relies
+// on this launch for that.  Where the drafting CTAs leave room for these, they are all there
+// by then, and the counts cost 0.15 us a call and give nothing; behind the scanning kernel
+// they cost as much as they gave (draft_step, 2 x 128k Zipf tokens, 12.2 -> 12.4 us).
 template <typename TH, bool COUNTED>
 __global__ void __launch_bounds__(kThreads, 2) score_deferred_kernel(const DraftParams p, int B) {
     constexpr bool HAS_H = !std::is_same<TH, NoHidden>::value;
@@ -1468,14 +1470,15 @@ inline IndexView index_view(void* base, size_t bytes, int B, int V) {
 // may have to leave some: then its launch is followed by score_deferred_kernel's.
 inline bool may_defer(const DraftParams& p, int64_t here) { return p.C_cap > here && p.T_cap > here; }
 
-template <typename TH, bool COUNTED>
+template <typename TH>
 pldp_status launch_deferred(const DraftParams& p, int B, cudaStream_t s, const char* what) {
-    int64_t blocks = resident_blocks(reinterpret_cast<const void*>(&score_deferred_kernel<TH, COUNTED>), kThreads, 0);
+    const auto kernel = p.count ? score_deferred_kernel<TH, true> : score_deferred_kernel<TH, false>;
+    int64_t blocks = resident_blocks(reinterpret_cast<const void*>(kernel), kThreads, 0);
     const int64_t most = p.C_cap < p.T_cap ? p.C_cap : p.T_cap;               // candidates of a sequence
     const int64_t need = (most + kWarps - 1) / kWarps * B;                    // units of one per warp
     if (blocks > need) blocks = need;
-    const cudaError_t e = launch_pdl(score_deferred_kernel<TH, COUNTED>, dim3(static_cast<unsigned>(blocks)),
-                                     dim3(kThreads), 0, s, 0, p, B);
+    const cudaError_t e =
+        launch_pdl(kernel, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, s, 0, p, B);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "%s: launch failed: %s", what, cudaGetErrorString(e));
     return PLDP_OK;
 }
@@ -1491,17 +1494,18 @@ pldp_status launch_t(const DraftParams& p0, int B, cudaStream_t s) {
     const cudaError_t e = launch_pdl(draft_step_kernel<TH, IVEC>, dim3(static_cast<unsigned>(B) * CL), dim3(kThreads), 0,
                                      s, CL > 1 ? CL : 0, p, CL, chunk);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "draft_step: launch failed: %s", cudaGetErrorString(e));
-    return p.defer ? launch_deferred<TH, false>(p, B, s, "draft_step") : PLDP_OK;
+    return p.defer ? launch_deferred<TH>(p, B, s, "draft_step") : PLDP_OK;
 }
 
 template <typename TH, bool IVEC>
 pldp_status launch_index_t(const DraftParams& p0, const IndexView& ix, int B, cudaStream_t s) {
     DraftParams p = p0;
     p.defer = may_defer(p, kCtaPasses * kMaxScoreBatch) ? ix.defer : nullptr;
+    p.count = p.defer != nullptr && 2 * B > sm_count();
     cudaError_t e = launch_pdl(draft_index_kernel<TH, IVEC>, dim3(static_cast<unsigned>(B)), dim3(kThreads), 0, s, 0,
                                p, ix);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "draft_step (indexed): launch failed: %s", cudaGetErrorString(e));
-    return p.defer ? launch_deferred<TH, true>(p, B, s, "draft_step (indexed)") : PLDP_OK;
+    return p.defer ? launch_deferred<TH>(p, B, s, "draft_step (indexed)") : PLDP_OK;
 }
 
 template <typename TH>
@@ -1624,10 +1628,11 @@ pldp_status launch_verify_draft_t(const VerifyArgs& va, const DraftParams& p0, c
                                   cudaStream_t s) {
     DraftParams p = p0;
     p.defer = may_defer(p, kCtaPasses * kMaxScoreBatch) ? ix.defer : nullptr;
+    p.count = p.defer != nullptr && 2 * B > sm_count();
     const cudaError_t e = launch_pdl(verify_draft_kernel<TH, IVEC>, dim3(static_cast<unsigned>(B)), dim3(kThreads), 0,
                                      s, 0, va, p, ix);
     if (e != cudaSuccess) return fail(PLDP_ERR_CUDA, "verify_draft: launch failed: %s", cudaGetErrorString(e));
-    return p.defer ? launch_deferred<TH, true>(p, B, s, "verify_draft") : PLDP_OK;
+    return p.defer ? launch_deferred<TH>(p, B, s, "verify_draft") : PLDP_OK;
 }
 
 template <typename TH>
