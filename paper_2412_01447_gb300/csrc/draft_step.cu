@@ -2,13 +2,17 @@
 // with the longest-suffix n-gram rule), ranking by hidden states (Eq. 3) and/or
 // by attentions (Eq. 2), and draft extraction (Sec. 4.3) -- in one call; and
 // pldp_verify_greedy_draft / pldp_verify_sample_draft: greedy or sampling
-// verification (Sec. 4.4) followed by the next step's drafting.  Three kernels:
+// verification (Sec. 4.4) followed by the next step's drafting.  The kernels:
 //  * draft_step_kernel scans the contexts (below);
 //  * draft_index_kernel looks the occurrences up in the incremental token index
 //    (further down), one CTA per sequence;
 //  * verify_draft_kernel runs the finish of verification (on the greedy pass's
 //    row keys, or on the draws of sampling) and then the indexed drafting in the
-//    same CTA.
+//    same CTA;
+//  * score_deferred_kernel, behind each of these, scores the sequences with many
+//    candidates;
+//  * index_build_kernel, with index_clear_kernel before it for large batches, builds
+//    the index.
 //
 // The scanning kernel: one thread-block cluster per sequence, a chunk of the context
 // per CTA.  Each CTA
@@ -45,7 +49,9 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr size_t kSeqWs = 16 + 256 * 16;                       // workspace per sequence (see pldp_draft_workspace_size)
+// Workspace per sequence.  The scanning call needs a DeferSlot each and one more; the size
+// stays what callers know it to be.
+constexpr size_t kSeqWs = 16 + 256 * 16;
 constexpr int64_t kPositionsPerCta = 1024;                     // scanned by a CTA at least; the batch sets the rest
 constexpr int kScanLoads = 8;                                  // vectors of ids in flight per lane (scan kernel)
 constexpr int kListPerWarp = 128;                              // positions listed per warp (scan kernel)

@@ -34,7 +34,7 @@ constexpr int64_t kSegBytes = 32 * kSegLoads * 16;   // 2 KB
 constexpr int kPassBlocksPerSm = 8;         // register cap: 8 CTAs of 8 warps per SM
 constexpr int kPassWaves = 11;              // grid = up to 11 waves of resident CTAs
 // fp32 logits whose rows are not whole vectors stream in vectors from this many bytes on
-constexpr int64_t kLongRow = 192 << 10, kRaggedLong = 16 << 20, kRaggedShort = 32 << 20;
+constexpr int64_t kLongRow = 192 << 10, kRaggedLong = 20 << 20, kRaggedShort = 32 << 20;
 
 __global__ void extract_draft_kernel(const int32_t* __restrict__ ids, int64_t ids_stride,
                                      const int32_t* __restrict__ seq_len, int64_t T_cap,
@@ -391,7 +391,7 @@ pldp_status launch_verify_pass(const void* logits, pldp_dtype dtype, VerifyArgs&
     // loads, 4 bytes a lane, are better up to some size, the larger the more often a row ends
     // (a segment that holds two rows takes the slow way): 11 rows of 32001 4.0 against 4.9 us,
     // 176 of 32001 7.3 / 7.6, 1664 of 5001 9.2 / 9.7, 704 of 32001 18.0 / 16.9; 44 of 128255
-    // 9.3 / 7.4, 11 of them 5.0 / 5.2.
+    // 9.3 / 7.4, 11 of them 5.0 / 5.2; 88 of 50257, L2 flushed, 8.2 / 9.9.
     const bool wide = dtype == PLDP_BF16 || bytes >= (row_bytes >= kLongRow ? kRaggedLong : kRaggedShort);
     const bool ragged =
         !vec && wide && aligned16(logits) && long_rows && bytes / static_cast<int64_t>(es) < (int64_t(1) << 31);
