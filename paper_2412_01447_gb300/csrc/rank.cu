@@ -379,8 +379,10 @@ int pick_split(int B, int C_cap, const void* kernel, size_t smem) {
 // one candidate a sequence after an L2 flush.
 //
 // Two kernels, two CTAs an SM or three: the one whose grid fills the larger share of its
-// slots, and on long lists also where they are equal, since more of the smaller CTAs are
-// then under way per sequence.  Lists of 64, two and three CTAs an SM: batch 64 9.0 / 10.3
+// slots, and on long lists the second also where the shares are equal: more SMs then work on
+// the longest list (up to 1024 candidates of Zipf tokens, L2 flushed, batch 64 22.6 / 20.5,
+// 128 39.1 / 34.3 us; lists that are all as long as each other lose 2-8 %, batch 64 x 512
+// 61 / 66 us).  Lists of 64, two and three CTAs an SM: batch 64 9.0 / 10.3
 // us, 100 12.9 / 11.7, 120 13.3 / 15.3, 160 18.7 / 14.9, 200 19.5 / 15.7, 300 12.9 / 15.1;
 // lists of 1024: batch 100 35.3 / 25.7, 128 110 / 101, 200 38.5 / 28.0 us (with a warp's
 // candidates one at a time, three CTAs an SM: 30.1, 126, 31.9).
