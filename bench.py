@@ -945,7 +945,7 @@ def time_rank_stress(pk, loop, w, flush_l2, peak, iters=32, warm=3):
                              flush_l2, iters, warm)
             rec["rank_attention_1024_rows"] = _call_stats(tw["rank_attention_1024_rows"], n_list * Rw * 2.0, peak)
             del A_wide
-        if V == max(2, T // 128):      # at most 256 occurrences per sequence: the launch's own scoring path
+        if V == max(2, T // 128):      # about 128 candidates per sequence, which the deferred launch scores
             t = _time_calls([("draft_step", lambda: pk.pldp_draft_step(
                 ids, L, 1, 1, cand, cnt, ml, w.K, draft, dlen, dws, H=loop.H, best_h=best_h, A=loop.A,
                 best_a=best_a, draft_from="hidden"))], flush_l2, iters, warm)

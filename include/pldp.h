@@ -332,6 +332,9 @@ PLDP_API size_t pldp_draft_workspace_size(int B);
  * every sequence (all but the last token, which the next draft step looks up).
  * Token ids outside [0, V) mark that sequence's index unusable (TOKEN_RANGE);
  * seq_len outside [0, T_cap] too (SEQ_LEN).  Memory: about B * V * 64 bytes.
+ * The last 32 (B + 1) bytes (rounded up to 256) are scratch of the drafting calls;
+ * memory without them does too, with the same results and slower calls on contexts
+ * that repeat their tokens much.
  */
 PLDP_API size_t pldp_index_size(int B, int V);
 PLDP_API pldp_status pldp_index_build(const int32_t* ids, int64_t ids_stride, const int32_t* seq_len,
@@ -470,9 +473,9 @@ PLDP_API size_t pldp_verify_sample_workspace_size(int B, int K, int V, pldp_dtyp
  * token index) on the context it has just extended, with the same results and
  * status bits as those two calls in turn.  Sec. 4.4 at temperature T > 0 (the
  * paper's sampled runs use T = 1, Table 2), then Eq. 1-3 and Sec. 4.3; the paper
- * has no fused form.  Three launches: the per-piece stats pass over the logits,
- * one warp per row that draws, then one CTA per sequence that accepts, appends
- * and drafts the next step.
+ * has no fused form.  Four launches: the per-piece stats pass over the logits,
+ * one warp per row that draws, one CTA per sequence that accepts, appends and
+ * drafts the next step, then the scoring of sequences with many candidates.
  *
  *  logits, dtype, V   this step's logits [B, K+1, V], as pldp_verify_sample.
  *  temperature        T > 0, finite (else PLDP_ERR_INVALID_ARG).

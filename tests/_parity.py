@@ -54,7 +54,7 @@ def gpu_step(buf, ids, seq_len, logits, ngram=(1, 3), H=None, A=None, row_idx=No
              agg=pk.PLDP_AGG_MAX, draft_from="hidden", threshold=float("-inf"), append=True,
              stream=None, fused=False):
     """One step through the C ABI; ids/seq_len are updated in place when append.
-    fused: the drafting half runs as the single pldp_draft_step launch."""
+    fused: the drafting half runs as the single pldp_draft_step call."""
     if fused:
         ri = None if row_idx is None or A is None else torch.as_tensor(row_idx, dtype=torch.int32,
                                                                         device=A.device)

@@ -1,4 +1,4 @@
-"""GPU parity of the fused drafting launch (pldp_draft_step) against the oracle,
+"""GPU parity of the fused drafting call (pldp_draft_step) against the oracle,
 over shapes that give one CTA per sequence (both rankings in one CTA) and full
 clusters (rankings split across CTAs), and over the degenerate inputs."""
 import numpy as np
@@ -45,8 +45,7 @@ def _compare(g, ids0, L0, H, A, row_idx, agg, ngram, C, K, draft_from, thr=float
     assert np.array_equal(g["status"].view(np.uint32), st)
 
 
-# B >= half the SMs with contexts up to 40k tokens take the one-CTA-per-sequence kernel
-# (whole context in shared memory); smaller batches take the cluster kernel.
+# one CTA per sequence (short contexts) to a cluster of eight (long contexts, small batches)
 @pytest.mark.parametrize("T,V,B", [(300, 5, 12), (4096, 50, 8), (20000, 7, 3), (36096, 3000, 16),
                                    (3000, 5, 96), (5000, 40, 96), (36096, 3000, 96), (2048, 2, 80)])
 @pytest.mark.parametrize("mode", ["both", "hidden", "attention"])

@@ -1,7 +1,7 @@
 """Attention rows kept in pinned host memory: the rankings read them in place
 (only the selected rows' values at the candidate keys cross the link) and give
 exactly the results of the same rows on the device, for the separate Eq. 2
-ranking and for the one-launch drafting with the token index, in both memory
+ranking and for the one-call drafting with the token index, in both memory
 orders (each row's keys side by side, or the R values of each key)."""
 import numpy as np
 import pytest
