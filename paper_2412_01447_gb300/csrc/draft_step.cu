@@ -507,10 +507,15 @@ __global__ void __launch_bounds__(kThreads, 2) score_deferred_kernel(const Draft
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     DeferSlot* slots = p.defer;
     const int G = static_cast<int>(gridDim.x);
-    const int n0 = tid < B ? static_cast<int>(__ldcg(&slots[tid].pending)) : 0;   // the first tile's
+    // (no more than a list holds, whatever was in scratch that was not cleared)
+    auto pending = [&](int b) -> unsigned {
+        const unsigned n = __ldcg(&slots[b].pending), cap = static_cast<unsigned>(p.C_cap);
+        return n < cap ? n : cap;
+    };
+    const int n0 = tid < B ? static_cast<int>(pending(tid)) : 0;   // the first tile's
     unsigned sum = n0, seqs = n0 > 0;
     for (int b = tid + kThreads; b < B; b += kThreads) {
-        const unsigned n = __ldcg(&slots[b].pending);
+        const unsigned n = pending(b);
         sum += n;
         seqs += n > 0;
     }
@@ -544,7 +549,7 @@ __global__ void __launch_bounds__(kThreads, 2) score_deferred_kernel(const Draft
     int64_t unit0 = 0;                                            // units of the tiles before
     for (int b0 = 0; b0 < B; b0 += kThreads) {
         // the tile's units: an exclusive scan over its sequences
-        const int n = b0 == 0 ? n0 : b0 + tid < B ? static_cast<int>(__ldcg(&slots[b0 + tid].pending)) : 0;
+        const int n = b0 == 0 ? n0 : b0 + tid < B ? static_cast<int>(pending(b0 + tid)) : 0;
         const int units = (n + U - 1) / U;
         int incl = units;
 #pragma unroll
