@@ -33,8 +33,6 @@ constexpr int kSegLoads = 4;                // 16-byte loads per lane per segmen
 constexpr int64_t kSegBytes = 32 * kSegLoads * 16;   // 2 KB
 constexpr int kPassBlocksPerSm = 8;         // register cap: 8 CTAs of 8 warps per SM
 constexpr int kPassWaves = 11;              // grid = up to 11 waves of resident CTAs
-// fp32 logits whose rows are not whole vectors stream in vectors from this many bytes on
-constexpr int64_t kLongRow = 192 << 10, kRaggedLong = 20 << 20, kRaggedShort = 32 << 20;
 
 __global__ void extract_draft_kernel(const int32_t* __restrict__ ids, int64_t ids_stride,
                                      const int32_t* __restrict__ seq_len, int64_t T_cap,
@@ -259,8 +257,7 @@ __device__ __forceinline__ void segment_rows(const T* __restrict__ logits, int64
 // 1. the row argmax pass.  W = warps in the grid.  PATH 0: 16-byte loads, rows of
 // at least a segment (the streaming path); 3: the same for rows that are not a whole number of 16
 // bytes (a vocabulary with an added token); 1: 16-byte loads, short rows; 2: element loads
-// (unaligned logits; rows that are not a whole number of 16 bytes where they are short, or
-// fp32 and few).
+// (unaligned logits, and short rows that are not a whole number of 16 bytes).
 template <typename T, int PATH>
 __global__ void __launch_bounds__(kThreads, PATH == 0 || PATH == 3 ? kPassBlocksPerSm : 4)
 verify_argmax_kernel(const T* __restrict__ logits, int64_t N, int64_t V, int64_t W,
@@ -381,20 +378,16 @@ pldp_status launch_verify_pass(const void* logits, pldp_dtype dtype, VerifyArgs&
     const size_t es = dtype == PLDP_F32 ? 4 : 2;
     const bool vec = aligned16(logits) && (static_cast<size_t>(a.V) * es) % 16 == 0;
     const int64_t bytes = static_cast<int64_t>(a.B) * (a.K + 1) * a.V * static_cast<int64_t>(es);
-    const int64_t row_bytes = static_cast<int64_t>(a.V) * static_cast<int64_t>(es);
-    const bool long_rows = row_bytes >= kSegBytes;
+    const bool long_rows = static_cast<int64_t>(a.V) * static_cast<int64_t>(es) >= kSegBytes;
     const bool small = bytes / 16 < (int64_t(1) << 31);     // 32-bit vector indices
     // Ragged rows of at least a segment stream like the others where their element indices
     // fit 32 bits (one stride past the end among them).  By element loads, 2 bytes a lane,
     // batch 128 x 13 rows of 128255 bf16 took 150 us, and 64 x 11 rows of 32001 27.5 us; so
-    // they take 68 and 18.4 us (rows of 128256 and 32000: 66 and 16.3), L2 flushed.  fp32 element
-    // loads, 4 bytes a lane, are better up to some size, the larger the more often a row ends
-    // (a segment that holds two rows takes the slow way): 11 rows of 32001 4.0 against 4.9 us,
-    // 176 of 32001 7.3 / 7.6, 1664 of 5001 9.2 / 9.7, 704 of 32001 18.0 / 16.9; 44 of 128255
-    // 9.3 / 7.4, 11 of them 5.0 / 5.2; 88 of 50257, L2 flushed, 8.2 / 9.9.
-    const bool wide = dtype == PLDP_BF16 || bytes >= (row_bytes >= kLongRow ? kRaggedLong : kRaggedShort);
-    const bool ragged =
-        !vec && wide && aligned16(logits) && long_rows && bytes / static_cast<int64_t>(es) < (int64_t(1) << 31);
+    // they take 68 and 18.4 us (rows of 128256 and 32000: 66 and 16.3), L2 flushed.
+    // (fp32 element loads, 4 bytes a lane, take 0.5-1 us less on few rows that are in L2, 11 of
+    // 32001 4.0 against 4.9 us, but 2.2 us more on 900 rows of 4257 behind a step's rankings,
+    // 11.8 against 9.6.)
+    const bool ragged = !vec && aligned16(logits) && long_rows && bytes / static_cast<int64_t>(es) < (int64_t(1) << 31);
     const int path = vec ? (long_rows && small ? 0 : 1) : ragged ? 3 : 2;
     if (dtype == PLDP_BF16) {
         if (path == 0) return launch_pass_t<__nv_bfloat16, 0>(logits, a, scratch, s, what);

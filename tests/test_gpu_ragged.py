@@ -20,7 +20,6 @@ DEV = "cuda"
                                      (2049, torch.bfloat16), (32001, torch.bfloat16), (511, torch.float32),
                                      (513, torch.float32), (1026, torch.float32), (32003, torch.float32)]
                          + [(V + r, torch.bfloat16) for V in (1024, 2048) for r in range(2, 7)]
-                         # fp32: element loads up to 32 MB, or 20 MB of rows of 192 KB
                          + [(12001, torch.float32), (12002, torch.float32)])
 @pytest.mark.parametrize("B,K", [(1, 1), (5, 7), (64, 10)])
 def test_greedy(lib, V, dtype, B, K):
